@@ -279,7 +279,7 @@ vl_status pairwise_impl(Exec& x, const double* E, int64_t lde, int m, int n, dou
   CovOut o;
   void* scratch;
   float *rho32 = nullptr, *c32 = nullptr;
-  double* rho64 = nullptr;
+  double *rho64 = nullptr, *c64 = nullptr;
   T* xt;
   double *pparts, *gpart, *Hr_w, *D_w;
   vl_status s = with_workspace(x, [&](Arena& a) {
@@ -293,6 +293,7 @@ vl_status pairwise_impl(Exec& x, const double* E, int64_t lde, int m, int n, dou
       c32 = a.take<float>((size_t)m * m);
     } else {
       rho64 = a.take<double>((size_t)m * m);
+      c64 = a.take<double>((size_t)m * m);
     }
     xt = a.take<T>((size_t)pl.n_pad * pl.m_pad);
     pparts = a.take<double>(nparts);
@@ -308,13 +309,13 @@ vl_status pairwise_impl(Exec& x, const double* E, int64_t lde, int m, int n, dou
   cudaStream_t st = x.s;
   if (cov_and_stats<T>(cx, E, lde, m, n, o, scratch) != VL_OK)
     return fail(h, VL_ERR_CUDA, "vl_pairwise_measure: tensor map encoding unavailable");
-  launch_pair_consts(o.C, m, rho32, c32, rho64, x.st, st);
+  launch_pair_consts(o.C, m, rho32, c32, rho64, c64, x.st, st);
   launch_transpose_std<T>(E, lde, m, n, o.mu, o.isd, xt, pl.m_pad, pl.n_pad, st);
   if (h->prof_start) cudaEventRecord(h->prof_start, st);
   if constexpr (sizeof(T) == 4)
     launch_pairwise_f32(xt, pl, rho32, c32, reinterpret_cast<float*>(pparts), st);
   else
-    launch_pairwise_f64(xt, pl, rho64, pparts, st);
+    launch_pairwise_f64(xt, pl, rho64, c64, pparts, st);
   if (h->prof_stop) cudaEventRecord(h->prof_stop, st);
   launch_measure_finalize(pparts, pl, o.hx, Hx, Hr, D, f32, st);
   return check_launch(h, "vl_pairwise_measure");
@@ -559,7 +560,7 @@ vl_status batch_prep(Exec& x, const vl_instance& I, InstBufs& b) {
   CovOut o{b.C, b.mu, b.isd, b.hx};
   if (cov_and_stats<float>(cx, b.E, n_eff, m, n_eff, o, scratch) != VL_OK)
     return fail(x.h, VL_ERR_CUDA, "vl_fit_batched: tensor map encoding unavailable");
-  launch_pair_consts(b.C, m, b.rho32, b.c32, nullptr, x.st, x.s);
+  launch_pair_consts(b.C, m, b.rho32, b.c32, nullptr, nullptr, x.st, x.s);
   launch_transpose_std<float>(b.E, n_eff, m, n_eff, b.mu, b.isd, b.xt, b.pl.m_pad, b.pl.n_pad,
                               x.s);
   return VL_OK;

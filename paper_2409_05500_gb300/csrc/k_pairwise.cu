@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "fx64.cuh"
 #include "vl_internal.cuh"
 
 namespace vl {
@@ -38,7 +39,6 @@ namespace {
 constexpr int TB = 32;        // variables per tile side
 constexpr int TT = 128;       // samples per shared-memory stage
 constexpr int KRUN = 16;      // samples per product/Kahan run (product <= 2^16)
-constexpr int NTH = 256;      // FP64 kernel threads: 16 x 16, each a 2 x 2 pair micro-tile
 constexpr float KAPPA = 2.8853900817779268f;       // 2 log2(e)
 constexpr float GAUSS_K = -0.08664339756999316f;   // -1 / (8 log2 e)
 
@@ -299,68 +299,70 @@ __global__ void __launch_bounds__(TB / MTI * 16, MINB)
   }
 }
 
-// Plain FP64 comparison kernel: per sample log cosh u = |u| + log1p(e^{-2|u|})
-// - ln 2 and u e^{-u^2/2} with CUDA's double-precision exp/log1p, FP64 sums.
-// Partials: k = 0 sum log cosh u, k = 1 sum u e^{-u^2/2}.
-__global__ void __launch_bounds__(NTH)
-    pairwise_f64_kernel(const double* __restrict__ xt, int m, int m_pad, int T, int n_real,
-                        int tps, const double* __restrict__ rho64, double* __restrict__ part) {
-  int I, J;
-  tile_coords(blockIdx.x, T, I, J);
+// FP64 measure.  The residuals are formed in FP64 (one FMA and one product
+// each), the per-sample functions and their sums in 63-bit fixed point
+// (fx64.cuh), which is closer to exact than FP64 functions and sums are.
+// Bound by the integer pipe (~170 instructions a residual sample) with the
+// FP64 pipe (two operations, 40 SM clocks a warp) close behind it.  m = 120,
+// n = 9997: 1.50 ms; with CUDA's FP64 exp and log1p, which keep the FP64 pipe
+// busy 20 times as long, 33.1 ms.
+// One pair a < b per thread, consecutive threads consecutive b (coalesced
+// loads of the time-major samples, a broadcast of x_a, no padded tiles), the
+// samples split over blockIdx.y.  Partials: k = 0 sum log cosh u, k = 1 sum
+// u e^{-u^2/2}.
+constexpr int FX_TH = 128;
+
+__device__ __forceinline__ void pair_of(int q, int m, int& a, int& b) {
+  // row a of the strict upper triangle starts at a (2 m - a - 1) / 2
+  const float w = 2.f * m - 1.f;
+  a = (int)((w - sqrtf(fmaxf(w * w - 8.f * (float)q, 0.f))) * 0.5f);
+  a = max(0, min(a, m - 2));
+  while (a > 0 && (int)((int64_t)a * (2 * m - a - 1) / 2) > q) --a;
+  while ((int)((int64_t)(a + 1) * (2 * m - a - 2) / 2) <= q) ++a;
+  b = a + 1 + q - (int)((int64_t)a * (2 * m - a - 1) / 2);
+}
+
+__global__ void __launch_bounds__(FX_TH)
+    pairwise_f64_kernel(const double* __restrict__ xt, int m, int m_pad, int n_real, int tps,
+                        const double* __restrict__ rho64, const double* __restrict__ c64,
+                        double* __restrict__ part) {
+  __shared__ fx::u64 te[fx::EXP_N], tl[fx::LOG_N];
+  __shared__ fx::u32 tr[fx::LOG_N];
+  const fx::Tab T{te, tl, tr};
+  fx::fill_tables(te, tl, tr);
+  __syncthreads();
+  const int q = blockIdx.x * FX_TH + threadIdx.x;
+  if (q >= m * (m - 1) / 2) return;
+  int a, b;
+  pair_of(q, m, a, b);
   const int split = blockIdx.y;
-  const int t0 = split * tps;
-  const int t1 = min(n_real, t0 + tps);
-  const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
-  const int gi0 = I * TB + 2 * ti, gj0 = J * TB + 2 * tj;
-  double rho[4], sc[4];
-  bool valid[4];
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    const int a = gi0 + (p >> 1), b = gj0 + (p & 1);
-    valid[p] = (a < b) && (b < m);
-    rho[p] = valid[p] ? rho64[(int64_t)a * m + b] : 0.0;
-    sc[p] = 1.0 / sqrt(1.0 - rho[p] * rho[p]);
-  }
-  double sA[8], sB[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) sA[q] = sB[q] = 0.0;
+  const int t0 = split * tps, t1 = min(n_real, t0 + tps);
+  const double rho = rho64[(int64_t)a * m + b], c = c64[(int64_t)a * m + b];
+  fx::Moments ma, mb;  // residual of a on b, of b on a
+  const double* row = xt + (int64_t)t0 * m_pad;
+  double xa = t0 < t1 ? row[a] : 0.0, xb = t0 < t1 ? row[b] : 0.0;
   for (int t = t0; t < t1; ++t) {
-    const double* row = xt + (int64_t)t * m_pad;
-    const double xa[2] = {row[gi0], row[gi0 + 1]};
-    const double xb[2] = {row[gj0], row[gj0 + 1]};
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      if (!valid[p]) continue;
-      const double a = xa[p >> 1], b = xb[p & 1];
-#pragma unroll
-      for (int d = 0; d < 2; ++d) {
-        const double self = d ? b : a, other = d ? a : b;
-        const double u = sc[p] * (self - rho[p] * other);
-        const double au = fabs(u);
-        sA[2 * p + d] += au + log1p(exp(-2.0 * au)) - LN2;
-        sB[2 * p + d] += u * exp(-0.5 * u * u);
-      }
+    const double va = xa, vb = xb;
+    row += m_pad;
+    if (t + 1 < t1) {
+      xa = row[a];
+      xb = row[b];
     }
+    fx::moments_add(ma, c * (va - rho * vb), T);
+    fx::moments_add(mb, c * (vb - rho * va), T);
   }
   const int64_t mm = (int64_t)m * m;
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    if (!valid[p]) continue;
-    const int a = gi0 + (p >> 1), b = gj0 + (p & 1);
-#pragma unroll
-    for (int d = 0; d < 2; ++d) {
-      const int64_t off = d ? ((int64_t)b * m + a) : ((int64_t)a * m + b);
-      double* base = part + (int64_t)split * 2 * mm + off;
-      base[0] = sA[2 * p + d];
-      base[mm] = sB[2 * p + d];
-    }
-  }
+  double* base = part + (int64_t)split * 2 * mm;
+  const int64_t ab = (int64_t)a * m + b, ba = (int64_t)b * m + a;
+  fx::moments_sums(ma, max(0, t1 - t0), base[ab], base[mm + ab]);
+  fx::moments_sums(mb, max(0, t1 - t0), base[ba], base[mm + ba]);
 }
 
 // rho_ij = C_ij / sqrt(C_ii C_jj) from the centred cross-product matrix C.
 __global__ void pair_consts_kernel(const double* __restrict__ C, int m,
                                    float* __restrict__ rho32, float* __restrict__ c32,
-                                   double* __restrict__ rho64, int* st) {
+                                   double* __restrict__ rho64, double* __restrict__ c64,
+                                   int* st) {
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)m * m) return;
   const int a = (int)(idx / m), b = (int)(idx % m);
@@ -376,7 +378,10 @@ __global__ void pair_consts_kernel(const double* __restrict__ C, int m,
     rho32[idx] = (float)r;
     c32[idx] = (float)((double)KAPPA / sqrt(1.0 - r * r));
   }
-  if (rho64) rho64[idx] = r;
+  if (rho64) {
+    rho64[idx] = r;
+    c64[idx] = fx::KAPPA64 / sqrt(1.0 - r * r);
+  }
 }
 
 // double-float accumulate (hi, lo) += x (TwoSum)
@@ -481,7 +486,16 @@ PairPlan plan_pairwise_slots(int m, int n, int slots, int tts, bool fp64, int nu
       splits = sp;
     }
   }
-  if (fp64) splits = std::min(std::max(1, (4 * num_sms + pl.tiles - 1) / pl.tiles), n);
+  if (fp64) {
+    // CTAs of FX_TH pairs, six to eight resident per SM: about four waves of
+    // them so that the last one is short, splits of at least 16 samples, and
+    // no more partials than vl_reserve counts
+    const int pb = (int)(((int64_t)m * (m - 1) / 2 + FX_TH - 1) / FX_TH);
+    const int64_t cap = 32 + 2048 * (int64_t)num_sms / ((int64_t)m * m);
+    splits = (int)std::min<int64_t>({(24 * (int64_t)num_sms + pb - 1) / pb, cap,
+                                     std::max(1, n_run / 16)});
+    splits = std::max(1, splits);
+  }
   int tps = (n_run + splits - 1) / splits;
   tps = ((tps + KRUN - 1) / KRUN) * KRUN;
   pl.splits = (n_run + tps - 1) / tps;
@@ -511,11 +525,11 @@ PairPlan plan_pairwise(int m, int n, int num_sms, bool fp64) {
   return plan_pairwise_slots(m, n, F32_MINB * num_sms, F32_TTS, fp64, num_sms);
 }
 
-void launch_pair_consts(const double* C, int m, float* rho32, float* c32, double* rho64, int* st,
-                        cudaStream_t s) {
+void launch_pair_consts(const double* C, int m, float* rho32, float* c32, double* rho64,
+                        double* c64, int* st, cudaStream_t s) {
   int64_t tot = (int64_t)m * m;
   note_launch();
-  pair_consts_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(C, m, rho32, c32, rho64, st);
+  pair_consts_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(C, m, rho32, c32, rho64, c64, st);
 }
 
 template <int MTI, int TTS, int MINB>
@@ -571,11 +585,12 @@ void launch_pairwise_f32_list(const PairJob* jobs, const int4* items, int nitems
 }
 
 void launch_pairwise_f64(const double* xt, const PairPlan& pl, const double* rho64,
-                         double* part, cudaStream_t s) {
-  dim3 grid(pl.tiles, pl.splits);
+                         const double* c64, double* part, cudaStream_t s) {
+  const int64_t pairs = (int64_t)pl.m * (pl.m - 1) / 2;
+  dim3 grid((unsigned)((pairs + FX_TH - 1) / FX_TH), pl.splits);
   note_launch();
-  pairwise_f64_kernel<<<grid, NTH, 0, s>>>(xt, pl.m, pl.m_pad, pl.m_pad / TB, pl.n,
-                                           pl.t_per_split, rho64, part);
+  pairwise_f64_kernel<<<grid, FX_TH, 0, s>>>(xt, pl.m, pl.m_pad, pl.n, pl.t_per_split, rho64,
+                                             c64, part);
 }
 
 void launch_measure_finalize(const void* part, const PairPlan& pl, const double* hx_mom,

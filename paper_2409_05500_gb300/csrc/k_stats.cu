@@ -12,6 +12,7 @@
 //                   layout the pairwise kernel stages into shared memory.
 #include <cmath>
 
+#include "fx64.cuh"
 #include "vl_internal.cuh"
 
 namespace vl {
@@ -126,14 +127,6 @@ __global__ void var_resid_init_kernel(const double* __restrict__ X, int64_t ldx,
     E[(int64_t)i * lde + t] = X[(int64_t)i * ldx + p + t] - off;
 }
 
-// Sample moments of the standardized variable for H(x_i):
-// A = mean log cosh u, B = mean u exp(-u^2/2).
-__device__ __forceinline__ void moments_one(double u, double& a, double& b) {
-  // FP64 path of the moments
-  double au = fabs(u);
-  a += au + log1p(exp(-2.0 * au)) - LN2;
-  b += u * exp(-0.5 * u * u);
-}
 __device__ __forceinline__ void kahan_f(float& S, float& C, float x) {
   float y = x - C;
   float t = S + y;
@@ -177,9 +170,24 @@ __global__ void __launch_bounds__(kStatThreads) standardize_kernel(
     return;
   }
   const double isd = 1.0 / sqrt(var);
+  // sample moments of the standardized variable for H(x_i): A = mean log cosh
+  // u, B = mean u e^{-u^2/2}
   double a = 0.0, b = 0.0;
-  if (sizeof(T) == 8) {
-    for (int t = threadIdx.x; t < n; t += blockDim.x) moments_one((e[t] - mu) * isd, a, b);
+  if constexpr (sizeof(T) == 8) {
+    // fixed-point functions and exact sums (fx64.cuh)
+    __shared__ fx::u64 te[fx::EXP_N], tl[fx::LOG_N];
+    __shared__ fx::u32 tr[fx::LOG_N];
+    const fx::Tab tab{te, tl, tr};
+    fx::fill_tables(te, tl, tr);
+    __syncthreads();
+    // kappa times the value the pairwise kernel reads, so that H(x_i) and the
+    // residuals' entropies share the rounding of 1/std, which D's differences
+    // then cancel
+    fx::Moments M;
+    int cnt = 0;
+    for (int t = threadIdx.x; t < n; t += blockDim.x, ++cnt)
+      fx::moments_add(M, fx::KAPPA64 * ((e[t] - mu) * isd), tab);
+    fx::moments_sums(M, cnt, a, b);
   } else {
     // FP32 per-sample functions (CUDA's accurate expf / log1pf), Kahan sums
     // of log cosh u + ln 2 (= |u| + log1p(e^{-2|u|})) and u e^{-u^2/2}

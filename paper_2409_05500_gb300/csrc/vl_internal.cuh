@@ -224,12 +224,14 @@ PairPlan plan_pairwise(int m, int n, int num_sms, bool fp64);
 // FP32 plan with sample splits of about split_len samples (batched launches,
 // where many instances fill the GPU together)
 PairPlan plan_pairwise_split(int m, int n, int split_len);
-void launch_pair_consts(const double* C, int m, float* rho32, float* c32, double* rho64, int* st,
-                        cudaStream_t s);
+// rho and kappa / sqrt(1 - rho^2) (kappa = 2 log2 e) as FP32 (rho32, c32) or
+// FP64 (rho64, c64) m x m arrays; the other two are NULL
+void launch_pair_consts(const double* C, int m, float* rho32, float* c32, double* rho64,
+                        double* c64, int* st, cudaStream_t s);
 void launch_pairwise_f32(const float* xt, const PairPlan& pl, const float* rho32,
                          const float* c32, float* part, cudaStream_t s);
 void launch_pairwise_f64(const double* xt, const PairPlan& pl, const double* rho64,
-                         double* part, cudaStream_t s);
+                         const double* c64, double* part, cudaStream_t s);
 // One instance of the FP32 pairwise kernel in a multi-instance launch.
 struct PairJob {
   const float* xt;

@@ -22,6 +22,36 @@ def _f64(*shape):
     return torch.empty(shape, dtype=torch.float64, device="cuda")
 
 
+# one pair; pairs just below, at and above one CTA of pairs (17 -> 136, 16 ->
+# 120); fewer samples than a split's minimum; a spike beyond |u| = 22, where the
+# fixed-point functions hand over to FP64
+@pytest.mark.parametrize("m,n,spike", [(2, 2, 0), (2, 17, 0), (16, 15, 0), (17, 33, 0),
+                                       (5, 1500, 30.0), (3, 6000, 75.0)])
+def test_fp64_measure_sizes_and_outliers(vl, h, m, n, spike):
+    rng = np.random.default_rng(m * 1000 + n)
+    E = rng.laplace(size=(m, n))
+    E[1:] += 0.4 * E[:-1]
+    if spike:
+        E[0, n // 2] = spike * E[0].std() * 1.5
+        E[-1, 0] = -spike * E[-1].std()
+    if n == 2:
+        E[:, 1] = E[:, 0] + 1.0 + np.arange(m)  # |rho| = 1: degenerate
+    Hx, Hr, D = _f64(m), _f64(m, m), _f64(m, m)
+    vl.vl_pairwise_measure(h, torch.from_numpy(E).cuda(), "fp64", Hx, Hr, D)
+    if n == 2:
+        with pytest.raises(vl.VLError) as ei:
+            h.sync()
+        assert ei.value.code == 4  # VL_ERR_DEGENERATE
+        return
+    h.sync()
+    ref = oracle.pairwise_measure(oracle.standardize(E))
+    off = ~np.eye(m, dtype=bool)
+    for got, want in ((Hx, ref["Ex"]), (Hr, np.where(off, ref["Er"], 0.0)), (D, ref["D"])):
+        want = np.asarray(want)
+        err = np.abs(got.cpu().numpy() - want)
+        assert err.max() <= 1e-11 * max(1.0, np.abs(want).max())
+
+
 @pytest.mark.parametrize("prec", ["mixed", "fp64"])
 @pytest.mark.parametrize("m", [513, 575, 576, 577])
 def test_fit_b_beyond_one_cluster(vl, h, prec, m):
