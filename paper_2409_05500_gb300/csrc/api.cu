@@ -406,7 +406,7 @@ vl_status order_certified_impl(Exec& x, const double* D, const double* E, int64_
     cws = a.take<char>(certify_ws_bytes(m, n));
   });
   if (s != VL_OK || x.measure) return s;
-  launch_causal_order(D, m, ows, order, nullptr, x.st, x.s, nullptr, certify_spick(cws, m));
+  launch_causal_order(D, m, ows, order, nullptr, x.st, x.s, certify_spick(cws, m));
   launch_certify(D, E, lde, m, n, ows, cws, order, stats, x.h->num_sms, x.s);
   if (gap) launch_order_gaps(ows, m, order, gap, x.s);
   return check_launch(x.h, "vl_causal_order_certified");

@@ -111,7 +111,7 @@ __global__ void cert_init_kernel(const double* __restrict__ D, int m, int* ctrl,
 // the step after it.
 __global__ void cert_round_kernel(const int32_t* __restrict__ order, int m, int round, int* ctrl,
                                   int* __restrict__ pos, int* __restrict__ flag,
-                                  int* __restrict__ ccount, const double* __restrict__ spick,
+                                  int* __restrict__ ccount, const float2* __restrict__ spick,
                                   const unsigned long long* __restrict__ dmax_bits,
                                   float* __restrict__ thr) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -121,7 +121,7 @@ __global__ void cert_round_kernel(const int32_t* __restrict__ order, int m, int 
     ccount[t] = 0;
     // the picked score of step t raised by its band, rounded up to FP32
     const double dmax = __longlong_as_double((long long)*dmax_bits);
-    const double sc = spick[t];
+    const double sc = (double)spick[t].x + (double)spick[t].y;
     thr[t] = __double2float_ru(sc + cert_band(sc, m - t, dmax));
   }
   if (t == 0 && round > 0) {
@@ -147,20 +147,20 @@ __global__ void cert_round_kernel(const int32_t* __restrict__ order, int m, int 
 // loaded while the current eight are replayed.
 constexpr int FLAG_GROUP = 8;
 
-__device__ __forceinline__ void flag_load(const float* __restrict__ pth,
-                                          const float* __restrict__ ptl, const int* ord, int m,
+__device__ __forceinline__ void flag_load(const float2* __restrict__ pt, const int* ord, int m,
                                           int i, int pi, int t0, float* h, float* l) {
 #pragma unroll
   for (int u = 0; u < FLAG_GROUP; ++u) {
     const int c = t0 + u < pi ? ord[t0 + u] : i;
-    h[u] = pth[(int64_t)c * m + i];
-    l[u] = ptl[(int64_t)c * m + i];
+    const float2 p = pt[(int64_t)c * m + i];
+    h[u] = p.x;
+    l[u] = p.y;
   }
 }
 
 __global__ void __launch_bounds__(32)
-    cert_flag_kernel(const float* __restrict__ pth, const float* __restrict__ ptl,
-                     const float* __restrict__ sh0, const float* __restrict__ sl0,
+    cert_flag_kernel(const float2* __restrict__ pt, const float* __restrict__ sh0,
+                     const float* __restrict__ sl0,
                      const int32_t* __restrict__ order, const int* __restrict__ pos,
                      const float* __restrict__ thr, int m, int* ctrl,
                      const unsigned long long* __restrict__ dmax_bits, int* __restrict__ flag,
@@ -180,9 +180,9 @@ __global__ void __launch_bounds__(32)
   const float bc = (float)CERT_C * dmax, be = (float)CERT_ETA * dmax;
   df::F2 s{sh0[i], sl0[i]};
   float ph[FLAG_GROUP], pl[FLAG_GROUP], nh[FLAG_GROUP], nl[FLAG_GROUP];
-  if (pi > 0) flag_load(pth, ptl, ord_s, m, i, pi, 0, ph, pl);
+  if (pi > 0) flag_load(pt, ord_s, m, i, pi, 0, ph, pl);
   for (int t0 = 0; t0 < pi; t0 += FLAG_GROUP) {
-    if (t0 + FLAG_GROUP < pi) flag_load(pth, ptl, ord_s, m, i, pi, t0 + FLAG_GROUP, nh, nl);
+    if (t0 + FLAG_GROUP < pi) flag_load(pt, ord_s, m, i, pi, t0 + FLAG_GROUP, nh, nl);
     // the group's scores first (the only dependent chain), then its tests
     float sf[FLAG_GROUP];
 #pragma unroll
@@ -406,12 +406,11 @@ __global__ void __launch_bounds__(RTH)
 // subtractions the first search made over steps 0 .. k*-1, step k* takes the
 // corrected pick, and the remaining steps search as before.
 template <int PER>
-__global__ void __launch_bounds__(OTH)
-    cert_resume_kernel(const float* __restrict__ pth, const float* __restrict__ ptl,
-                       const float* __restrict__ sh0, const float* __restrict__ sl0, int m,
-                       int32_t* __restrict__ order, const int* __restrict__ pos,
-                       const int* __restrict__ pick, const int* ctrl,
-                       double* __restrict__ spick, int* __restrict__ stats) {
+__global__ void __launch_bounds__(STH)
+    cert_resume_kernel(const float2* __restrict__ pt, const float* __restrict__ sh0,
+                       const float* __restrict__ sl0, int m, int32_t* __restrict__ order,
+                       const int* __restrict__ pos, const int* __restrict__ pick,
+                       const int* ctrl, float2* __restrict__ spick, int* __restrict__ stats) {
   if (!ctrl[C_ACTIVE]) return;
   const int ks = ctrl[C_FIRST];
   if (ks >= m) return;
@@ -420,7 +419,7 @@ __global__ void __launch_bounds__(OTH)
   bool alive[PER];
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
-    const int i = threadIdx.x + q * blockDim.x;
+    const int i = threadIdx.x + q * STH;
     alive[q] = i < m && pos[i] >= ks;
     hi[q] = alive[q] ? sh0[i] : 0.f;
     lo[q] = alive[q] ? sl0[i] : 0.f;
@@ -429,17 +428,21 @@ __global__ void __launch_bounds__(OTH)
     const int c = order[l];
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-      const int i = threadIdx.x + q * blockDim.x;
-      if (alive[q]) df_sub(hi[q], lo[q], pth[(int64_t)c * m + i], ptl[(int64_t)c * m + i]);
+      const int i = threadIdx.x + q * STH;
+      if (alive[q]) {
+        const float2 p = pt[(int64_t)c * m + i];
+        df_sub(hi[q], lo[q], p.x, p.y);
+      }
     }
   }
   // every thread has read order[0 .. ks-1] before thread 0 overwrites order[ks ..]
   __syncthreads();
-  search_steps<PER>(hi, lo, alive, m, ks, pick[ks], order, spick, nullptr,
-                    [&](int c, int i, float& h, float& l) {
-                      h = pth[(int64_t)c * m + i];
-                      l = ptl[(int64_t)c * m + i];
-                    });
+  search_steps<PER, SW>(
+      hi, lo, alive, m, ks, pick[ks], order, spick,
+      [&](int c, int q) {
+        return pt[(int64_t)c * m + min((int)threadIdx.x + q * STH, m - 1)];
+      },
+      NoAhead());
 }
 
 // Steps after a pick changed in the last round were not verified again.
@@ -457,7 +460,8 @@ struct CertWs {
   unsigned long long* dmax;
   int* stats;
   int *pos, *flag, *ccount, *cand, *pick;
-  double *spick, *hx, *D64;
+  float2* spick;
+  double *hx, *D64;
   float* thr;
   unsigned *need, *done;
   int2* pairs;
@@ -484,7 +488,7 @@ CertWs cert_layout(void* base, int m, int n) {
   w.ccount = a.take<int>(m);
   w.cand = a.take<int>((size_t)m * CMAX);
   w.pick = a.take<int>(m);
-  w.spick = a.take<double>(m);
+  w.spick = a.take<float2>(m);
   w.thr = a.take<float>(m);
   w.hx = a.take<double>(m);
   w.D64 = a.take<double>(mm);
@@ -498,7 +502,7 @@ CertWs cert_layout(void* base, int m, int n) {
 
 size_t certify_ws_bytes(int m, int n) { return cert_layout(nullptr, m, n).bytes; }
 
-double* certify_spick(void* cert_ws, int m) { return cert_layout(cert_ws, m, 0).spick; }
+float2* certify_spick(void* cert_ws, int m) { return cert_layout(cert_ws, m, 0).spick; }
 
 void launch_certify(const double* D, const double* E, int64_t lde, int m, int n, void* order_ws,
                     void* cert_ws, int32_t* order, int32_t* stats_out, int num_sms,
@@ -512,14 +516,17 @@ void launch_certify(const double* D, const double* E, int64_t lde, int m, int n,
   note_launch();
   cert_init_kernel<<<std::min(1024, std::max(1, (int)(((size_t)m * m + 255) / 256))), 256, 0, s>>>(
       D, m, w.ctrl, w.dmax);
-  const int per = m <= OTH ? 1 : (m <= 2 * OTH ? 2 : 4);
-  const int nthr = std::min(OTH, ((m + per - 1) / per + 31) / 32 * 32);
+  const auto resume = m <= STH       ? cert_resume_kernel<1>
+                      : m <= 2 * STH ? cert_resume_kernel<2>
+                      : m <= 4 * STH ? cert_resume_kernel<4>
+                      : m <= 8 * STH ? cert_resume_kernel<8>
+                                     : cert_resume_kernel<16>;
   for (int r = 0; r < CERT_ROUNDS; ++r) {
     note_launch();
     cert_round_kernel<<<gb, 256, 0, s>>>(order, m, r, w.ctrl, w.pos, w.flag, w.ccount, w.spick,
                                          w.dmax, w.thr);
     note_launch();
-    cert_flag_kernel<<<(m + 31) / 32, 32, 8 * (size_t)m, s>>>(ow.pth, ow.ptl, ow.sh, ow.sl, order, w.pos,
+    cert_flag_kernel<<<(m + 31) / 32, 32, 8 * (size_t)m, s>>>(ow.pt, ow.sh, ow.sl, order, w.pos,
                                                    w.thr, m, w.ctrl, w.dmax, w.flag, w.ccount,
                                                    w.cand);
     note_launch();
@@ -534,15 +541,8 @@ void launch_certify(const double* D, const double* E, int64_t lde, int m, int n,
     cert_decide_kernel<<<m, RTH, 0, s>>>(order, w.pos, m, w.ctrl, w.flag, w.ccount, w.cand,
                                         w.D64, w.done, w.pick);
     note_launch();
-    if (per == 1)
-      cert_resume_kernel<1><<<1, nthr, 0, s>>>(ow.pth, ow.ptl, ow.sh, ow.sl, m, order, w.pos,
-                                               w.pick, w.ctrl, w.spick, w.stats);
-    else if (per == 2)
-      cert_resume_kernel<2><<<1, nthr, 0, s>>>(ow.pth, ow.ptl, ow.sh, ow.sl, m, order, w.pos,
-                                               w.pick, w.ctrl, w.spick, w.stats);
-    else
-      cert_resume_kernel<4><<<1, nthr, 0, s>>>(ow.pth, ow.ptl, ow.sh, ow.sl, m, order, w.pos,
-                                               w.pick, w.ctrl, w.spick, w.stats);
+    resume<<<1, STH, 0, s>>>(ow.pt, ow.sh, ow.sl, m, order, w.pos, w.pick, w.ctrl, w.spick,
+                             w.stats);
   }
   note_launch();
   cert_tail_kernel<<<1, 1, 0, s>>>(m, w.ctrl, w.stats);

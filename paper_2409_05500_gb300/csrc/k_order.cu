@@ -8,17 +8,14 @@
 // on this part, so the running sums S_i = M_i are kept as double-float pairs
 // (hi + lo, two FP32 numbers, ~48-bit significand) and updated with TwoSum
 // after each pick, S_i -= P_{i,c}.  The argmin compares an order-preserving
-// 64-bit integer key built from (hi, lo) and the index with two warp
-// reduction instructions (__reduce_min_sync) and no branch, so no
-// floating-point compare sits on the critical path; scores closer than about
-// 2^-35 relative are taken as tied and go by index.
+// 64-bit integer key built from (hi, lo) and the index, so no floating-point
+// compare sits on the critical path; scores closer than about 2^-35 relative
+// are taken as tied and go by index (order_search.cuh).
 // The initial sums are computed in FP64 by a parallel kernel; the per-step
 // relative gaps are computed after the search by another.  Subtracting the
 // removed column instead of re-summing over U gives the same sums as the
 // literal recomputation up to rounding (~1e-14 relative).
 #include <algorithm>
-#include <cfloat>
-#include <climits>
 #include <mutex>
 
 #include "order_search.cuh"
@@ -29,12 +26,11 @@ namespace vl {
 namespace {
 
 using namespace search;
-static_assert(VL_MAX_M <= 4 * OTH, "ordering holds at most four variables per thread");
+static_assert(VL_MAX_M <= 16 * STH, "ordering holds at most sixteen variables per thread");
 static_assert(VL_MAX_M <= 4096, "the search key holds the variable index in 12 bits");
 
-// Pt_hi/lo[c * m + i] = min(0, D[i * m + c])^2 as a double-float pair.
-__global__ void pt_kernel(const double* __restrict__ D, int m, float* __restrict__ pth,
-                          float* __restrict__ ptl, int* st) {
+// Pt[c * m + i] = min(0, D[i * m + c])^2 as a double-float pair.
+__global__ void pt_kernel(const double* __restrict__ D, int m, float2* __restrict__ pt, int* st) {
   __shared__ double tile[32][33];
   const int c0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -54,8 +50,7 @@ __global__ void pt_kernel(const double* __restrict__ D, int m, float* __restrict
     if (c < m && i < m) {
       double v = tile[tx][r];
       float hi = (float)v;
-      pth[(int64_t)c * m + i] = hi;
-      ptl[(int64_t)c * m + i] = (float)(v - (double)hi);
+      pt[(int64_t)c * m + i] = make_float2(hi, (float)(v - (double)hi));
     }
   }
 }
@@ -80,40 +75,117 @@ __global__ void rowsum_kernel(const double* __restrict__ D, int m, float* __rest
   }
 }
 
-// Search with P in global memory (L2): Pt_hi/lo[c * m + i] = P_{i,c}.
-template <int PER>
-__global__ void __launch_bounds__(OTH) order_kernel(const float* __restrict__ pth,
-                                                    const float* __restrict__ ptl,
-                                                    const float* __restrict__ sh0,
-                                                    const float* __restrict__ sl0, int m,
-                                                    int32_t* __restrict__ order,
-                                                    double* __restrict__ spick,
-                                                    long long* __restrict__ prof) {
-  float hi[PER], lo[PER];
-  bool alive[PER];
+// This thread's variables at the start of the search.
+template <int PER, int NW>
+__device__ __forceinline__ void load_scores(const float* __restrict__ sh0,
+                                            const float* __restrict__ sl0, int m,
+                                            float (&hi)[PER], float (&lo)[PER],
+                                            bool (&alive)[PER]) {
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
-    const int i = threadIdx.x + q * blockDim.x;
+    const int i = threadIdx.x + q * 32 * NW;
     alive[q] = i < m;
     hi[q] = alive[q] ? sh0[i] : 0.f;
     lo[q] = alive[q] ? sl0[i] : 0.f;
   }
-  search_steps<PER>(hi, lo, alive, m, 0, -1, order, spick, prof,
-                    [&](int c, int i, float& h, float& l) {
-    h = pth[(int64_t)c * m + i];
-    l = ptl[(int64_t)c * m + i];
-  });
+}
+
+// Where P_{i,c} comes from decides a step's latency (measured dependent loads:
+// L2 300 to 530 clocks, distributed shared memory 290, a CTA's own shared
+// memory 33, L1 38), and m decides what fits:
+//   m <= 160        P in the CTA's own shared memory (order_local_kernel),
+//   160 < m <= 448  in the shared memory of a cluster (order_cluster_kernel),
+//   beyond          in L2, with the columns of likely picks fetched into L1
+//                   ahead of time (order_kernel).
+// Measured, whole call without gaps, against a search with one variable per
+// thread, a branch around every dead variable, P in L2 below m = 64 and beyond
+// 448 (no fetching ahead) and in a cluster between: m = 32 27 -> 17 us, 64
+// 37 -> 22, 100 52 -> 29, 160 74 -> 41, 256 107 -> 78, 400 165 -> 133, 800
+// 561 -> 371, 1600 1444 -> 1108.
+
+// Search with P in global memory: Pt[c * m + i] = P_{i,c}.  The eventual pick
+// is usually some warp's minimum for a few steps before it wins (in 60 to 80 %
+// of the steps, on measured D), so each warp, when its minimum changes, brings
+// that variable's column into L1: one asynchronous four-byte copy per line, to
+// a word nobody reads (prefetch.global.L1 leaves L1 untouched on this part, and
+// a plain load's destination register made later steps wait for it).
+template <int PER>
+__global__ void __launch_bounds__(STH) order_kernel(const float2* __restrict__ pt,
+                                                    const float* __restrict__ sh0,
+                                                    const float* __restrict__ sl0, int m,
+                                                    int32_t* __restrict__ order,
+                                                    float2* __restrict__ spick) {
+  float hi[PER], lo[PER];
+  bool alive[PER];
+  load_scores<PER, SW>(sh0, sl0, m, hi, lo, alive);
+  __shared__ uint32_t sinks[STH];
+  const uint32_t sink = (uint32_t)__cvta_generic_to_shared(&sinks[threadIdx.x]);
+  int last = -1;
+  search_steps<PER, SW>(
+      hi, lo, alive, m, 0, -1, order, spick,
+      [&](int c, int q) {
+        return __ldg(pt + (int64_t)c * m + min((int)threadIdx.x + q * STH, m - 1));
+      },
+      [&](int j) {
+        if (j == last || j >= m) return;
+        last = j;
+        const char* col = reinterpret_cast<const char*>(pt + (int64_t)j * m);
+        for (int o = (threadIdx.x & 31) * 128; o < 8 * m; o += 32 * 128)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sink), "l"(col + o));
+      });
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+
+// Copy cnt columns' rows i0 .. i0 + R - 1 of P into sm[c R + il] (zeros beyond
+// m), eight loads in flight per thread.
+__device__ __forceinline__ void stage_rows(const float2* __restrict__ pt, int m, int i0, int R,
+                                           float2* sm) {
+  const int tot = R * m;
+  for (int b = threadIdx.x; b < tot; b += 8 * blockDim.x) {
+    float2 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int idx = b + u * blockDim.x;
+      const int c = idx / R, i = i0 + idx - c * R;
+      v[u] = idx < tot && i < m ? __ldg(pt + (int64_t)c * m + i) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int idx = b + u * blockDim.x;
+      if (idx < tot) sm[idx] = v[u];
+    }
+  }
+}
+
+constexpr int OL_MAX_M = 160;  // 8 m^2 bytes fit one CTA's shared memory
+constexpr int OC_TH = 512;     // threads that stage P (the first 32 NW of them search)
+
+// The search with all of P in this CTA's shared memory, one variable per thread.
+template <int NW>
+__global__ void __launch_bounds__(OC_TH) order_local_kernel(const float2* __restrict__ pt,
+                                                            const float* __restrict__ sh0,
+                                                            const float* __restrict__ sl0, int m,
+                                                            int32_t* __restrict__ order,
+                                                            float2* __restrict__ spick) {
+  extern __shared__ __align__(16) float2 oc_rows[];
+  stage_rows(pt, m, 0, m, oc_rows);
+  __syncthreads();
+  if (threadIdx.x >= 32 * NW) return;
+  float hi[1], lo[1];
+  bool alive[1];
+  load_scores<1, NW>(sh0, sl0, m, hi, lo, alive);
+  const int i = min((int)threadIdx.x, m - 1);
+  search_steps<1, NW>(
+      hi, lo, alive, m, 0, -1, order, spick, [&](int c, int) { return oc_rows[c * m + i]; },
+      NoAhead());
 }
 
 // The same search with P held in distributed shared memory: a cluster of
 // OC_CTAS CTAs, CTA t keeping the rows i in [t R, (t+1) R) of P for every
 // column c (R = ceil(m / OC_CTAS), layout [c][i - t R] as (hi, lo) pairs).  CTA 0
-// runs the search; the others only hold their rows until it is done.  A
-// step's load of P_{i,c} is then a distributed-shared-memory load (about 200
-// clocks) instead of an L2 load of Pt (about 750 clocks on this part, two
-// thirds of a step at m = 400).  The only synchronisation is a cluster barrier
-// after the rows are loaded and one at the end, so no CTA leaves while its
-// rows can still be read.
+// runs the search; the others only hold their rows until it is done.  The only
+// synchronisation is a cluster barrier after the rows are loaded and one at the
+// end, so no CTA leaves while its rows can still be read.
 constexpr int OC_CTAS = 8;
 constexpr int OC_MAX_M = 448;  // R m (hi, lo) pairs must fit one CTA's shared memory
 
@@ -122,57 +194,55 @@ inline size_t oc_smem(int m) {
   return (size_t)R * m * sizeof(float2);
 }
 
-__global__ void __launch_bounds__(OTH) order_cluster_kernel(const float* __restrict__ pth,
-                                                            const float* __restrict__ ptl,
-                                                            const float* __restrict__ sh0,
-                                                            const float* __restrict__ sl0, int m,
-                                                            int32_t* __restrict__ order,
-                                                            double* __restrict__ spick) {
+template <int NW>
+__global__ void __launch_bounds__(OC_TH) order_cluster_kernel(const float2* __restrict__ pt,
+                                                              const float* __restrict__ sh0,
+                                                              const float* __restrict__ sl0, int m,
+                                                              int32_t* __restrict__ order,
+                                                              float2* __restrict__ spick) {
   extern __shared__ __align__(16) float2 oc_rows[];
   unsigned rank;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   const int R = (m + OC_CTAS - 1) / OC_CTAS;
-  const int i0 = (int)rank * R;
-  for (int idx = threadIdx.x; idx < R * m; idx += blockDim.x) {
-    const int c = idx / R, il = idx - c * R, i = i0 + il;
-    oc_rows[idx] = i < m ? make_float2(pth[(int64_t)c * m + i], ptl[(int64_t)c * m + i])
-                         : make_float2(0.f, 0.f);
-  }
+  stage_rows(pt, m, (int)rank * R, R, oc_rows);
   __syncthreads();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  if (rank == 0) {
-    const int i = threadIdx.x;
+  if (rank == 0 && threadIdx.x < 32 * NW) {
     float hi[1], lo[1];
     bool alive[1];
-    alive[0] = i < m;
-    hi[0] = alive[0] ? sh0[i] : 0.f;
-    lo[0] = alive[0] ? sl0[i] : 0.f;
+    load_scores<1, NW>(sh0, sl0, m, hi, lo, alive);
     // this thread's row: owner CTA and local index, as a shared::cluster base
-    const int own = min(i / R, OC_CTAS - 1);
+    const int i = min((int)threadIdx.x, m - 1), own = i / R;
     uint32_t base = (uint32_t)__cvta_generic_to_shared(oc_rows) + 8u * (uint32_t)(i - own * R);
     asm volatile("mapa.shared::cluster.u32 %0, %0, %1;" : "+r"(base) : "r"(own));
     const uint32_t stride = 8u * (uint32_t)R;
-    search_steps<1>(hi, lo, alive, m, 0, -1, order, spick, nullptr,
-                    [&](int c, int, float& h, float& l) {
-      asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"
-                   : "=f"(h), "=f"(l)
-                   : "r"(base + stride * (uint32_t)c)
-                   : "memory");
-    });
+    search_steps<1, NW>(
+        hi, lo, alive, m, 0, -1, order, spick,
+        [&](int c, int) {
+          float2 v;
+          asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"
+                       : "=f"(v.x), "=f"(v.y)
+                       : "r"(base + stride * (uint32_t)c)
+                       : "memory");
+          return v;
+        },
+        NoAhead());
   }
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Launch the cluster search; false if m is out of its range or the cluster
-// cannot be launched (the caller then runs order_kernel).
-bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, double* spick,
+// Launch the cluster search; false if the cluster cannot be launched (the
+// caller then runs order_kernel).
+template <int NW>
+bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, float2* spick,
                           cudaStream_t s) {
-  if (m < 64 || m > OC_MAX_M) return false;
   static bool attr = false;
   if (!attr) {
-    if (cudaFuncSetAttribute(order_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(order_cluster_kernel<NW>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)oc_smem(OC_MAX_M)) != cudaSuccess) {
       cudaGetLastError();
       return false;
@@ -181,7 +251,7 @@ bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, double* spick
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(OC_CTAS, 1, 1);
-  cfg.blockDim = dim3((m + 31) / 32 * 32, 1, 1);
+  cfg.blockDim = dim3(OC_TH, 1, 1);
   cfg.dynamicSmemBytes = oc_smem(m);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -192,7 +262,7 @@ bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, double* spick
   cfg.attrs = at;
   cfg.numAttrs = 1;
   note_launch();
-  if (cudaLaunchKernelEx(&cfg, order_cluster_kernel, (const float*)w.pth, (const float*)w.ptl,
+  if (cudaLaunchKernelEx(&cfg, order_cluster_kernel<NW>, (const float2*)w.pt,
                          (const float*)w.sh, (const float*)w.sl, m, order, spick) !=
       cudaSuccess) {
     cudaGetLastError();
@@ -201,35 +271,93 @@ bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, double* spick
   return true;
 }
 
-// Gaps after the search, from the order: variable i replays its score
-// S_i = sum_{j in U} P_ij step by step in FP64; at the step that picks it, it
-// records its score as the minimum s1[k]; at earlier steps it offers its
-// score to the step's runner-up s2[k] (atomic minimum of an ordered key).
-// Steps are taken eight at a time so that their loads overlap.
-__global__ void gap_scores_kernel(const float* __restrict__ pth, const float* __restrict__ ptl,
-                                  const float* __restrict__ sh0, const float* __restrict__ sl0,
-                                  const int32_t* __restrict__ order, int m,
-                                  double* __restrict__ s1, unsigned long long* __restrict__ s2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
+template <int NW>
+void launch_order_local(const OrderWs& w, int m, int32_t* order, float2* spick, cudaStream_t s) {
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(order_local_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         OL_MAX_M * OL_MAX_M * (int)sizeof(float2));
+    attr = true;
+  }
+  note_launch();
+  order_local_kernel<NW><<<1, OC_TH, (size_t)m * m * sizeof(float2), s>>>(w.pt, w.sh, w.sl, m,
+                                                                         order, spick);
+}
+
+// Gaps after the search, from the order: variable i replays its score S_i =
+// sum_{j in U} P_ij step by step in FP64; at the step that picks it, it records
+// its score as the minimum s1[k]; at earlier steps it offers its score to the
+// step's runner-up s2[k] (atomic minimum of an ordered key).  The replay is a
+// serial chain of FP64 subtractions per variable (about 40 clocks each), so
+// everything else is kept off it: a CTA takes GAP_V variables and GAP_T steps at
+// a time, all threads load and convert the tile's P (FP64 conversions issue at
+// 1.6 per clock per SM: few variables per CTA spread them over the SMs), one
+// warp runs the chains, and one thread per step reduces the GAP_V scores to one
+// atomic.  The gaps of m = 800 add 62 us (260 us with one thread doing all of it
+// for each variable).
+constexpr int GAP_V = 8, GAP_T = 64, GAP_TH = 128;
+__global__ void __launch_bounds__(GAP_TH)
+    gap_scores_kernel(const float2* __restrict__ pt, const float* __restrict__ sh0,
+                      const float* __restrict__ sl0, const int32_t* __restrict__ order, int m,
+                      double* __restrict__ s1, unsigned long long* __restrict__ s2) {
+  constexpr int PER = GAP_V * GAP_T / GAP_TH;
+  __shared__ double ps[GAP_T][GAP_V];  // P_i,order[k], then the scores before step k
+  __shared__ int pos[GAP_V];           // the step of i's own pick, once reached
+  const int tid = threadIdx.x, v = tid % GAP_V, i0 = blockIdx.x * GAP_V;
+  const int i = min(i0 + v, m - 1);
+  if (tid < GAP_V) pos[tid] = i0 + tid < m ? m : -1;
   double s = (double)sh0[i] + (double)sl0[i];
-  for (int t0 = 0; t0 < m; t0 += 8) {
-    int cs[8];
-    double p[8];
+  float2 p[PER];  // the next tile's entries of steps t = tid / GAP_V + q GAP_TH / GAP_V
+  int c[PER];
+  auto load = [&](int t0) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) cs[u] = t0 + u < m ? order[t0 + u] : i;
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      p[u] = (double)pth[(int64_t)cs[u] * m + i] + (double)ptl[(int64_t)cs[u] * m + i];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if (cs[u] == i) {
-        if (t0 + u < m) s1[t0 + u] = s;
-        return;
-      }
-      atomicMin(&s2[t0 + u], dkey(s));
-      s -= p[u];
+    for (int q = 0; q < PER; ++q) {
+      const int k = t0 + tid / GAP_V + q * (GAP_TH / GAP_V);
+      c[q] = k < m ? order[k] : -1;
     }
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+      p[q] = c[q] >= 0 ? pt[(int64_t)c[q] * m + i] : make_float2(0.f, 0.f);
+  };
+  load(0);
+  __syncthreads();
+  for (int t0 = 0; t0 < m; t0 += GAP_T) {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int t = tid / GAP_V + q * (GAP_TH / GAP_V);
+      ps[t][v] = (double)p[q].x + (double)p[q].y;
+      if (c[q] == i0 + v) pos[v] = t0 + t;
+    }
+    __syncthreads();
+    if (t0 + GAP_T < m) load(t0 + GAP_T);
+    if (tid < GAP_V) {
+#pragma unroll 8
+      for (int t = 0; t < GAP_T; ++t) {
+        const double x = ps[t][v];
+        ps[t][v] = s;
+        s -= x;
+      }
+    }
+    __syncthreads();
+    const int k = t0 + tid;
+    bool more = false;
+    if (tid < GAP_T && k < m) {
+      unsigned long long best = ~0ull;
+#pragma unroll
+      for (int u = 0; u < GAP_V; ++u) {
+        const double x = ps[tid][u];
+        if (k == pos[u]) s1[k] = x;
+        if (k < pos[u]) {
+          const unsigned long long key = dkey(x);
+          best = key < best ? key : best;
+        }
+      }
+      if (best != ~0ull) {
+        atomicMin(&s2[k], best);
+        more = true;  // a later step may still see one of these variables
+      }
+    }
+    if (!__syncthreads_or(more)) break;
   }
 }
 
@@ -251,21 +379,21 @@ __global__ void gap_kernel(const double* __restrict__ s1, const unsigned long lo
 OrderWs order_ws_layout(void* ws, int m) {
   OrderWs w;
   char* p = static_cast<char*>(ws);
-  w.pth = reinterpret_cast<float*>(p);
-  w.ptl = w.pth + (size_t)m * m;
-  w.sh = w.ptl + (size_t)m * m;
+  w.pt = reinterpret_cast<float2*>(p);
+  w.sh = reinterpret_cast<float*>(w.pt + (size_t)m * m);
   w.sl = w.sh + m;
   w.s1 = reinterpret_cast<double*>(((uintptr_t)(w.sl + m) + 15) & ~(uintptr_t)15);
   w.s2 = reinterpret_cast<unsigned long long*>(w.s1 + m);
   return w;
 }
 
-void launch_order_gaps(void* ws, int m, const int32_t* order, double* gap, cudaStream_t s) {
+void launch_order_gaps(void* ws, int m, const int32_t* order, double* gap,
+                       cudaStream_t s) {
   const OrderWs w = order_ws_layout(ws, m);
   cudaMemsetAsync(w.s2, 0xff, (size_t)m * sizeof(unsigned long long), s);
   note_launch();
-  gap_scores_kernel<<<(m + 127) / 128, 128, 0, s>>>(w.pth, w.ptl, w.sh, w.sl, order, m, w.s1,
-                                                      w.s2);
+  gap_scores_kernel<<<(m + GAP_V - 1) / GAP_V, GAP_TH, 0, s>>>(w.pt, w.sh, w.sl, order, m,
+                                                                   w.s1, w.s2);
   note_launch();
   gap_kernel<<<(m + 255) / 256, 256, 0, s>>>(w.s1, w.s2, m, gap);
 }
@@ -276,28 +404,35 @@ size_t order_ws_bytes(int m) {
 }
 
 void launch_causal_order(const double* D, int m, void* ws, int32_t* order, double* gap, int* st,
-                         cudaStream_t s, long long* prof, double* spick) {
+                         cudaStream_t s, float2* spick) {
   const OrderWs w = order_ws_layout(ws, m);
   dim3 grid((m + 31) / 32, (m + 31) / 32), block(32, 8);
   note_launch();
-  pt_kernel<<<grid, block, 0, s>>>(D, m, w.pth, w.ptl, st);
+  pt_kernel<<<grid, block, 0, s>>>(D, m, w.pt, st);
   note_launch();
   rowsum_kernel<<<(m + 7) / 8, 256, 0, s>>>(D, m, w.sh, w.sl);
-  // P in distributed shared memory (64 <= m <= 448), unless profiling
-  if (!prof && launch_order_cluster(w, m, order, spick, s)) {
-    if (gap) launch_order_gaps(ws, m, order, gap, s);
-    return;
+  const bool cluster = m > OL_MAX_M && m <= OC_MAX_M &&
+                       (m <= 256 ? launch_order_cluster<8>(w, m, order, spick, s)
+                                 : launch_order_cluster<16>(w, m, order, spick, s));
+  if (m <= 32) {
+    launch_order_local<1>(w, m, order, spick, s);
+  } else if (m <= 64) {
+    launch_order_local<2>(w, m, order, spick, s);
+  } else if (m <= 128) {
+    launch_order_local<4>(w, m, order, spick, s);
+  } else if (m <= OL_MAX_M) {
+    launch_order_local<8>(w, m, order, spick, s);
+  } else if (!cluster) {
+    note_launch();
+    if (m <= 2 * STH)
+      order_kernel<2><<<1, STH, 0, s>>>(w.pt, w.sh, w.sl, m, order, spick);
+    else if (m <= 4 * STH)
+      order_kernel<4><<<1, STH, 0, s>>>(w.pt, w.sh, w.sl, m, order, spick);
+    else if (m <= 8 * STH)
+      order_kernel<8><<<1, STH, 0, s>>>(w.pt, w.sh, w.sl, m, order, spick);
+    else
+      order_kernel<16><<<1, STH, 0, s>>>(w.pt, w.sh, w.sl, m, order, spick);
   }
-  // variables per thread: PER = 1 up to 1024 variables, then 2 and 4
-  const int per = m <= OTH ? 1 : (m <= 2 * OTH ? 2 : 4);
-  const int nthr = std::min(OTH, ((m + per - 1) / per + 31) / 32 * 32);
-  note_launch();
-  if (per == 1)
-    order_kernel<1><<<1, nthr, 0, s>>>(w.pth, w.ptl, w.sh, w.sl, m, order, spick, prof);
-  else if (per == 2)
-    order_kernel<2><<<1, nthr, 0, s>>>(w.pth, w.ptl, w.sh, w.sl, m, order, spick, prof);
-  else
-    order_kernel<4><<<1, nthr, 0, s>>>(w.pth, w.ptl, w.sh, w.sl, m, order, spick, prof);
   if (gap) launch_order_gaps(ws, m, order, gap, s);
 }
 

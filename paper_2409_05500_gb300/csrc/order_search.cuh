@@ -6,7 +6,7 @@
 // pairs (hi + lo, two FP32 numbers, ~48-bit significand) updated with TwoSum,
 // because FP64 issues at 1/64 of the FP32 rate on this part.  The argmin
 // compares an order-preserving 64-bit integer key built from (hi, lo) and the
-// index with two warp reduction instructions and no branch.
+// index.
 #pragma once
 
 #include "vl_internal.cuh"
@@ -14,7 +14,9 @@
 namespace vl {
 namespace search {
 
-constexpr int OTH = 1024;  // threads of the one-CTA search
+constexpr int SW = 8;           // warps of a search with several variables per thread
+constexpr int STH = 32 * SW;    // and its threads
+constexpr int SW_MAX = 16;      // most warps that search
 
 // order-preserving map float -> uint32 (valid for every non-NaN value)
 __device__ __forceinline__ uint32_t fkey(float f) {
@@ -37,26 +39,16 @@ __device__ __forceinline__ void df_sub(float& hi, float& lo, float ph, float pl)
   hi = h2;
 }
 
-// clock64 read ordered after `dep` is available
-__device__ __forceinline__ long long clock_after(float dep) {
-  long long t;
-  asm volatile("mov.u64 %0, %%clock64;" : "=l"(t) : "f"(dep));
-  return t;
-}
-
 // Search key of a live variable: (fkey(hi), fkey(lo) with its low 12 bits
 // replaced by the index).  Compared as a 64-bit integer it orders by the
 // double-float score and then by index; dropping 12 bits of lo merges
 // scores closer than about 2^-35 relative into index order, far below any
 // gap the method distinguishes.  A dead variable is (~0, ~0).
-__device__ __forceinline__ uint2 skey(float hi, float lo, int i) {
-  return make_uint2(fkey(hi), (fkey(lo) & 0xfffff000u) | (uint32_t)i);
+// The score a key encodes (lo without its 12 index bits), as a pair.
+__device__ __forceinline__ float2 skey_pair(uint2 k) {
+  return make_float2(fkey_inv(k.x), fkey_inv(k.y & 0xfffff000u));
 }
-// The score a key encodes (lo without its 12 index bits).
-__device__ __forceinline__ double skey_score(uint2 k) {
-  return (double)fkey_inv(k.x) + (double)fkey_inv(k.y & 0xfffff000u);
-}
-// warp-wide minimum key, in every lane (two REDUX, no branches)
+// warp-wide minimum key, in every lane
 __device__ __forceinline__ uint2 warp_kmin(uint2 k) {
   const uint32_t full = 0xffffffffu;
   const uint32_t h = __reduce_min_sync(full, k.x);
@@ -74,69 +66,76 @@ __device__ __forceinline__ double dkey_inv(unsigned long long k) {
   return __longlong_as_double((long long)b);
 }
 
-// Steps kbeg .. m-1 of the search, one CTA of up to 1024 threads, each owning
-// PER variables (i = tid + q*nthr).  A step: every warp reduces its keys
-// (warp_kmin) and lane 0 writes the warp minimum to a shared slot of the
-// step's parity; one barrier; every warp then reduces the warp minima itself,
-// so all threads learn the pick c without a second barrier (slots alternate by
-// parity: a warp can run at most one step ahead of the slowest); S_i -=
-// P_{i,c}.  forced >= 0 makes step kbeg pick that variable without a search
+struct NoAhead {
+  __device__ __forceinline__ void operator()(int) const {}
+};
+
+// Steps kbeg .. m-1 of the search by the first NW warps of a CTA (NW = 1, 2, 4,
+// 8 or 16; a named barrier, so the CTA may hold more), each thread owning PER
+// variables (i = tid + q 32 NW).  A step is one latency chain: keys (the
+// smallest high word over the thread and the warp first, then the low words
+// that go with it), the warp's minimum to a shared slot of the step's parity,
+// one barrier, the minimum over the NW slots (in every warp), the fetch of P's
+// column, S_i -= P_{i,c}.  No branch depends on a variable: dead ones compute
+// along, so that every warp takes the same straight path.  No second barrier:
+// slots alternate by parity and a warp can run at most one step ahead of the
+// slowest.  forced >= 0 makes step kbeg pick that variable without a search
 // (its score is then not recorded).  spick (optional): the winning score of
-// every searched step.  fetch(c, i, h, l) loads P_{i,c} as the double-float
-// pair (h, l).  prof (optional): clock64 stamps of thread 0, five per step:
-// start, warp minimum written, after the barrier, pick known, update done.
-template <int PER, class Fetch>
+// every searched step, as a pair.  fetch(c, q) loads P_{i,c} as a pair for the
+// thread's variable q (any valid address for i >= m); ahead(j), called by every
+// warp while the fetch is in flight, names the warp's own candidate, a likely
+// later pick.
+template <int PER, int NW, class Fetch, class Ahead>
 __device__ __forceinline__ void search_steps(float (&hi)[PER], float (&lo)[PER],
                                              bool (&alive)[PER], int m, int kbeg, int forced,
                                              int32_t* __restrict__ order,
-                                             double* __restrict__ spick,
-                                             long long* __restrict__ prof, Fetch fetch) {
-  __shared__ uint2 wb[2][32];
-  const int nthr = blockDim.x, nw = (nthr + 31) >> 5;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint2 dead = make_uint2(0xffffffffu, 0xffffffffu);
+                                             float2* __restrict__ spick, Fetch fetch,
+                                             Ahead ahead) {
+  __shared__ uint2 wb[2][SW_MAX];
+  constexpr int nthr = 32 * NW;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // a live variable's high key is below ~0 (only a NaN's can reach it)
+  uint32_t dead[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) dead[q] = alive[q] ? 0u : 0xffffffffu;
   for (int k = kbeg; k < m; ++k) {
-    const int ph = k & 1;
-    int c;
-    if (k == kbeg && forced >= 0) {
-      c = forced;
-    } else {
-      if (prof && threadIdx.x == 0) prof[5 * k] = clock64();
-      uint2 b = dead;
+    int c = forced, own = -1;
+    if (k != kbeg || forced < 0) {
+      uint32_t hk[PER], bh = 0xffffffffu, bl = 0xffffffffu;
 #pragma unroll
       for (int q = 0; q < PER; ++q) {
-        const uint2 cq = alive[q] ? skey(hi[q], lo[q], (int)threadIdx.x + q * nthr) : dead;
-        if (cq.x < b.x || (cq.x == b.x && cq.y < b.y)) b = cq;
+        hk[q] = fkey(hi[q]) | dead[q];
+        bh = min(bh, hk[q]);
       }
-      const uint2 w = warp_kmin(b);
-      if (lane == 0) wb[ph][wid] = w;
-      if (prof && threadIdx.x == 0) prof[5 * k + 1] = clock64();
-      __syncthreads();
-      if (prof && threadIdx.x == 0) prof[5 * k + 2] = clock64();
-      // block level, redundantly in every warp
-      const uint2 a = lane < nw ? wb[ph][lane] : dead;
-      const uint2 g = warp_kmin(a);
+      bh = __reduce_min_sync(0xffffffffu, bh);
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        const uint32_t lk =
+            ((fkey(lo[q]) & 0xfffff000u) | (uint32_t)(threadIdx.x + q * nthr)) | dead[q];
+        bl = min(bl, hk[q] == bh ? lk : 0xffffffffu);
+      }
+      bl = __reduce_min_sync(0xffffffffu, bl);
+      uint2 g = make_uint2(bh, bl);
+      own = (int)(bl & 0xfffu);
+      if constexpr (NW > 1) {
+        const int ph = k & 1;
+        if (lane == 0) wb[ph][wid] = g;
+        asm volatile("bar.sync 1, %0;" ::"n"(nthr) : "memory");
+        g = warp_kmin(wb[ph][lane & (NW - 1)]);
+      }
       c = (int)(g.y & 0xfffu);
-      if (prof && threadIdx.x == 0) prof[5 * k + 3] = clock64();
-      if (spick && threadIdx.x == 0) spick[k] = skey_score(g);
+      if (spick && threadIdx.x == 0) spick[k] = skey_pair(g);
     }
+    float2 p[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) p[q] = fetch(c, q);
     if (threadIdx.x == 0) order[k] = c;
-    float ch[PER], cl[PER];
+    ahead(own);
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
-      ch[q] = cl[q] = 0.f;
-      if (alive[q]) fetch(c, (int)threadIdx.x + q * nthr, ch[q], cl[q]);
+      df_sub(hi[q], lo[q], p[q].x, p[q].y);
+      if ((int)threadIdx.x + q * nthr == c) dead[q] = 0xffffffffu;
     }
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      const int i = threadIdx.x + q * nthr;
-      if (!alive[q]) continue;
-      if (i == c)
-        alive[q] = false;
-      else
-        df_sub(hi[q], lo[q], ch[q], cl[q]);
-    }
-    if (prof && threadIdx.x == 0) prof[5 * k + 4] = clock_after(hi[0]);
   }
 }
 

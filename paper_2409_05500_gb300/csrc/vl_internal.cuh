@@ -248,10 +248,11 @@ void launch_pairwise_f32_list(const PairJob* jobs, const int4* items, int nitems
 void launch_measure_finalize(const void* part, const PairPlan& pl, const double* hx_mom,
                              double* Hx, double* Hr, double* D, bool fp32_parts, cudaStream_t s);
 
-// Ordering (k_order.cu).  Its workspace: P^T as double-float (pth, ptl),
+// Ordering (k_order.cu).  Its workspace: P^T as double-float pairs (pt),
 // the initial row sums (sh, sl) and the gap scratch (s1, s2).
 struct OrderWs {
-  float *pth, *ptl, *sh, *sl;
+  float2* pt;
+  float *sh, *sl;
   double* s1;
   unsigned long long* s2;
 };
@@ -259,10 +260,10 @@ OrderWs order_ws_layout(void* ws, int m);
 size_t order_ws_bytes(int m);
 // per-step relative gaps of an order over the workspace's P (after a search)
 void launch_order_gaps(void* ws, int m, const int32_t* order, double* gap, cudaStream_t s);
-// spick (optional): the winning score of every step, for the certification
-// of near ties (k_certify.cu).
+// spick (optional): the winning score of every step as a double-float pair,
+// for the certification of near ties (k_certify.cu).
 void launch_causal_order(const double* D, int m, void* ws, int32_t* order, double* gap, int* st,
-                         cudaStream_t s, long long* prof = nullptr, double* spick = nullptr);
+                         cudaStream_t s, float2* spick = nullptr);
 
 // Tensor-core exact-slice Gram products (k_tcgram.cu).  Operands are three
 // bf16 slice planes S[z][r][k] (k < Kpad = tg_kpad(K), a multiple of 64; row
@@ -294,7 +295,7 @@ bool launch_tc_var_resid(const Ctx& cx, const float* Xc, int64_t ldc, const doub
 // stats_out (device, 4 ints, may be NULL): flagged steps, pairs re-evaluated,
 // picks changed, steps left unverified.
 size_t certify_ws_bytes(int m, int n);
-double* certify_spick(void* cert_ws, int m);
+float2* certify_spick(void* cert_ws, int m);
 void launch_certify(const double* D, const double* E, int64_t lde, int m, int n, void* order_ws,
                     void* cert_ws, int32_t* order, int32_t* stats_out, int num_sms,
                     cudaStream_t s);

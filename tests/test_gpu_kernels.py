@@ -68,3 +68,50 @@ def test_fit_b_beyond_one_cluster(vl, h, prec, m):
     h.sync()
     ref = oracle.fp64.b0_ldl(E, list(perm))
     assert np.abs(B0.cpu().numpy() - ref).max() <= (1e-4 if prec == "mixed" else 1e-10)
+
+
+def _order_fp64(D):
+    """Algorithm 1 with running FP64 sums: the order, each step's relative gap, and
+    how far that gap may be off: the sums start from pairs of 48 bits and take m
+    subtractions, so each score carries up to (m + 16) 2^-49 of its initial sum."""
+    m = D.shape[0]
+    P = np.minimum(D, 0.0) ** 2
+    np.fill_diagonal(P, 0.0)
+    S0 = P.sum(1)
+    S, alive = S0.copy(), np.ones(m, dtype=bool)
+    order, gap, slack = [], [], []
+    for _ in range(m):
+        left = np.flatnonzero(alive)
+        by = left[np.argsort(S[left], kind="stable")[:2]]
+        order.append(int(by[0]))
+        gap.append(np.inf)
+        slack.append(0.0)
+        if len(by) == 2:
+            a, b = P[np.ix_(by, left)].sum(1)
+            gap[-1] = (b - a) / max(a, b, 1e-300)
+            slack[-1] = 4 * (m + 16) * 2.0 ** -49 * S0[by].max() / max(a, b, 1e-300)
+        alive[by[0]] = False
+        S = S - P[:, by[0]]
+    return order, np.array(gap), np.array(slack)
+
+
+# the last size of each search (warps, variables per thread, where P is kept)
+# and the first of the next
+@pytest.mark.parametrize("m", [1, 31, 32, 33, 64, 65, 128, 129, 160, 161, 256, 257, 448, 449, 512,
+                               513, 1024, 1025, 2048, 2049])
+def test_order_at_the_edges_of_its_searches(vl, h, m):
+    rng = np.random.default_rng(m)
+    A = rng.normal(size=(m, m)) + 3.0 * rng.normal(size=m)[:, None]
+    D = A - A.T
+    if m > 40:  # not antisymmetric everywhere: both directions penalised
+        D[3, 7] = D[7, 3] = -2.0
+    order = torch.empty(m, dtype=torch.int32, device="cuda")
+    gap = _f64(m)
+    vl.vl_causal_order(h, torch.from_numpy(D).cuda(), order, gap)
+    h.sync()
+    want, want_gap, slack = _order_fp64(D)
+    assert order.cpu().tolist() == want
+    got = gap.cpu().numpy()
+    assert np.array_equal(np.isinf(got), np.isinf(want_gap))
+    fin = np.isfinite(want_gap)
+    assert np.all(np.abs(got[fin] - want_gap[fin]) <= 1e-9 + slack[fin])
