@@ -909,8 +909,13 @@ void chol_blocked(const Ctx& cx, T* A, int64_t lda, int n, T* dinv, double* diag
   const int NB = CHOL_NB;
   cudaStream_t s = cx.s;
   const double rel_tol = pivot_floor > 0 ? pivot_floor : (sizeof(T) == 4 ? 1e-6 : 1e-12);
+  note_launch();
+  save_diag_kernel<T><<<(n + 255) / 256, 256, 0, s>>>(A, lda, n, diag0);
   if constexpr (sizeof(T) == 4) {
     if (n <= SINGLE_MAX) {
+      if (launch_chol_cluster(A, lda, n, dinv, diag0, (float)rel_tol,
+                              reinterpret_cast<float*>(cx.part), 2 * cx.part_cap, cx.st, s))
+        return;
       const size_t smem1 = chol_single_smem(SINGLE_MAX);
       static bool attr1 = false;
       if (!attr1) {
@@ -918,9 +923,6 @@ void chol_blocked(const Ctx& cx, T* A, int64_t lda, int n, T* dinv, double* diag
                              (int)smem1);
         attr1 = true;
       }
-      note_launch();
-      save_diag_kernel<T><<<(n + 255) / 256, 256, 0, s>>>(A, lda, n, diag0);
-      if (launch_chol_cluster(A, lda, n, dinv, diag0, (float)rel_tol, cx.st, s)) return;
       note_launch();
       chol_single_kernel<<<1, STH, chol_single_smem(n), s>>>(A, lda, n, dinv, diag0,
                                                             (float)rel_tol, cx.st);
@@ -934,8 +936,6 @@ void chol_blocked(const Ctx& cx, T* A, int64_t lda, int n, T* dinv, double* diag
                          (int)smem);
     attr_set = true;
   }
-  note_launch();
-  save_diag_kernel<T><<<(n + 255) / 256, 256, 0, s>>>(A, lda, n, diag0);
   for (int k0 = 0; k0 < n; k0 += NB) {
     const int nb = std::min(NB, n - k0);
     T* dblk = dinv + (int64_t)(k0 / NB) * NB * NB;

@@ -196,13 +196,15 @@ size_t gemm_part_need(int M, int N, int K);
 template <class T>
 bool launch_trsm_ring(const T* L, int64_t lda, const T* dinv, int n, T* R, int64_t ldr, int nrhs,
                       bool backward, cudaStream_t s);
-// Cholesky of an FP32 matrix with n <= 512 on one thread-block cluster; false
-// if not launched (n out of range or no cluster resources).
+// Cholesky of an FP32 matrix with n <= 512 on one thread-block cluster, with a
+// scratch (scratch_cap floats, 16-byte aligned) for the tiles its CTAs exchange;
+// false if not launched (n out of range, scratch too small or no cluster
+// resources).
 bool launch_chol_cluster(float* A, int64_t lda, int n, float* dinv, const double* diag0,
-                         float rel_tol, int* st, cudaStream_t s,
-                         unsigned long long* prof = nullptr);
-template <class T>
+                         float rel_tol, float* scratch, size_t scratch_cap, int* st,
+                         cudaStream_t s);
 // pivot_floor > 0 replaces the default relative pivot floor.
+template <class T>
 void chol_blocked(const Ctx& c, T* A, int64_t lda, int n, T* dinv, double* diag0,
                   double pivot_floor = -1.0);
 // Solve L Y = R (forward) then optionally L^T X = Y (backward) for nrhs

@@ -52,10 +52,13 @@ def test_fp64_measure_sizes_and_outliers(vl, h, m, n, spike):
         assert err.max() <= 1e-11 * max(1.0, np.abs(want).max())
 
 
-@pytest.mark.parametrize("prec", ["mixed", "fp64"])
-@pytest.mark.parametrize("m", [513, 575, 576, 577])
-def test_fit_b_beyond_one_cluster(vl, h, prec, m):
-    """The blocked factorisation: last blocks of 1, 63, 64 and 1 rows."""
+# one cluster: the last block of 1, 31 and 32 rows, the chain alone (up to 96),
+# one worker, seven, all of its range; beyond, the 64-wide blocks: last ones of
+# 1, 63, 64 and 1 rows
+@pytest.mark.parametrize("prec,m", [("mixed", m) for m in (2, 31, 32, 33, 64, 65, 96, 97, 128, 129,
+                                                           320, 385, 511, 512, 513, 575, 576, 577)]
+                         + [("fp64", m) for m in (513, 575, 576, 577)])
+def test_fit_b_at_the_edges_of_the_factorisations(vl, h, prec, m):
     rng = np.random.default_rng(m)
     n = 2 * m + 7
     L = np.tril(rng.uniform(-0.4, 0.4, (m, m)) * (rng.random((m, m)) < 3.0 / m), -1)
