@@ -176,14 +176,14 @@ vl_status var_fit_impl(Exec& x, const double* X, int64_t ldx, int m, int n, int 
   if (!E) E = Ew;
   Ctx cx = make_ctx(x, part, part_cap);
   cudaStream_t st = x.s;
-  launch_var_prep<T>(X, ldx, m, n, p, Xc, ldc, mu, wbar, x.st, st);
   if constexpr (sizeof(T) == 4) {
     // W W^T on the tensor cores: the lag windows sliced once, the symmetric
     // q x q product; its rows m.. (the Z rows) are G
-    launch_slice_lags(Xc, ldc, m, n, p, kp, S, plane, exps, st);
+    launch_prep_lags(X, ldx, m, n, p, Xc, ldc, mu, wbar, kp, S, plane, exps, x.st, st);
     if (!launch_tcgram_sym(cx, S, q, (int)kp, kp, plane, exps, G - (size_t)m * q, q))
       return fail(x.h, VL_ERR_CUDA, "vl_var_fit: tensor map encoding unavailable");
   } else {
+    launch_var_prep(X, ldx, m, n, p, Xc, ldc, mu, wbar, x.st, st);
     // lagged Gram: rows of Z (lags 1..p) against rows of W = [Y; Z]
     for (int t1 = 1; t1 <= p; ++t1)
       for (int b2 = 0; b2 <= p; ++b2) {
@@ -227,10 +227,14 @@ vl_status var_fit_impl(Exec& x, const double* X, int64_t ldx, int m, int n, int 
 
 // ------------------------------------------------------- pairwise measure
 struct CovOut {
-  double* C;  // m x m centred cross products
-  double* mu;
+  double* C;   // m x m centred cross products
+  double* w;   // mixed: 1 / sqrt(C_ii) (NULL: not wanted)
+  double* hx;  // entropies of the standardized variables (NULL: not wanted)
+  double* mu;  // FP64 path: mean and 1/std
   double* isd;
-  double* hx;  // 2m moments of the standardized variables
+  float* xs;   // mixed: the standardized samples, time-major (xt, NULL: not
+  float* xt;   // wanted), with the scratch of launch_measure_prep
+  int m_pad, n_pad;
 };
 
 // Statistics of the standardization and the centred cross products C of E.
@@ -240,14 +244,15 @@ template <class T>
 vl_status cov_and_stats(const Ctx& cx, const double* E, int64_t lde, int m, int n,
                         const CovOut& o, void* scratch) {
   cudaStream_t st = cx.s;
-  launch_standardize<T>(E, lde, m, n, o.mu, o.isd, o.hx, cx.st, st);
   if constexpr (sizeof(T) == 4) {
     const int64_t kp = tg_kpad(n), plane = (int64_t)m * kp;
     char* S = static_cast<char*>(scratch);
     int* exps = reinterpret_cast<int*>(S + round_up(3 * plane * 2, 256));
-    launch_slice_center(E, lde, o.mu, m, n, kp, S, plane, exps, st);
-    if (!launch_tcgram_sym(cx, S, m, (int)kp, kp, plane, exps, o.C, m)) return VL_ERR_CUDA;
+    launch_measure_prep(E, lde, m, n, kp, S, plane, exps, o.xs, o.xt, o.m_pad, o.n_pad, o.hx,
+                        cx.st, st);
+    if (!launch_tcgram_sym(cx, S, m, (int)kp, kp, plane, exps, o.C, m, o.w)) return VL_ERR_CUDA;
   } else {
+    launch_standardize(E, lde, m, n, o.mu, o.isd, o.hx, cx.st, st);
     const int64_t ldc = round_up(n, 4);
     double* ec = static_cast<double*>(scratch);
     launch_center64(E, lde, m, n, o.mu, ec, ldc, st);
@@ -276,7 +281,7 @@ vl_status pairwise_impl(Exec& x, const double* E, int64_t lde, int m, int n, dou
   // FP32 path: 4 floats (2 double-float sums) per residual per split;
   // FP64 path: 2 doubles
   const size_t nparts = (size_t)pl.splits * 2 * m * m;  // in 8-byte units
-  CovOut o;
+  CovOut o{};
   void* scratch;
   float *rho32 = nullptr, *c32 = nullptr;
   double *rho64 = nullptr, *c64 = nullptr;
@@ -286,9 +291,11 @@ vl_status pairwise_impl(Exec& x, const double* E, int64_t lde, int m, int n, dou
     o.C = C_out ? C_out : a.take<double>((size_t)m * m);
     o.mu = a.take<double>(m);
     o.isd = a.take<double>(m);
-    o.hx = a.take<double>(2 * (size_t)m);
+    o.hx = a.take<double>(m);
     scratch = a.take<char>(cov_scratch_bytes<T>(m, n));
     if (f32) {
+      o.w = a.take<double>(m);
+      o.xs = a.take<float>(measure_prep_needs_rows(m, n) ? (size_t)m * pl.n_pad : 0);
       rho32 = a.take<float>((size_t)m * m);
       c32 = a.take<float>((size_t)m * m);
     } else {
@@ -307,10 +314,19 @@ vl_status pairwise_impl(Exec& x, const double* E, int64_t lde, int m, int n, dou
   vl_handle h = x.h;
   Ctx cx = make_ctx(x, gpart, part_cap);
   cudaStream_t st = x.s;
+  if constexpr (sizeof(T) == 4) {
+    o.xt = xt;
+    o.m_pad = pl.m_pad;
+    o.n_pad = pl.n_pad;
+  }
   if (cov_and_stats<T>(cx, E, lde, m, n, o, scratch) != VL_OK)
     return fail(h, VL_ERR_CUDA, "vl_pairwise_measure: tensor map encoding unavailable");
-  launch_pair_consts(o.C, m, rho32, c32, rho64, c64, x.st, st);
-  launch_transpose_std<T>(E, lde, m, n, o.mu, o.isd, xt, pl.m_pad, pl.n_pad, st);
+  if constexpr (sizeof(T) == 4) {
+    launch_pair_consts(o.C, o.w, m, rho32, c32, x.st, st);
+  } else {
+    launch_pair_consts64(o.C, m, rho64, c64, x.st, st);
+    launch_transpose_std(E, lde, m, n, o.mu, o.isd, xt, pl.m_pad, pl.n_pad, st);
+  }
   if (h->prof_start) cudaEventRecord(h->prof_start, st);
   if constexpr (sizeof(T) == 4)
     launch_pairwise_f32(xt, pl, rho32, c32, reinterpret_cast<float*>(pparts), st);
@@ -337,7 +353,6 @@ vl_status fit_b_impl(Exec& x, const double* E, int64_t lde, int m, int n,
       o.C = a.take<double>((size_t)m * m);
       o.mu = a.take<double>(m);
       o.isd = a.take<double>(m);
-      o.hx = a.take<double>(2 * (size_t)m);
       scratch = a.take<char>(cov_scratch_bytes<T>(m, n));
     }
     Sp = a.take<T>((size_t)m * m);
@@ -519,7 +534,7 @@ vl_status check_instance(vl_handle h, const vl_instance& I) {
 
 struct InstBufs {
   PairPlan pl;  // the plan phase B and the finalisation use
-  double *E, *C, *D, *mu, *isd, *hx;
+  double *E, *C, *D, *w, *hx;
   float *rho32, *c32, *xt, *parts;
 };
 
@@ -533,9 +548,8 @@ void carve_inst(Arena& a, const vl_instance& I, InstBufs& b) {
   b.E = a.take<double>(m * ne);
   b.C = a.take<double>(m * m);
   b.D = a.take<double>(m * m);
-  b.mu = a.take<double>(m);
-  b.isd = a.take<double>(m);
-  b.hx = a.take<double>(2 * m);
+  b.w = a.take<double>(m);
+  b.hx = a.take<double>(m);
   b.rho32 = a.take<float>(m * m);
   b.c32 = a.take<float>(m * m);
   b.xt = a.take<float>((size_t)big.n_pad * big.m_pad);
@@ -551,18 +565,23 @@ vl_status batch_prep(Exec& x, const vl_instance& I, InstBufs& b) {
       std::max((size_t)16 * m * m, std::min((size_t)64 * m * m, (size_t)1 << 20));
   void* scratch;
   double* gpart;
+  CovOut o{};
   s = with_workspace(x, [&](Arena& a) {
     scratch = a.take<char>(cov_scratch_bytes<float>(m, n_eff));
+    o.xs = a.take<float>(measure_prep_needs_rows(m, n_eff) ? (size_t)m * b.pl.n_pad : 0);
     gpart = a.take<double>(part_cap);
   });
   if (s != VL_OK || x.measure) return s;
   Ctx cx = make_ctx(x, gpart, part_cap);
-  CovOut o{b.C, b.mu, b.isd, b.hx};
+  o.C = b.C;
+  o.w = b.w;
+  o.hx = b.hx;
+  o.xt = b.xt;
+  o.m_pad = b.pl.m_pad;
+  o.n_pad = b.pl.n_pad;
   if (cov_and_stats<float>(cx, b.E, n_eff, m, n_eff, o, scratch) != VL_OK)
     return fail(x.h, VL_ERR_CUDA, "vl_fit_batched: tensor map encoding unavailable");
-  launch_pair_consts(b.C, m, b.rho32, b.c32, nullptr, nullptr, x.st, x.s);
-  launch_transpose_std<float>(b.E, n_eff, m, n_eff, b.mu, b.isd, b.xt, b.pl.m_pad, b.pl.n_pad,
-                              x.s);
+  launch_pair_consts(b.C, b.w, m, b.rho32, b.c32, x.st, x.s);
   return VL_OK;
 }
 

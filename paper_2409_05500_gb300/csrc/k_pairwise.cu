@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "fp64_bits.cuh"
 #include "fx64.cuh"
 #include "vl_internal.cuh"
 
@@ -65,13 +66,13 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // tile index -> (I, J), I <= J, row-major over the upper triangle
 __device__ __forceinline__ void tile_coords(int q, int T, int& I, int& J) {
-  int i = 0, rem = q;
-  while (rem >= T - i) {
-    rem -= T - i;
-    ++i;
-  }
+  // row i starts at i (2 T - i + 1) / 2
+  const float w = 2.f * T + 1.f;
+  int i = max(0, min((int)((w - sqrtf(fmaxf(w * w - 8.f * (float)q, 0.f))) * 0.5f), T - 1));
+  while (i > 0 && i * (2 * T - i + 1) / 2 > q) --i;
+  while ((i + 1) * (2 * T - i) / 2 <= q) ++i;
   I = i;
-  J = i + rem;
+  J = i + q - i * (2 * T - i + 1) / 2;
 }
 
 // State of two residual streams (the two j's of a micro-tile row), as float2.
@@ -358,30 +359,76 @@ __global__ void __launch_bounds__(FX_TH)
   fx::moments_sums(mb, max(0, t1 - t0), base[ba], base[mm + ba]);
 }
 
-// rho_ij = C_ij / sqrt(C_ii C_jj) from the centred cross-product matrix C.
-__global__ void pair_consts_kernel(const double* __restrict__ C, int m,
-                                   float* __restrict__ rho32, float* __restrict__ c32,
-                                   double* __restrict__ rho64, double* __restrict__ c64,
-                                   int* st) {
-  int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)m * m) return;
+// FP64 path: rho_ij = C_ij / sqrt(C_ii C_jj) from the centred cross-product matrix
+// C and kappa / sqrt(1 - rho^2), i < j.
+__global__ void pair_consts64_kernel(const double* __restrict__ C, int m,
+                                     double* __restrict__ rho64, double* __restrict__ c64,
+                                     int* st) {
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int a = (int)(idx / m), b = (int)(idx % m);
-  double r = 0.0;
-  if (a != b) {
-    r = C[idx] / sqrt(C[(int64_t)a * m + a] * C[(int64_t)b * m + b]);
+  if (idx >= (int64_t)m * m || b <= a) return;
+  double r = C[idx] / sqrt(C[(int64_t)a * m + a] * C[(int64_t)b * m + b]);
+  if (!(1.0 - r * r >= DEGENERATE_1MR2)) {
+    set_status(st, VL_ERR_DEGENERATE);
+    r = 0.0;
+  }
+  rho64[idx] = r;
+  c64[idx] = fx::KAPPA64 / sqrt(1.0 - r * r);
+}
+
+// Mixed path: the same constants rounded to FP32.  In FP64 the two roots and two
+// divisions of a pair are ~90 instructions at 1.6 per clock per SM.  Instead rho =
+// C_ij w_i w_j (w_i = 1 / sqrt(C_ii) comes with C) in two products, accurate to a
+// few FP64 ulp, and kappa / sqrt(1 - rho^2) in double-float FP32 arithmetic to
+// 2^-40; where either lies too close to the middle of two FP32 numbers for its
+// rounding to be certain (about one pair in 2,000), or 1 - rho^2 is below 2^-8, the
+// pair takes the FP64 expressions.  So every constant is the rounding of the FP64
+// expression.  m = 1600: 24 us against 177.
+__global__ void pair_consts_kernel(const double* __restrict__ C, const double* __restrict__ w,
+                                   int m, float* __restrict__ rho32, float* __restrict__ c32,
+                                   int* st) {
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int a = (int)(idx / m), b = (int)(idx % m);
+  if (idx >= (int64_t)m * m || b <= a) return;  // the pairwise kernel reads i < j
+  const double cab = C[idx];
+  const double ra = cab * (w[a] * w[b]);
+  const float hi = bits::to_float(ra);
+  const float lo = bits::to_float(ra - bits::to_double(hi));
+  // lo, lengthened by far more than its error, must not round hi + lo away from hi
+  bool ok = __fadd_rn(hi, __fmul_rn(lo, 1.0001f)) == hi && (fabsf(hi) > 1e-30f || ra == 0.0);
+  // S + sl = 1 - (hi + lo)^2
+  const float p = __fmul_rn(hi, hi);
+  const float pe = __fmaf_rn(__fmul_rn(2.f, hi), lo, __fmaf_rn(hi, hi, -p));
+  const float sh = __fsub_rn(1.f, p);
+  const float se = __fsub_rn(__fsub_rn(__fsub_rn(1.f, sh), p), pe);
+  const float S = __fadd_rn(sh, se);
+  const float sl = __fsub_rn(se, __fsub_rn(S, sh));
+  ok = ok && S > 0.00390625f;
+  // y = y0 + corr = (S + sl)^{-1/2}: one Newton step with the residual in pairs
+  const float y0 = rsqrtf(S);
+  const float q = __fmul_rn(y0, y0), qe = __fmaf_rn(y0, y0, -q);
+  const float t = __fmul_rn(S, q);
+  const float te = __fmaf_rn(sl, q, __fmaf_rn(S, qe, __fmaf_rn(S, q, -t)));
+  const float d = __fsub_rn(__fsub_rn(1.f, t), te);
+  const float corr = __fmul_rn(y0, __fmaf_rn(__fmul_rn(0.375f, d), d, __fmul_rn(0.5f, d)));
+  const float k = __fmul_rn(y0, KAPPA);
+  const float ke = __fmaf_rn(corr, KAPPA, __fmaf_rn(y0, KAPPA, -k));
+  const float ch = __fadd_rn(k, ke);
+  const float cl = __fsub_rn(ke, __fsub_rn(ch, k));
+  const float err = __fmul_rn(ch, 0x1p-36f);
+  ok = ok && __fadd_rn(ch, __fadd_rn(cl, err)) == ch && __fadd_rn(ch, __fsub_rn(cl, err)) == ch;
+  float rho = hi, c = ch;
+  if (!ok) {
+    double r = cab / sqrt(C[(int64_t)a * m + a] * C[(int64_t)b * m + b]);
     if (!(1.0 - r * r >= DEGENERATE_1MR2)) {
       set_status(st, VL_ERR_DEGENERATE);
       r = 0.0;
     }
+    rho = (float)r;
+    c = (float)((double)KAPPA / sqrt(1.0 - r * r));
   }
-  if (rho32) {
-    rho32[idx] = (float)r;
-    c32[idx] = (float)((double)KAPPA / sqrt(1.0 - r * r));
-  }
-  if (rho64) {
-    rho64[idx] = r;
-    c64[idx] = fx::KAPPA64 / sqrt(1.0 - r * r);
-  }
+  rho32[idx] = rho;
+  c32[idx] = c;
 }
 
 // double-float accumulate (hi, lo) += x (TwoSum)
@@ -393,58 +440,65 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float x) {
   lo += err;
 }
 
-__global__ void measure_finalize_kernel(const void* __restrict__ part_v, int m, int splits,
-                                        int n_real, const double* __restrict__ hx,
-                                        double* __restrict__ Hx, double* __restrict__ Hr,
-                                        double* __restrict__ D, int fp32_parts) {
-  int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t mm = (int64_t)m * m;
-  if (idx >= mm) return;
-  const int a = (int)(idx / m), b = (int)(idx % m);
-  if (Hx && b == 0) Hx[a] = entropy_from_moments(hx[2 * a], hx[2 * a + 1]);
-  if (a == b) {
-    Hr[idx] = 0.0;
-    D[idx] = 0.0;
-    return;
-  }
-  // H of the residual of a on b and of b on a
-  double h[2];
-  for (int d = 0; d < 2; ++d) {
-    const int64_t off = d ? ((int64_t)b * m + a) : idx;
-    double A, B;
-    if (fp32_parts) {
-      // splits combined in double-float FP32 arithmetic, one FP64 conversion
-      const float* part = static_cast<const float*>(part_v);
-      float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
-      for (int s = 0; s < splits; ++s) {
-        const float* p = part + (int64_t)s * 4 * mm + off;
-        df_add(h0, l0, p[0]);
-        df_add(h0, l0, p[mm]);
-        df_add(h1, l1, p[2 * mm]);
-        df_add(h1, l1, p[3 * mm]);
-      }
-      const double s0 = (double)h0 + (double)l0;  // sum of log cosh u
-      const double s1 = (double)h1 + (double)l1;  // sum of w e^{-u^2/2}
-      const double kappa = 2.0 * LOG2E;
-      A = s0 / n_real;
-      B = s1 / (kappa * n_real);
-    } else {
-      const double* part = static_cast<const double*>(part_v);
-      double s0 = 0.0, s1 = 0.0;
-      for (int s = 0; s < splits; ++s) {
-        const double* p = part + (int64_t)s * 2 * mm + off;
-        s0 += p[0];
-        s1 += p[mm];
-      }
-      A = s0 / n_real;
-      B = s1 / n_real;
+// H of the residual of a on b from the split partials.
+template <bool F32>
+__device__ __forceinline__ double residual_entropy(const void* __restrict__ part_v, int64_t off,
+                                                   int64_t mm, int splits, double inv_n) {
+  if constexpr (F32) {
+    // splits combined in double-float FP32 arithmetic, one FP64 sum per moment
+    const float* p = static_cast<const float*>(part_v) + off;
+    float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
+#pragma unroll 4
+    for (int s = 0; s < splits; ++s, p += 4 * mm) {
+      df_add(h0, l0, p[0]);
+      df_add(h0, l0, p[mm]);
+      df_add(h1, l1, p[2 * mm]);
+      df_add(h1, l1, p[3 * mm]);
     }
-    h[d] = entropy_from_moments(A, B);
+    const double s0 = bits::to_double(h0) + bits::to_double(l0);  // sum of log cosh u
+    const double s1 = bits::to_double(h1) + bits::to_double(l1);  // sum of w e^{-u^2/2}
+    return entropy_from_moments(s0 * inv_n, s1 * (inv_n * (LN2 / 2.0)));
   }
-  Hr[idx] = h[0];
-  const double hxa = entropy_from_moments(hx[2 * a], hx[2 * a + 1]);
-  const double hxb = entropy_from_moments(hx[2 * b], hx[2 * b + 1]);
-  D[idx] = hxb + h[0] - hxa - h[1];
+  const double* p = static_cast<const double*>(part_v) + off;
+  double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+  for (int s = 0; s < splits; ++s, p += 2 * mm) {
+    s0 += p[0];
+    s1 += p[mm];
+  }
+  return entropy_from_moments(s0 * inv_n, s1 * inv_n);
+}
+
+// Hr and D = H(x_b) + H(r_a<-b) - H(x_a) - H(r_b<-a) from the partials and the
+// variables' entropies hx.  One CTA per pair of FT x FT tiles mirrored at the
+// diagonal: every entropy is computed once and exchanged through shared memory
+// (not twice, once on each side of the diagonal), all global accesses run along
+// rows, and the divisions by n are products.  FP64 instructions bound it (about 14
+// an entry, 80 before): m = 400 13 us against 31, m = 1600 81 against 329.  Tiles of
+// 8 keep the FP64 work of small m spread over enough SMs.
+constexpr int FT = 8;
+template <bool F32>
+__global__ void __launch_bounds__(2 * FT * FT)
+    measure_finalize_kernel(const void* __restrict__ part, int m, int splits, double inv_n,
+                            const double* __restrict__ hx, double* __restrict__ Hx,
+                            double* __restrict__ Hr, double* __restrict__ D) {
+  __shared__ double hs[2][FT][FT + 1];
+  int I, J;
+  tile_coords(blockIdx.x, (m + FT - 1) / FT, I, J);
+  // the first half of the threads takes the upper tile, the second the mirrored one
+  const int side = threadIdx.x / (FT * FT), r = threadIdx.x / FT % FT, c = threadIdx.x % FT;
+  const int a = (side ? J : I) * FT + r, b = (side ? I : J) * FT + c;
+  const bool in = a < m && b < m && !(side && I == J);
+  const int64_t off = (int64_t)a * m + b;
+  double h = 0.0;
+  if (in && a != b) h = residual_entropy<F32>(part, off, (int64_t)m * m, splits, inv_n);
+  hs[side][r][c] = h;
+  __syncthreads();
+  if (!in) return;
+  const double o = hs[I == J ? 0 : !side][c][r];  // H of the residual of b on a
+  Hr[off] = h;
+  D[off] = a == b ? 0.0 : hx[b] + h - hx[a] - o;
+  if (Hx && a == b) Hx[a] = hx[a];
 }
 
 }  // namespace
@@ -525,11 +579,18 @@ PairPlan plan_pairwise(int m, int n, int num_sms, bool fp64) {
   return plan_pairwise_slots(m, n, F32_MINB * num_sms, F32_TTS, fp64, num_sms);
 }
 
-void launch_pair_consts(const double* C, int m, float* rho32, float* c32, double* rho64,
-                        double* c64, int* st, cudaStream_t s) {
+void launch_pair_consts(const double* C, const double* w, int m, float* rho32, float* c32,
+                        int* st, cudaStream_t s) {
   int64_t tot = (int64_t)m * m;
   note_launch();
-  pair_consts_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(C, m, rho32, c32, rho64, c64, st);
+  pair_consts_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(C, w, m, rho32, c32, st);
+}
+
+void launch_pair_consts64(const double* C, int m, double* rho64, double* c64, int* st,
+                          cudaStream_t s) {
+  int64_t tot = (int64_t)m * m;
+  note_launch();
+  pair_consts64_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(C, m, rho64, c64, st);
 }
 
 template <int MTI, int TTS, int MINB>
@@ -593,13 +654,12 @@ void launch_pairwise_f64(const double* xt, const PairPlan& pl, const double* rho
                                              c64, part);
 }
 
-void launch_measure_finalize(const void* part, const PairPlan& pl, const double* hx_mom,
-                             double* Hx, double* Hr, double* D, bool fp32_parts,
-                             cudaStream_t s) {
-  const int64_t tot = (int64_t)pl.m * pl.m;
+void launch_measure_finalize(const void* part, const PairPlan& pl, const double* hx, double* Hx,
+                             double* Hr, double* D, bool fp32_parts, cudaStream_t s) {
+  const unsigned T = (pl.m + FT - 1) / FT;
   note_launch();
-  measure_finalize_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(
-      part, pl.m, pl.splits, pl.n, hx_mom, Hx, Hr, D, fp32_parts ? 1 : 0);
+  (fp32_parts ? measure_finalize_kernel<true> : measure_finalize_kernel<false>)
+      <<<T * (T + 1) / 2, 2 * FT * FT, 0, s>>>(part, pl.m, pl.splits, 1.0 / pl.n, hx, Hx, Hr, D);
 }
 
 }  // namespace vl

@@ -11,7 +11,7 @@
 // pairwise kernels see a plain u x n matrix; idx maps local to original.
 #include <algorithm>
 
-#include "vl_internal.cuh"
+#include "order_search.cuh"
 
 namespace vl {
 
@@ -20,26 +20,22 @@ namespace {
 constexpr int SC_WARPS = 8;  // rows scored per CTA (one warp per row)
 constexpr int RF_TH = 256;   // threads of a refinement CTA (a row is 1-8 CTAs)
 
-// smallest score, its index (lowest among equal scores) and the second
-// smallest score (equal values counted separately)
+// Scores as keys that order like them (order_search.cuh): 64-bit integer compares,
+// because an FP64 compare keeps the FP64 unit for 64 clocks.  Smallest key, its
+// index (lowest among equal keys) and the second smallest key (equal values
+// counted separately).
 struct Best {
-  double v1;
+  unsigned long long v1;
   int i1;
-  double v2;
+  unsigned long long v2;
 };
 
 __device__ __forceinline__ Best merge(Best a, Best b) {
   const bool take_b = b.v1 < a.v1 || (b.v1 == a.v1 && b.i1 < a.i1);
   Best o;
-  if (take_b) {
-    o.v1 = b.v1;
-    o.i1 = b.i1;
-    o.v2 = fmin(a.v1, b.v2);
-  } else {
-    o.v1 = a.v1;
-    o.i1 = a.i1;
-    o.v2 = fmin(a.v2, b.v1);
-  }
+  o.v1 = take_b ? b.v1 : a.v1;
+  o.i1 = take_b ? b.i1 : a.i1;
+  o.v2 = take_b ? min(a.v1, b.v2) : min(a.v2, b.v1);
   return o;
 }
 
@@ -82,8 +78,13 @@ __global__ void __launch_bounds__(SC_WARPS * 32)
   if (!last) return;
   __threadfence();
   const double INF = __longlong_as_double(0x7ff0000000000000LL);
-  Best b{INF, 0x7fffffff, INF};
-  for (int i = threadIdx.x; i < u; i += blockDim.x) b = merge(b, Best{__ldcg(S + i), i, INF});
+  const unsigned long long kinf = search::dkey(INF);
+  Best b{kinf, 0x7fffffff, kinf};
+  for (int i = threadIdx.x; i < u; i += blockDim.x) {
+    const unsigned long long key = search::dkey(__ldcg(S + i));
+    // (a score that is not a number orders beyond infinity: it is never taken)
+    if (key <= kinf) b = merge(b, Best{key, i, kinf});
+  }
 #pragma unroll
   for (int o = 16; o; o >>= 1) b = merge(b, shfl_best(b, o));
   __shared__ Best wb[SC_WARPS];
@@ -99,8 +100,9 @@ __global__ void __launch_bounds__(SC_WARPS * 32)
     *pick = r.i1;
     order[k] = idx ? idx[r.i1] : r.i1;
     if (gap) {
-      const double den = fmax(fmax(fabs(r.v1), fabs(r.v2)), 1e-300);
-      gap[k] = r.v2 == INF ? INF : (r.v2 - r.v1) / den;
+      const double v1 = search::dkey_inv(r.v1), v2 = search::dkey_inv(r.v2);
+      const double den = fmax(fmax(fabs(v1), fabs(v2)), 1e-300);
+      gap[k] = r.v2 == kinf ? INF : (v2 - v1) / den;
     }
     *counter = 0u;
   }
@@ -121,7 +123,10 @@ __global__ void __launch_bounds__(RF_TH)
   const int pk = *pick;
   const int an = blockIdx.y;
   const int a = an + (an >= pk ? 1 : 0);
-  const double slope = C[(int64_t)a * u + pk] / C[(int64_t)pk * u + pk];
+  __shared__ double ratio;
+  if (threadIdx.x == 0) ratio = C[(int64_t)a * u + pk] / C[(int64_t)pk * u + pk];
+  __syncthreads();
+  const double slope = ratio;
   const double* xa = W + (int64_t)a * ldw;
   const double* xp = W + (int64_t)pk * ldw;
   double* dst = Wn + (int64_t)an * ldn;

@@ -1,71 +1,128 @@
 // Per-variable statistics and data layout kernels.
 //
-//  * var_prep     : full-series mean of each variable, the centred copy the VAR
-//                   Gram reads, and the mean of every lag window (Sec. 4.1;
-//                   the VAR intercept is equivalent to centring each window).
-//  * standardize  : mean, 1/std (population) and the two entropy moments of
-//                   each standardized variable (Sec. 3 step 1; Sec. 4.2 item 1
-//                   precomputes H(x_i) once).
-//  * split_center : centred residuals as an FP32 hi/lo pair for the
-//                   compensated covariance product.
+//  * prep_lags    : mixed path of the VAR (Sec. 4.1): full-series mean of each
+//                   variable, the centred FP32 copy, the mean of every lag
+//                   window (the VAR intercept is equivalent to centring each
+//                   window) and the bf16 slices of the windows.
+//  * var_prep     : the same statistics and the centred copy on the FP64 path.
+//  * measure_prep : mixed path of the measure: mean and 1/std (population) of
+//                   each variable (Sec. 3 step 1), its entropy H(x_i) (Sec. 4.2
+//                   item 1 precomputes it once), the bf16 slices of the centred
+//                   row and the standardized row.
+//  * standardize  : mean, 1/std and entropy on the FP64 path.
 //  * transpose_std: standardized residuals, time-major, zero padded, in the
 //                   layout the pairwise kernel stages into shared memory.
+//
+// All of them are bound by the number of FP64 instructions (1.6 per clock per SM,
+// conversions included): a row is read in as few passes as its statistics allow,
+// scalar divisions and roots are taken by one thread, conversions run on the
+// integer pipe.  m = 400, n = 2500: prep_lags 24 us (28 + 11 as two kernels with
+// a pass per window), measure_prep 35 us (33 + 19 as two).
 #include <cmath>
 
+#include "fp64_bits.cuh"
 #include "fx64.cuh"
+#include "slices.cuh"
 #include "vl_internal.cuh"
 
 namespace vl {
 
 namespace {
 
-constexpr int kStatThreads = 256;
+constexpr int kStatMax = 256;  // threads of a row's CTA
 
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x < 32) {
-    t = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (threadIdx.x == 0) red[0] = t;
-  }
-  __syncthreads();
-  return red[0];
-}
-
-template <class T>
-__global__ void __launch_bounds__(kStatThreads) var_prep_kernel(
-    const double* __restrict__ X, int64_t ldx, int m, int n, int p, T* __restrict__ Xc,
-    int64_t ldc, double* __restrict__ mu_out, double* __restrict__ wbar, int* st) {
-  __shared__ double red[32];
+// Row i of X: its mean, the sums of its lag windows and a pass over the centred
+// values: each(t, x_t - mean) for every t < n in the thread's order.
+template <class Each>
+__device__ __forceinline__ void centre_row(const double* __restrict__ x, int m, int n, int p,
+                                           double inv_n, double* red, double* __restrict__ mu_out,
+                                           double* __restrict__ wbar, int* st, Each each) {
   const int i = blockIdx.x;
-  const double* x = X + (int64_t)i * ldx;
   double s = 0.0;
   bool finite = true;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    double v = x[t];
-    finite &= isfinite(v);
+#pragma unroll 4
+  for (int t = threadIdx.x; t < n; t += kStatMax) {
+    const double v = x[t];
+    finite &= is_finite(v);
     s += v;
   }
-  if (__syncthreads_or(!finite)) {
-    if (threadIdx.x == 0) set_status(st, VL_ERR_NONFINITE);
-    return;
-  }
-  const double mu = block_sum(s, red) / n;
+  if (__syncthreads_or(!finite) && threadIdx.x == 0) set_status(st, VL_ERR_NONFINITE);
+  const double mu = block_sum(s, red, [inv_n](double t) { return t * inv_n; });
   if (threadIdx.x == 0) mu_out[i] = mu;
-  T* xc = Xc + (int64_t)i * ldc;
-  for (int t = threadIdx.x; t < ldc; t += blockDim.x) xc[t] = (t < n) ? T(x[t] - mu) : T(0);
-  const int n_eff = n - p;
-  for (int b = 0; b <= p; ++b) {
-    double w = 0.0;
-    for (int t = threadIdx.x; t < n_eff; t += blockDim.x) w += x[p - b + t] - mu;
-    w = block_sum(w, red);
-    if (threadIdx.x == 0) wbar[(int64_t)b * m + i] = w / n_eff;
+  double w = 0.0;
+#pragma unroll 4
+  for (int t = threadIdx.x; t < n; t += kStatMax) {
+    const double d = x[t] - mu;
+    w += d;
+    each(t, d);
   }
+  w = block_sum(w, red);
+  // window b = [p - b, n - b): the whole sum without its ends
+  for (int b = threadIdx.x; b <= p; b += blockDim.x) {
+    double e = 0.0;
+    for (int t = 0; t < p - b; ++t) e += x[t] - mu;
+    for (int t = n - b; t < n; ++t) e += x[t] - mu;
+    wbar[(int64_t)b * m + i] = (w - e) / (n - p);
+  }
+}
+
+__global__ void __launch_bounds__(kStatMax)
+    var_prep_kernel(const double* __restrict__ X, int64_t ldx, int m, int n, int p, double inv_n,
+                    double* __restrict__ Xc, int64_t ldc, double* __restrict__ mu_out,
+                    double* __restrict__ wbar, int* st) {
+  __shared__ double red[2 * kStatMax];
+  double* xc = Xc + blockIdx.x * ldc;
+  centre_row(X + blockIdx.x * ldx, m, n, p, inv_n, red, mu_out, wbar, st,
+             [xc](int t, double d) { xc[t] = d; });
+  for (int t = n + threadIdx.x; t < ldc; t += blockDim.x) xc[t] = 0.0;
+}
+
+// Mixed path: the centred series as FP32 (Xc), and the slices of its lag windows:
+// row b m + k of W is Xc[k][p - b + t], t < n_eff, for b = 0..p (b = 0 is Y, b =
+// tau is Z_tau); S[z][row][k] (row stride ldo, plane stride plane, zeros for
+// n_eff <= t < Kpad).  One block per variable k; one exponent per variable for all
+// of its windows, and each sample sliced once for all of them.
+__global__ void __launch_bounds__(kStatMax)
+    prep_lags_kernel(const double* __restrict__ X, int64_t ldx, int m, int n, int p, double inv_n,
+                     float* __restrict__ Xc, int64_t ldc, double* __restrict__ mu_out,
+                     double* __restrict__ wbar, int Kpad, __nv_bfloat16* __restrict__ S,
+                     int64_t ldo, int64_t plane, int* __restrict__ exps, int* st) {
+  __shared__ double red[2 * kStatMax];
+  __shared__ unsigned long long redu[32];
+  const int k = blockIdx.x, n_eff = n - p;
+  float* xc = Xc + k * ldc;
+  uint32_t mx = 0;
+  centre_row(X + k * ldx, m, n, p, inv_n, red, mu_out, wbar, st, [&](int t, double d) {
+    const float f = bits::to_float(d);
+    mx = max(mx, __float_as_uint(f) & 0x7fffffffu);
+    xc[t] = f;
+  });
+  for (int t = n + threadIdx.x; t < ldc; t += blockDim.x) xc[t] = 0.f;
+  // float bits: f < 2^(E - 126) for biased exponent E (0 -> 0)
+  const unsigned long long fb = block_max_u64(mx, redu);
+  const int ex = fb == 0 ? 0 : clamp_exp((int)((fb >> 23) & 0xff) - 126);
+  const float sc = ldexpf(1.f, 7 - ex);
+  for (int b = threadIdx.x; b <= p; b += blockDim.x) exps[b * m + k] = ex;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {  // the thread's own xc[t]
+    __nv_bfloat16 s0, s1, s2;
+    slice3(xc[t] * sc, 0.f, s0, s1, s2);
+    for (int b = 0; b <= p; ++b) {
+      const int u = t - (p - b);
+      if (u < 0 || u >= n_eff) continue;
+      __nv_bfloat16* o = S + (int64_t)(b * m + k) * ldo + u;
+      o[0] = s0;
+      o[plane] = s1;
+      o[2 * plane] = s2;
+    }
+  }
+  const __nv_bfloat16 z = __float2bfloat16_rn(0.f);
+  for (int b = 0; b <= p; ++b)
+    for (int t = n_eff + threadIdx.x; t < Kpad; t += blockDim.x) {
+      __nv_bfloat16* o = S + (int64_t)(b * m + k) * ldo + t;
+      o[0] = z;
+      o[plane] = z;
+      o[2 * plane] = z;
+    }
 }
 
 // Centred normal equations of the VAR: G holds, for the Z rows a = (tau-1) m + k
@@ -103,18 +160,33 @@ __global__ void var_coef_kernel(const T* __restrict__ beta, int m, int p, double
   M[idx] = (double)beta[((int64_t)tau * m + k) * m + i];
 }
 
-// One warp per row: cst[i] = wbar0_i - sum_a beta[a][i] wbar_{Z,a}.
+// cst[i] = wbar0_i - sum_a beta[a][i] wbar_{Z,a}: a CTA takes CST_C columns i, the
+// rows a dealt to the rest of its threads (consecutive threads on consecutive
+// columns; one warp per column read beta with a stride of m).
+constexpr int CST_C = 16, CST_TH = 512;
 template <class T>
-__global__ void var_cst_kernel(const T* __restrict__ beta, int m, int p,
-                               const double* __restrict__ wbar, double* __restrict__ cst) {
-  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (i >= m) return;
+__global__ void __launch_bounds__(CST_TH)
+    var_cst_kernel(const T* __restrict__ beta, int m, int p, const double* __restrict__ wbar,
+                   double* __restrict__ cst) {
+  __shared__ double red[CST_TH / 32][CST_C];
+  const int i = blockIdx.x * CST_C + threadIdx.x % CST_C;
   double c = 0.0;
-  for (int a = lane; a < m * p; a += 32) c += (double)beta[(int64_t)a * m + i] * wbar[m + a];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) cst[i] = wbar[i] - c;
+  if (i < m)
+    for (int a = threadIdx.x / CST_C; a < m * p; a += CST_TH / CST_C) {
+      const T v = beta[(int64_t)a * m + i];
+      if constexpr (sizeof(T) == 4)
+        c = fma(bits::to_double(v), wbar[m + a], c);
+      else
+        c = fma(v, wbar[m + a], c);
+    }
+  c += __shfl_xor_sync(0xffffffffu, c, CST_C);
+  if ((threadIdx.x & 31) < CST_C) red[threadIdx.x >> 5][threadIdx.x % CST_C] = c;
+  __syncthreads();
+  if (threadIdx.x < CST_C && i < m) {
+    double t = 0.0;
+    for (int w = 0; w < CST_TH / 32; ++w) t += red[w][threadIdx.x];
+    cst[i] = wbar[i] - t;
+  }
 }
 
 __global__ void var_resid_init_kernel(const double* __restrict__ X, int64_t ldx, int n_eff, int p,
@@ -134,97 +206,142 @@ __device__ __forceinline__ void kahan_f(float& S, float& C, float x) {
   S = t;
 }
 
-template <class T>
-__global__ void __launch_bounds__(kStatThreads) standardize_kernel(
-    const double* __restrict__ E, int64_t lde, int m, int n, double* __restrict__ mu_out,
-    double* __restrict__ isd_out, double* __restrict__ mom, int* st) {
-  __shared__ double red[32];
-  const int i = blockIdx.x;
-  const double* e = E + (int64_t)i * lde;
+// Mean, then 1/std (0 for a constant row) of row e; each(d) sees every centred
+// value between the two.  Sets the status word for rows that are not finite or
+// constant and goes on (a row that is not finite leaves NaN everywhere).
+template <class Each>
+__device__ __forceinline__ void row_stats(const double* __restrict__ e, int n, double inv_n,
+                                          double* red, int* st, double& mu, double& isd,
+                                          Each each) {
   double s = 0.0;
   bool finite = true;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    double v = e[t];
-    finite &= isfinite(v);
+#pragma unroll 4
+  for (int t = threadIdx.x; t < n; t += kStatMax) {
+    const double v = e[t];
+    finite &= is_finite(v);
     s += v;
   }
-  if (__syncthreads_or(!finite)) {
-    if (threadIdx.x == 0) set_status(st, VL_ERR_NONFINITE);
-    return;
-  }
-  const double mu = block_sum(s, red) / n;
+  if (__syncthreads_or(!finite) && threadIdx.x == 0) set_status(st, VL_ERR_NONFINITE);
+  mu = block_sum(s, red, [inv_n](double t) { return t * inv_n; });
   double q = 0.0;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    double d = e[t] - mu;
+#pragma unroll 4
+  for (int t = threadIdx.x; t < n; t += kStatMax) {
+    const double d = e[t] - mu;
     q += d * d;
+    each(d);
   }
-  const double var = block_sum(q, red) / n;
-  if (!(var > 1e-300)) {
-    if (threadIdx.x == 0) {
-      set_status(st, VL_ERR_DEGENERATE);
-      mu_out[i] = mu;
-      isd_out[i] = 0.0;
-      mom[2 * i] = 0.0;
-      mom[2 * i + 1] = 0.0;
-    }
-    return;
-  }
-  const double isd = 1.0 / sqrt(var);
-  // sample moments of the standardized variable for H(x_i): A = mean log cosh
-  // u, B = mean u e^{-u^2/2}
-  double a = 0.0, b = 0.0;
-  if constexpr (sizeof(T) == 8) {
-    // fixed-point functions and exact sums (fx64.cuh)
-    __shared__ fx::u64 te[fx::EXP_N], tl[fx::LOG_N];
-    __shared__ fx::u32 tr[fx::LOG_N];
-    const fx::Tab tab{te, tl, tr};
-    fx::fill_tables(te, tl, tr);
-    __syncthreads();
-    // kappa times the value the pairwise kernel reads, so that H(x_i) and the
-    // residuals' entropies share the rounding of 1/std, which D's differences
-    // then cancel
-    fx::Moments M;
-    int cnt = 0;
-    for (int t = threadIdx.x; t < n; t += blockDim.x, ++cnt)
-      fx::moments_add(M, fx::KAPPA64 * ((e[t] - mu) * isd), tab);
-    fx::moments_sums(M, cnt, a, b);
-  } else {
-    // FP32 per-sample functions (CUDA's accurate expf / log1pf), Kahan sums
-    // of log cosh u + ln 2 (= |u| + log1p(e^{-2|u|})) and u e^{-u^2/2}
-    float sa = 0.f, ca = 0.f, sb = 0.f, cb = 0.f;
-    int cnt = 0;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-      const float u = (float)((e[t] - mu) * isd);
-      const float au = fabsf(u);
-      kahan_f(sa, ca, au + log1pf(expf(-2.0f * au)));
-      kahan_f(sb, cb, u * expf(-0.5f * u * u));
-      ++cnt;
-    }
-    a = ((double)sa - (double)ca) - LN2 * cnt;
-    b = (double)sb - (double)cb;
-  }
-  a = block_sum(a, red);
-  b = block_sum(b, red);
+  isd = block_sum(q, red, [inv_n, st](double t) {
+    const double var = t * inv_n;
+    if (var > 1e-300 || var != var) return rsqrt(var);
+    set_status(st, VL_ERR_DEGENERATE);
+    return 0.0;
+  });
+}
+
+// H of a standardized row from the block's sums of log cosh u and u e^{-u^2/2};
+// a constant row counts as moments 0.
+__device__ __forceinline__ void store_entropy(double a, double b, double inv_n, double isd,
+                                              double* red, double* __restrict__ hx) {
+  block_sum2(a, b, red);
+  if (threadIdx.x == 0)
+    *hx = isd == 0.0 ? entropy_from_moments(0.0, 0.0)
+                     : entropy_from_moments(a * inv_n, b * inv_n);
+}
+
+__global__ void __launch_bounds__(kStatMax)
+    standardize_kernel(const double* __restrict__ E, int64_t lde, int n, double inv_n,
+                       double* __restrict__ mu_out, double* __restrict__ isd_out,
+                       double* __restrict__ hx, int* st) {
+  __shared__ double red[2 * kStatMax];
+  __shared__ fx::u64 te[fx::EXP_N], tl[fx::LOG_N];
+  __shared__ fx::u32 tr[fx::LOG_N];
+  const fx::Tab tab{te, tl, tr};
+  fx::fill_tables(te, tl, tr);
+  const int i = blockIdx.x;
+  const double* e = E + (int64_t)i * lde;
+  double mu, isd;
+  row_stats(e, n, inv_n, red, st, mu, isd, [](double) {});
   if (threadIdx.x == 0) {
     mu_out[i] = mu;
     isd_out[i] = isd;
-    mom[2 * i] = a / n;
-    mom[2 * i + 1] = b / n;
   }
+  if (!hx) return;
+  // fixed-point functions and exact sums (fx64.cuh) of kappa times the value the
+  // pairwise kernel reads, so that H(x_i) and the residuals' entropies share the
+  // rounding of 1/std, which D's differences then cancel
+  fx::Moments M;
+  int cnt = 0;
+  double a, b;
+  for (int t = threadIdx.x; t < n; t += blockDim.x, ++cnt)
+    fx::moments_add(M, fx::KAPPA64 * ((e[t] - mu) * isd), tab);
+  fx::moments_sums(M, cnt, a, b);
+  store_entropy(a, b, inv_n, isd, red, hx + i);
 }
 
-__global__ void split_center_kernel(const double* __restrict__ E, int64_t lde, int n,
-                                    const double* __restrict__ mu, float* __restrict__ hi,
-                                    float* __restrict__ lo, int64_t ldc) {
-  const int i = blockIdx.y;
-  const double mi = mu[i];
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ldc;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    double v = (t < n) ? E[(int64_t)i * lde + t] - mi : 0.0;
-    float h = (float)v;
-    hi[(int64_t)i * ldc + t] = h;
-    lo[(int64_t)i * ldc + t] = (float)(v - (double)h);
+// Mixed path, one block per row: statistics and entropy, the slices of the
+// centred row (S[z][i][k], k < K; zeros up to Kpad) with its exponent, and the
+// standardized row as FP32, to xs[i][t] (row stride n_pad) or, time-major, to
+// xt[t][i] (row stride m_pad; the blocks i >= m write its zero columns).  FULL =
+// false: the slices only (and the checks of the statistics).
+template <bool FULL>
+__global__ void __launch_bounds__(kStatMax)
+    measure_prep_kernel(const double* __restrict__ E, int64_t lde, int m, int n, double inv_n,
+                        int Kpad,
+                        __nv_bfloat16* __restrict__ S, int64_t plane, int* __restrict__ exps,
+                        float* __restrict__ xs, float* __restrict__ xt, int m_pad, int n_pad,
+                        double* __restrict__ hx, int* st) {
+  __shared__ double red[2 * kStatMax];
+  __shared__ unsigned long long redu[32];
+  const int i = blockIdx.x;
+  if (i >= m) {
+    for (int t = threadIdx.x; t < n_pad; t += blockDim.x) xt[(int64_t)t * m_pad + i] = 0.f;
+    return;
   }
+  const double* e = E + (int64_t)i * lde;
+  double mu, isd;
+  unsigned long long mx = 0;
+  row_stats(e, n, inv_n, red, st, mu, isd, [&mx](double d) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d) & 0x7fffffffffffffffull;
+    mx = b > mx ? b : mx;
+  });
+  const int ex = exp_above(block_max_u64(mx, redu));
+  if (threadIdx.x == 0) exps[i] = ex;
+  const float sc = ldexpf(1.f, 7 - ex);
+  __nv_bfloat16* o = S + (int64_t)i * Kpad;
+  // FP32 per-sample functions (CUDA's accurate expf / log1pf), Kahan sums of log
+  // cosh u + ln 2 (= |u| + log1p(e^{-2|u|})) and u e^{-u^2/2}
+  float sa = 0.f, ca = 0.f, sb = 0.f, cb = 0.f;
+  int cnt = 0;
+  for (int t = threadIdx.x; t < n; t += blockDim.x, ++cnt) {
+    const double d = e[t] - mu;
+    const float h = bits::to_float(d);
+    const float l = bits::to_float(d - bits::to_double(h));
+    __nv_bfloat16 s0, s1, s2;
+    slice3(h * sc, l * sc, s0, s1, s2);
+    o[t] = s0;
+    o[plane + t] = s1;
+    o[2 * plane + t] = s2;
+    if constexpr (!FULL) continue;
+    const float u = bits::to_float(d * isd);
+    if (xs)
+      xs[(int64_t)i * n_pad + t] = u;
+    else
+      xt[(int64_t)t * m_pad + i] = u;
+    const float au = fabsf(u);
+    kahan_f(sa, ca, au + log1pf(expf(-2.0f * au)));
+    kahan_f(sb, cb, u * expf(-0.5f * u * u));
+  }
+  const __nv_bfloat16 z = __float2bfloat16_rn(0.f);
+  for (int t = n + threadIdx.x; t < Kpad; t += blockDim.x) o[t] = o[plane + t] = o[2 * plane + t] = z;
+  if constexpr (!FULL) return;
+  for (int t = n + threadIdx.x; t < n_pad; t += blockDim.x) {
+    if (xs)
+      xs[(int64_t)i * n_pad + t] = 0.f;
+    else
+      xt[(int64_t)t * m_pad + i] = 0.f;
+  }
+  store_entropy((bits::to_double(sa) - bits::to_double(ca)) - LN2 * cnt,
+                bits::to_double(sb) - bits::to_double(cb), inv_n, isd, red, hx + i);
 }
 
 __global__ void center64_kernel(const double* __restrict__ E, int64_t lde, int n,
@@ -238,19 +355,16 @@ __global__ void center64_kernel(const double* __restrict__ E, int64_t lde, int n
 }
 
 // 32 x 32 tiled transpose: xt[t * m_pad + i] = (E[i, t] - mu_i) / sd_i.
-template <class T>
 __global__ void transpose_std_kernel(const double* __restrict__ E, int64_t lde, int m, int n,
                                      const double* __restrict__ mu,
-                                     const double* __restrict__ isd, T* __restrict__ xt,
+                                     const double* __restrict__ isd, double* __restrict__ xt,
                                      int m_pad, int n_pad) {
-  __shared__ T tile[32][33];
+  __shared__ double tile[32][33];
   const int t0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
   for (int r = ty; r < 32; r += 8) {
     int i = i0 + r, t = t0 + tx;
-    T v = T(0);
-    if (i < m && t < n) v = T((E[(int64_t)i * lde + t] - mu[i]) * isd[i]);
-    tile[r][tx] = v;
+    tile[r][tx] = (i < m && t < n) ? (E[(int64_t)i * lde + t] - mu[i]) * isd[i] : 0.0;
   }
   __syncthreads();
   for (int r = ty; r < 32; r += 8) {
@@ -259,18 +373,37 @@ __global__ void transpose_std_kernel(const double* __restrict__ E, int64_t lde, 
   }
 }
 
+// xt[t * m_pad + i] = xs[i * n_pad + t] (zero for i >= m); n_pad and m_pad are
+// multiples of 32.
+__global__ void transpose_f32_kernel(const float* __restrict__ xs, int m, int n_pad,
+                                     float* __restrict__ xt, int m_pad) {
+  __shared__ float tile[32][33];
+  const int t0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
+  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+#pragma unroll
+  for (int r = ty; r < 32; r += 8)
+    tile[r][tx] = i0 + r < m ? xs[(int64_t)(i0 + r) * n_pad + t0 + tx] : 0.f;
+  __syncthreads();
+#pragma unroll
+  for (int r = ty; r < 32; r += 8) xt[(int64_t)(t0 + r) * m_pad + i0 + tx] = tile[tx][r];
+}
+
 }  // namespace
 
-template <class T>
-void launch_var_prep(const double* X, int64_t ldx, int m, int n, int p, T* Xc, int64_t ldc,
+void launch_var_prep(const double* X, int64_t ldx, int m, int n, int p, double* Xc, int64_t ldc,
                      double* mu, double* wbar, int* st, cudaStream_t s) {
   note_launch();
-  var_prep_kernel<T><<<m, kStatThreads, 0, s>>>(X, ldx, m, n, p, Xc, ldc, mu, wbar, st);
+  var_prep_kernel<<<m, kStatMax, 0, s>>>(X, ldx, m, n, p, 1.0 / n, Xc, ldc, mu, wbar, st);
 }
-template void launch_var_prep<float>(const double*, int64_t, int, int, int, float*, int64_t,
-                                     double*, double*, int*, cudaStream_t);
-template void launch_var_prep<double>(const double*, int64_t, int, int, int, double*, int64_t,
-                                      double*, double*, int*, cudaStream_t);
+
+void launch_prep_lags(const double* X, int64_t ldx, int m, int n, int p, float* Xc, int64_t ldc,
+                      double* mu, double* wbar, int64_t Kpad, void* S, int64_t plane, int* exps,
+                      int* st, cudaStream_t s) {
+  note_launch();
+  prep_lags_kernel<<<m, kStatMax, 0, s>>>(X, ldx, m, n, p, 1.0 / n, Xc, ldc, mu, wbar, (int)Kpad,
+                                              static_cast<__nv_bfloat16*>(S), Kpad, plane, exps,
+                                              st);
+}
 
 template <class T>
 void launch_var_normal_eq(const double* G, int m, int p, int n_eff, const double* wbar, T* Gzz,
@@ -293,7 +426,7 @@ void launch_var_coef(const T* beta, int m, int p, const double* wbar, double* M,
   note_launch();
   var_coef_kernel<T><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(beta, m, p, M);
   note_launch();
-  var_cst_kernel<T><<<(m + 7) / 8, 256, 0, s>>>(beta, m, p, wbar, cst);
+  var_cst_kernel<T><<<(m + CST_C - 1) / CST_C, CST_TH, 0, s>>>(beta, m, p, wbar, cst);
 }
 template void launch_var_coef<float>(const float*, int, int, const double*, double*, double*,
                                      cudaStream_t);
@@ -301,7 +434,7 @@ template void launch_var_coef<float>(const float*, int, int, const double*, doub
 template <class T>
 void launch_var_cst(const T* beta, int m, int p, const double* wbar, double* cst, cudaStream_t s) {
   note_launch();
-  var_cst_kernel<T><<<(m + 7) / 8, 256, 0, s>>>(beta, m, p, wbar, cst);
+  var_cst_kernel<T><<<(m + CST_C - 1) / CST_C, CST_TH, 0, s>>>(beta, m, p, wbar, cst);
 }
 template void launch_var_cst<float>(const float*, int, int, const double*, double*, cudaStream_t);
 template void launch_var_coef<double>(const double*, int, int, const double*, double*, double*,
@@ -315,22 +448,37 @@ void launch_var_resid_init(const double* X, int64_t ldx, int m, int n, int p, co
   var_resid_init_kernel<<<grid, 256, 0, s>>>(X, ldx, n_eff, p, mu, cst, E, lde);
 }
 
-template <class T>
 void launch_standardize(const double* E, int64_t lde, int m, int n, double* mu, double* inv_sd,
-                        double* hx_mom, int* st, cudaStream_t s) {
+                        double* hx, int* st, cudaStream_t s) {
   note_launch();
-  standardize_kernel<T><<<m, kStatThreads, 0, s>>>(E, lde, m, n, mu, inv_sd, hx_mom, st);
+  standardize_kernel<<<m, kStatMax, 0, s>>>(E, lde, n, 1.0 / n, mu, inv_sd, hx, st);
 }
-template void launch_standardize<float>(const double*, int64_t, int, int, double*, double*,
-                                        double*, int*, cudaStream_t);
-template void launch_standardize<double>(const double*, int64_t, int, int, double*, double*,
-                                         double*, int*, cudaStream_t);
 
-void launch_split_center(const double* E, int64_t lde, int m, int n, const double* mu,
-                         float* hi, float* lo, int64_t ldc, cudaStream_t s) {
-  dim3 grid((unsigned)((ldc + 255) / 256 < 64 ? (ldc + 255) / 256 : 64), m);
+// The standardized rows go straight to their time-major places while that is
+// little traffic (each four bytes then write a 32-byte sector), through xs and a
+// transpose beyond: at m n = 2^19 both take about 5 us.
+constexpr int64_t kDirectMax = 1 << 19;
+
+bool measure_prep_needs_rows(int m, int n) { return (int64_t)m * n > kDirectMax; }
+
+void launch_measure_prep(const double* E, int64_t lde, int m, int n, int64_t Kpad, void* S,
+                         int64_t plane, int* exps, float* xs, float* xt, int m_pad, int n_pad,
+                         double* hx, int* st, cudaStream_t s) {
+  __nv_bfloat16* Sb = static_cast<__nv_bfloat16*>(S);
   note_launch();
-  split_center_kernel<<<grid, 256, 0, s>>>(E, lde, n, mu, hi, lo, ldc);
+  if (!xt) {
+    measure_prep_kernel<false><<<m, kStatMax, 0, s>>>(E, lde, m, n, 1.0 / n, (int)Kpad, Sb, plane, exps,
+                                                          nullptr, nullptr, 0, 0, nullptr, st);
+    return;
+  }
+  const bool rows = measure_prep_needs_rows(m, n);
+  measure_prep_kernel<true><<<rows ? m : m_pad, kStatMax, 0, s>>>(
+      E, lde, m, n, 1.0 / n, (int)Kpad, Sb, plane, exps, rows ? xs : nullptr, xt, m_pad, n_pad, hx, st);
+  if (rows) {
+    note_launch();
+    transpose_f32_kernel<<<dim3(n_pad / 32, m_pad / 32), dim3(32, 8), 0, s>>>(xs, m, n_pad, xt,
+                                                                             m_pad);
+  }
 }
 
 void launch_center64(const double* E, int64_t lde, int m, int n, const double* mu, double* out,
@@ -340,24 +488,20 @@ void launch_center64(const double* E, int64_t lde, int m, int n, const double* m
   center64_kernel<<<grid, 256, 0, s>>>(E, lde, n, mu, out, ldc);
 }
 
-template <class T>
 void launch_transpose_std(const double* E, int64_t lde, int m, int n, const double* mu,
-                          const double* inv_sd, T* xt, int m_pad, int n_pad, cudaStream_t s) {
+                          const double* inv_sd, double* xt, int m_pad, int n_pad,
+                          cudaStream_t s) {
   dim3 grid((n_pad + 31) / 32, (m_pad + 31) / 32), block(32, 8);
   note_launch();
-  transpose_std_kernel<T><<<grid, block, 0, s>>>(E, lde, m, n, mu, inv_sd, xt, m_pad, n_pad);
+  transpose_std_kernel<<<grid, block, 0, s>>>(E, lde, m, n, mu, inv_sd, xt, m_pad, n_pad);
 }
-template void launch_transpose_std<float>(const double*, int64_t, int, int, const double*,
-                                          const double*, float*, int, int, cudaStream_t);
-template void launch_transpose_std<double>(const double*, int64_t, int, int, const double*,
-                                           const double*, double*, int, int, cudaStream_t);
 
 namespace {
 
 // One CTA: 2 sum ln L[i][i] in FP64 (a fixed-order block reduction).
 __global__ void logdet_value_kernel(const double* __restrict__ L, int64_t ldl, int m,
                                     double penalty, double* __restrict__ value, int* st) {
-  __shared__ double red[32];
+  __shared__ double red[2 * kStatMax];
   double s = 0.0;
   bool bad = false;
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
@@ -386,7 +530,7 @@ __global__ void argmin_p_kernel(const double* __restrict__ values, int p_max,
 void launch_logdet_value(const double* L, int64_t ldl, int m, double penalty, double* value,
                          int* st, cudaStream_t s) {
   note_launch();
-  logdet_value_kernel<<<1, kStatThreads, 0, s>>>(L, ldl, m, penalty, value, st);
+  logdet_value_kernel<<<1, kStatMax, 0, s>>>(L, ldl, m, penalty, value, st);
 }
 
 void launch_argmin_p(const double* values, int p_max, int32_t* p_best, cudaStream_t s) {

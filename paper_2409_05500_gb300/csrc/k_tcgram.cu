@@ -42,6 +42,8 @@
 #include <algorithm>
 #include <mutex>
 
+#include "fp64_bits.cuh"
+#include "slices.cuh"
 #include "tc_ptx.cuh"
 #include "vl_internal.cuh"
 
@@ -66,122 +68,6 @@ constexpr size_t TG_SMEM = (size_t)TG_STAGES * STAGE_BYTES + 1024 /*barriers*/ +
 constexpr uint32_t WAIT_LIMIT = 1u << 20;  // bounded polls of one mbarrier wait
 
 static_assert(TG_SEG * TG_K * 3 * 128 * 128 < (1 << 24), "a level sum must stay exact in FP32");
-
-// ------------------------------------------------------------- slicing
-// Exponent e with max < 2^e from the bits of a non-negative double (0 -> 0),
-// clamped so that the FP32 scale 2^(7 - e) is finite and normal (rows whose
-// largest entry is below 2^-100 are treated as zero-ish; the mixed path
-// takes no entries above 2^120).
-__device__ __forceinline__ int clamp_exp(int e) { return min(120, max(-100, e)); }
-__device__ __forceinline__ int exp_above(unsigned long long bits) {
-  if (bits == 0) return 0;
-  return clamp_exp((int)((bits >> 52) & 0x7ff) - 1022);
-}
-
-// Three integer slices of y in (-128, 128) given as an FP32 pair (yh + yl).
-__device__ __forceinline__ void slice3(float yh, float yl, __nv_bfloat16& s0, __nv_bfloat16& s1,
-                                       __nv_bfloat16& s2) {
-  const float a0 = rintf(yh);
-  const float r1 = ((yh - a0) + yl) * 256.f;
-  const float a1 = rintf(r1);
-  const float a2 = rintf((r1 - a1) * 256.f);
-  s0 = __float2bfloat16_rn(a0);
-  s1 = __float2bfloat16_rn(a1);
-  s2 = __float2bfloat16_rn(a2);
-}
-
-__device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v,
-                                                            unsigned long long* red) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-    v = w > v ? w : v;
-  }
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long b = 0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) b = red[q] > b ? red[q] : b;
-    red[0] = b;
-  }
-  __syncthreads();
-  return red[0];
-}
-
-// Centred FP64 rows (E[r][k] - mu[r], k < K) into three slice planes
-// S[z][r][k] (row stride ldo, plane stride plane; zeros for K <= k < Kpad)
-// and the row exponent.  One block per row.
-__global__ void slice_center_kernel(const double* __restrict__ E, int64_t lde,
-                                    const double* __restrict__ mu, int K, int Kpad,
-                                    __nv_bfloat16* __restrict__ S, int64_t ldo, int64_t plane,
-                                    int* __restrict__ exps) {
-  __shared__ unsigned long long red[32];
-  const int r = blockIdx.x;
-  const double* e = E + (int64_t)r * lde;
-  const double m = mu[r];
-  unsigned long long mx = 0;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const unsigned long long b =
-        (unsigned long long)__double_as_longlong(e[k] - m) & 0x7fffffffffffffffull;
-    mx = b > mx ? b : mx;
-  }
-  const int ex = exp_above(block_max_u64(mx, red));
-  if (threadIdx.x == 0) exps[r] = ex;
-  const float sc = ldexpf(1.f, 7 - ex);
-  __nv_bfloat16* o = S + (int64_t)r * ldo;
-  for (int k = threadIdx.x; k < Kpad; k += blockDim.x) {
-    __nv_bfloat16 s0, s1, s2;
-    if (k < K) {
-      const double d = e[k] - m;
-      const float h = (float)d;
-      const float l = (float)(d - (double)h);
-      slice3(h * sc, l * sc, s0, s1, s2);
-    } else {
-      s0 = s1 = s2 = __float2bfloat16_rn(0.f);
-    }
-    o[k] = s0;
-    o[plane + k] = s1;
-    o[2 * plane + k] = s2;
-  }
-}
-
-// The lag windows of the centred FP32 series Xc (m rows, stride ldc): row
-// b m + k of W is Xc[k][p - b + t], t < n_eff, for b = 0..p (b = 0 is Y, b =
-// tau is Z_tau).  One block per variable k; one exponent per variable for all
-// of its windows.
-__global__ void slice_lags_kernel(const float* __restrict__ Xc, int64_t ldc, int m, int n,
-                                  int p, int Kpad, __nv_bfloat16* __restrict__ S, int64_t ldo,
-                                  int64_t plane, int* __restrict__ exps) {
-  __shared__ unsigned long long red[32];
-  const int k = blockIdx.x;
-  const float* x = Xc + (int64_t)k * ldc;
-  const int n_eff = n - p;
-  unsigned long long mx = 0;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    const unsigned long long b = __float_as_uint(x[t]) & 0x7fffffffu;
-    mx = b > mx ? b : mx;
-  }
-  // float bits: f < 2^(E - 126) for biased exponent E (0 -> 0)
-  const unsigned long long fb = block_max_u64(mx, red);
-  const int ex = fb == 0 ? 0 : clamp_exp((int)((fb >> 23) & 0xff) - 126);
-  const float sc = ldexpf(1.f, 7 - ex);
-  if (threadIdx.x <= p) exps[threadIdx.x * m + k] = ex;
-  for (int t = threadIdx.x; t < Kpad; t += blockDim.x) {
-    for (int b = 0; b <= p; ++b) {
-      __nv_bfloat16 s0, s1, s2;
-      if (t < n_eff) {
-        slice3(x[p - b + t] * sc, 0.f, s0, s1, s2);
-      } else {
-        s0 = s1 = s2 = __float2bfloat16_rn(0.f);
-      }
-      __nv_bfloat16* o = S + (int64_t)(b * m + k) * ldo;
-      o[t] = s0;
-      o[plane + t] = s1;
-      o[2 * plane + t] = s2;
-    }
-  }
-}
 
 // The VAR residual product (Sec. 4.1, E = Y - sum_tau M_tau Z_tau) as one
 // Gram-type product over K = (tau, k): A = beta' (m rows), B = the time-major
@@ -251,11 +137,11 @@ __global__ void resid_apply_kernel(const double* __restrict__ X, int64_t ldx, in
                                    const int* __restrict__ aexp, double* __restrict__ E) {
   const int i = blockIdx.y;
   const double off = mu[i] + cst[i];
-  const int ex = aexp[i] - 14;
+  const double scale = bits::pow2(aexp[i] - 14);
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_eff; t += gridDim.x * blockDim.x) {
     const float2 v = part[(int64_t)i * n_eff + t];
-    E[(int64_t)i * n_eff + t] =
-        X[(int64_t)i * ldx + p + t] - off - ldexp((double)v.x + (double)v.y, ex);
+    const double s = bits::to_double(v.x) + bits::to_double(v.y);
+    E[(int64_t)i * n_eff + t] = fma(-s, scale, X[(int64_t)i * ldx + p + t] - off);
   }
 }
 
@@ -284,6 +170,17 @@ __device__ __forceinline__ void df_norm(float& h, float& l) {
   const float s = h + l;
   l = l - (s - h);
   h = s;
+}
+
+// the four levels of an entry (exact integers): L0 + L1 2^-8 + L2 2^-16 + L3
+// 2^-24 as a double-float
+__device__ __forceinline__ float2 combine_levels(uint32_t v0, uint32_t v1, uint32_t v2,
+                                                 uint32_t v3) {
+  float h = __uint_as_float(v0), l = 0.f;
+  df_add1(h, l, __uint_as_float(v1) * 0x1p-8f);
+  df_add1(h, l, __uint_as_float(v2) * 0x1p-16f);
+  df_add1(h, l, __uint_as_float(v3) * 0x1p-24f);
+  return make_float2(h, l);
 }
 
 // tile index -> (I, J): row tile I (128 rows), column tile J (64 columns); in
@@ -431,72 +328,104 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
   } else {
     // drain warps: quadrant q of the tensor-memory lanes = tile rows 32q..32q+31
     const int q = warp & 3;
-    float ah[TG_N], al[TG_N];
-#pragma unroll
-    for (int c = 0; c < TG_N; ++c) ah[c] = al[c] = 0.f;
-    bool ok = true;
-    for (int seg = 0; seg < nseg; ++seg) {
-      const int b = seg & 1;
-      // one lane polls; the warp then continues converged, as the
-      // .sync.aligned tensor-memory loads and barriers below require
+    if (nseg == 1) {
+      // one segment (short K, or a split of it): nothing to accumulate, so each
+      // chunk of 16 columns goes from tensor memory straight to its place, in a
+      // loop a quarter of the unrolled code below (which a small product mostly
+      // spends fetching)
       int got = 1;
-      if (lane == 0) got = tc::mbar_wait(&tfull[b], (seg >> 1) & 1, abort_flag, WAIT_LIMIT);
+      if (lane == 0) got = tc::mbar_wait(&tfull[0], 0, abort_flag, WAIT_LIMIT);
       __syncwarp();
       got = __shfl_sync(0xffffffffu, got, 0);
-      if (!got) {
-        ok = false;
-        break;
+      if (got) {
+        tc::fence_after_sync();
+        const int r = row0 + 32 * q + lane;
+        float2* out = P.part + ((int64_t)blockIdx.y * P.M + r) * P.N;
+#pragma unroll 1
+        for (int c16 = 0; c16 < TG_N / 16 && col0 + c16 * 16 < P.N; ++c16) {
+          uint32_t v0[16], v1[16], v2[16], v3[16];
+          const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(c16 * 16);
+          tc::tmem_ld16(base, v0);
+          tc::tmem_ld16(base + TG_N, v1);
+          tc::tmem_ld16(base + 2 * TG_N, v2);
+          tc::tmem_ld16(base + 3 * TG_N, v3);
+          tc::tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const int c = col0 + c16 * 16 + j;
+            float2 v = combine_levels(v0[j], v1[j], v2[j], v3[j]);
+            df_norm(v.x, v.y);
+            if (r < P.M && c < P.N) out[c] = v;
+          }
+        }
+      } else {
+        *abort_flag = 1;
       }
-      tc::fence_after_sync();
+      __syncwarp();
+    } else {
+      float ah[TG_N], al[TG_N];
 #pragma unroll
-      for (int c16 = 0; c16 < TG_N / 16; ++c16) {
-        uint32_t v0[16], v1[16], v2[16], v3[16];
-        const uint32_t base =
-            tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * TG_LEV * TG_N + c16 * 16);
-        tc::tmem_ld16(base, v0);
-        tc::tmem_ld16(base + TG_N, v1);
-        tc::tmem_ld16(base + 2 * TG_N, v2);
-        tc::tmem_ld16(base + 3 * TG_N, v3);
-        tc::tmem_wait_ld();
+      for (int c = 0; c < TG_N; ++c) ah[c] = al[c] = 0.f;
+      bool ok = true;
+      for (int seg = 0; seg < nseg; ++seg) {
+        const int b = seg & 1;
+        // one lane polls; the warp then continues converged, as the
+        // .sync.aligned tensor-memory loads and barriers below require
+        int got = 1;
+        if (lane == 0) got = tc::mbar_wait(&tfull[b], (seg >> 1) & 1, abort_flag, WAIT_LIMIT);
+        __syncwarp();
+        got = __shfl_sync(0xffffffffu, got, 0);
+        if (!got) {
+          ok = false;
+          break;
+        }
+        tc::fence_after_sync();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          // exact integers: L0 + L1 2^-8 + L2 2^-16 + L3 2^-24 as a double-float
-          float h = __uint_as_float(v0[j]), l = 0.f;
-          df_add1(h, l, __uint_as_float(v1[j]) * 0x1p-8f);
-          df_add1(h, l, __uint_as_float(v2[j]) * 0x1p-16f);
-          df_add1(h, l, __uint_as_float(v3[j]) * 0x1p-24f);
-          const int c = c16 * 16 + j;
-          df_add1(ah[c], al[c], h);
-          al[c] += l;
-          df_norm(ah[c], al[c]);
+        for (int c16 = 0; c16 < TG_N / 16; ++c16) {
+          uint32_t v0[16], v1[16], v2[16], v3[16];
+          const uint32_t base =
+              tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * TG_LEV * TG_N + c16 * 16);
+          tc::tmem_ld16(base, v0);
+          tc::tmem_ld16(base + TG_N, v1);
+          tc::tmem_ld16(base + 2 * TG_N, v2);
+          tc::tmem_ld16(base + 3 * TG_N, v3);
+          tc::tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float2 v = combine_levels(v0[j], v1[j], v2[j], v3[j]);
+            const int c = c16 * 16 + j;
+            df_add1(ah[c], al[c], v.x);
+            al[c] += v.y;
+            df_norm(ah[c], al[c]);
+          }
+        }
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&tempty[b]);
+      }
+      // stage the 128 x 64 tile in the (now idle) first pipeline stage, then
+      // store it row by row with consecutive threads on consecutive columns
+      float2* tile = reinterpret_cast<float2*>(smem);  // [128][TG_N + 1]
+      if (!ok) {
+        *abort_flag = 1;
+      } else {
+        const int r = 32 * q + lane;
+#pragma unroll
+        for (int c = 0; c < TG_N; ++c) tile[r * (TG_N + 1) + c] = make_float2(ah[c], al[c]);
+      }
+      __syncwarp();
+      asm volatile("bar.sync 1, 128;" ::: "memory");  // the four drain warps, always
+      if (!*abort_flag) {
+        const int t = threadIdx.x - 64;
+        float2* base = P.part + (int64_t)blockIdx.y * P.M * P.N;
+        for (int idx = t; idx < TG_M * TG_N; idx += 128) {
+          const int rr = idx / TG_N, cc = idx % TG_N;
+          if (row0 + rr < P.M && col0 + cc < P.N)
+            base[(int64_t)(row0 + rr) * P.N + col0 + cc] = tile[rr * (TG_N + 1) + cc];
         }
       }
-      tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&tempty[b]);
     }
-    // stage the 128 x 64 tile in the (now idle) first pipeline stage, then
-    // store it row by row with consecutive threads on consecutive columns
-    float2* tile = reinterpret_cast<float2*>(smem);  // [128][TG_N + 1]
-    if (!ok) {
-      *abort_flag = 1;
-    } else {
-      const int r = 32 * q + lane;
-#pragma unroll
-      for (int c = 0; c < TG_N; ++c) tile[r * (TG_N + 1) + c] = make_float2(ah[c], al[c]);
-    }
-    __syncwarp();
-    asm volatile("bar.sync 1, 128;" ::: "memory");  // the four drain warps, always
-    if (!*abort_flag) {
-      const int t = threadIdx.x - 64;
-      float2* base = P.part + (int64_t)blockIdx.y * P.M * P.N;
-      for (int idx = t; idx < TG_M * TG_N; idx += 128) {
-        const int rr = idx / TG_N, cc = idx % TG_N;
-        if (row0 + rr < P.M && col0 + cc < P.N)
-          base[(int64_t)(row0 + rr) * P.N + col0 + cc] = tile[rr * (TG_N + 1) + cc];
-      }
-    }
-    __syncwarp();
   }
   // teardown: TMA copies still in flight (only after an abort) land before
   // the CTA exits; then tensor memory is released
@@ -515,10 +444,10 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
 }
 
 // Split-K partials (double-float) -> FP64, scaled by 2^(e_i + e_j - 14), into
-// C[i][j] and C[j][i] for i <= j (symmetric mode).
+// C[i][j] and C[j][i] for i <= j (symmetric mode).  w (optional): 1 / sqrt(C_ii).
 __global__ void tg_reduce_sym_kernel(const float2* __restrict__ part, int splits, int N,
                                      const int* __restrict__ exps, double* __restrict__ C,
-                                     int64_t ldc) {
+                                     int64_t ldc, double* __restrict__ w) {
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)N * N) return;
   const int i = (int)(idx / N), j = (int)(idx % N);
@@ -529,7 +458,9 @@ __global__ void tg_reduce_sym_kernel(const float2* __restrict__ part, int splits
     df_add1(h, l, v.x);
     l += v.y;
   }
-  const double v = ldexp((double)h + (double)l, exps[i] + exps[j] - 14);
+  const double v =
+      (bits::to_double(h) + bits::to_double(l)) * bits::pow2(exps[i] + exps[j] - 14);
+  if (w && i == j) w[i] = 1.0 / sqrt(v);
   C[(int64_t)i * ldc + j] = v;
   C[(int64_t)j * ldc + i] = v;
 }
@@ -584,7 +515,7 @@ int64_t tg_kpad(int K) { return ((int64_t)K + TG_K - 1) / TG_K * TG_K; }
 // rows in S.  Returns false if the tensor maps cannot be made (the caller
 // then has no tensor-core path); launch errors surface at check_launch.
 bool launch_tcgram_sym(const Ctx& cx, const void* S, int N, int Kpad, int64_t ldo, int64_t plane,
-                       const int* exps, double* C, int64_t ldc) {
+                       const int* exps, double* C, int64_t ldc, double* w) {
   CUtensorMap mA, mB;
   if (!make_slice_map(&mA, S, Kpad, N, ldo, plane, TG_M) ||
       !make_slice_map(&mB, S, Kpad, N, ldo, plane, TG_N))
@@ -618,7 +549,7 @@ bool launch_tcgram_sym(const Ctx& cx, const void* S, int N, int Kpad, int64_t ld
   tcgram_kernel<<<dim3(tiles, splits), TG_THREADS, TG_SMEM, cx.s>>>(mA, mB, P);
   note_launch();
   tg_reduce_sym_kernel<<<(unsigned)((per + 255) / 256), 256, 0, cx.s>>>(P.part, splits, N, exps,
-                                                                       C, ldc);
+                                                                       C, ldc, w);
   return true;
 }
 
@@ -671,20 +602,6 @@ bool launch_tc_var_resid(const Ctx& cx, const float* Xc, int64_t ldc, const doub
   resid_apply_kernel<<<dim3((n_eff + 255) / 256 < 16 ? (n_eff + 255) / 256 : 16, m), 256, 0,
                        cx.s>>>(X, ldx, m, n_eff, p, mu, cst, P.part, aexp, E);
   return true;
-}
-
-void launch_slice_center(const double* E, int64_t lde, const double* mu, int m, int K,
-                         int64_t Kpad, void* S, int64_t plane, int* exps, cudaStream_t s) {
-  note_launch();
-  slice_center_kernel<<<m, 256, 0, s>>>(E, lde, mu, K, (int)Kpad,
-                                         static_cast<__nv_bfloat16*>(S), Kpad, plane, exps);
-}
-
-void launch_slice_lags(const float* Xc, int64_t ldc, int m, int n, int p, int64_t Kpad, void* S,
-                       int64_t plane, int* exps, cudaStream_t s) {
-  note_launch();
-  slice_lags_kernel<<<m, 256, 0, s>>>(Xc, ldc, m, n, p, (int)Kpad,
-                                       static_cast<__nv_bfloat16*>(S), Kpad, plane, exps);
 }
 
 }  // namespace vl

@@ -118,10 +118,13 @@ vl_status fail(vl_handle h, vl_status code, const std::string& msg);
 vl_status check_launch(vl_handle h, const char* what);
 
 // ------------------------------------------------------- kernel launchers
-// Statistics / layout kernels (k_stats.cu)
-template <class T>
-void launch_var_prep(const double* X, int64_t ldx, int m, int n, int p, T* Xc, int64_t ldc,
+// Statistics / layout kernels (k_stats.cu).  var_prep: FP64 path; prep_lags:
+// mixed path, with the slices of the lag windows (see launch_tcgram_sym).
+void launch_var_prep(const double* X, int64_t ldx, int m, int n, int p, double* Xc, int64_t ldc,
                      double* mu, double* wbar, int* st, cudaStream_t s);
+void launch_prep_lags(const double* X, int64_t ldx, int m, int n, int p, float* Xc, int64_t ldc,
+                      double* mu, double* wbar, int64_t Kpad, void* S, int64_t plane, int* exps,
+                      int* st, cudaStream_t s);
 // VAR normal equations from the lagged Gram G (mp x m(p+1), FP64, uncentred
 // in the windows): Gzz = centred Z Z^T (T, mp x mp), Gzy = centred Z Y^T
 // (T, mp x m).
@@ -158,16 +161,20 @@ void launch_refine_apply(float* beta, const float* delta, int m, int p, double* 
                          cudaStream_t s);
 void launch_var_resid_init(const double* X, int64_t ldx, int m, int n, int p, const double* mu,
                            const double* cst, double* E, int64_t lde, cudaStream_t s);
-template <class T>
+// FP64 path: mean, 1/std and entropy hx of every row (hx NULL: the first two).
 void launch_standardize(const double* E, int64_t lde, int m, int n, double* mu, double* inv_sd,
-                        double* hx_mom, int* st, cudaStream_t s);
-void launch_split_center(const double* E, int64_t lde, int m, int n, const double* mu,
-                         float* hi, float* lo, int64_t ldc, cudaStream_t s);
+                        double* hx, int* st, cudaStream_t s);
+// Mixed path: entropies hx, the slices of the centred rows (S, exps) and the
+// standardized time-major samples xt (n_pad x m_pad); xs: scratch of m x n_pad
+// floats if measure_prep_needs_rows.  xt NULL: the slices only.
+bool measure_prep_needs_rows(int m, int n);
+void launch_measure_prep(const double* E, int64_t lde, int m, int n, int64_t Kpad, void* S,
+                         int64_t plane, int* exps, float* xs, float* xt, int m_pad, int n_pad,
+                         double* hx, int* st, cudaStream_t s);
 void launch_center64(const double* E, int64_t lde, int m, int n, const double* mu, double* out,
                      int64_t ldc, cudaStream_t s);
-template <class T>
 void launch_transpose_std(const double* E, int64_t lde, int m, int n, const double* mu,
-                          const double* inv_sd, T* xt, int m_pad, int n_pad, cudaStream_t s);
+                          const double* inv_sd, double* xt, int m_pad, int n_pad, cudaStream_t s);
 
 // Dense linear algebra (k_linalg.cu).  A "view" addresses element (r, k) at
 // base[r * rs + k * ks].  gemm computes C[r, c] = alpha * sum_k A(r,k) B(c,k)
@@ -226,10 +233,12 @@ PairPlan plan_pairwise(int m, int n, int num_sms, bool fp64);
 // FP32 plan with sample splits of about split_len samples (batched launches,
 // where many instances fill the GPU together)
 PairPlan plan_pairwise_split(int m, int n, int split_len);
-// rho and kappa / sqrt(1 - rho^2) (kappa = 2 log2 e) as FP32 (rho32, c32) or
-// FP64 (rho64, c64) m x m arrays; the other two are NULL
-void launch_pair_consts(const double* C, int m, float* rho32, float* c32, double* rho64,
-                        double* c64, int* st, cudaStream_t s);
+// rho and kappa / sqrt(1 - rho^2) (kappa = 2 log2 e) for i < j from the cross
+// products C, as FP32 (w: 1 / sqrt(C_ii)) or FP64 m x m arrays
+void launch_pair_consts(const double* C, const double* w, int m, float* rho32, float* c32,
+                        int* st, cudaStream_t s);
+void launch_pair_consts64(const double* C, int m, double* rho64, double* c64, int* st,
+                          cudaStream_t s);
 void launch_pairwise_f32(const float* xt, const PairPlan& pl, const float* rho32,
                          const float* c32, float* part, cudaStream_t s);
 void launch_pairwise_f64(const double* xt, const PairPlan& pl, const double* rho64,
@@ -247,8 +256,9 @@ PairJob make_pair_job(const float* xt, const PairPlan& pl, const float* rho32, c
 // items: (job, tile, split, 0), largest first; grid: CTAs (about one per SM)
 void launch_pairwise_f32_list(const PairJob* jobs, const int4* items, int nitems, int grid,
                               cudaStream_t s);
-void launch_measure_finalize(const void* part, const PairPlan& pl, const double* hx_mom,
-                             double* Hx, double* Hr, double* D, bool fp32_parts, cudaStream_t s);
+// hx: the variables' entropies
+void launch_measure_finalize(const void* part, const PairPlan& pl, const double* hx, double* Hx,
+                             double* Hr, double* D, bool fp32_parts, cudaStream_t s);
 
 // Ordering (k_order.cu).  Its workspace: P^T as double-float pairs (pt),
 // the initial row sums (sh, sl) and the gap scratch (s1, s2).
@@ -270,17 +280,14 @@ void launch_causal_order(const double* D, int m, void* ws, int32_t* order, doubl
 // Tensor-core exact-slice Gram products (k_tcgram.cu).  Operands are three
 // bf16 slice planes S[z][r][k] (k < Kpad = tg_kpad(K), a multiple of 64; row
 // stride Kpad, plane stride `plane` elements) with a power-of-two exponent
-// per row.  slice_center: rows E[r] - mu[r] (FP64); slice_lags: the lag
-// windows of the centred FP32 series Xc, row b m + k = Xc[k][p - b + t].
+// per row, made by launch_measure_prep (centred rows of E) and launch_prep_lags
+// (the lag windows of the centred series, row b m + k = Xc[k][p - b + t]).
 // launch_tcgram_sym: C = (S S^T) scaled back, N x N FP64 symmetric, using
-// the context's split-K scratch; false if the tensor maps cannot be made.
+// the context's split-K scratch, and w_i = 1 / sqrt(C_ii) if w is given; false if
+// the tensor maps cannot be made.
 int64_t tg_kpad(int K);
-void launch_slice_center(const double* E, int64_t lde, const double* mu, int m, int K,
-                         int64_t Kpad, void* S, int64_t plane, int* exps, cudaStream_t s);
-void launch_slice_lags(const float* Xc, int64_t ldc, int m, int n, int p, int64_t Kpad, void* S,
-                       int64_t plane, int* exps, cudaStream_t s);
 bool launch_tcgram_sym(const Ctx& cx, const void* S, int N, int Kpad, int64_t ldo, int64_t plane,
-                       const int* exps, double* C, int64_t ldc);
+                       const int* exps, double* C, int64_t ldc, double* w = nullptr);
 // The VAR residuals E = X[:, p:] - mu - cst - sum_tau M_tau Z_tau as one
 // tensor-core product (beta: FP32 mp x m; vexp: the variables' slice
 // exponents of launch_slice_lags); false if the tensor maps cannot be made or

@@ -73,6 +73,28 @@ def test_fit_b_at_the_edges_of_the_factorisations(vl, h, prec, m):
     assert np.abs(B0.cpu().numpy() - ref).max() <= (1e-4 if prec == "mixed" else 1e-10)
 
 
+# tiles of the finalisation (7, 8, 9 variables); one and two exact segments of
+# the tensor-core product (256 and 257 samples); standardized samples written in
+# place and transposed (m n on either side of 2^19).  Variables 0 and 1 are nearly
+# collinear (1 - rho^2 about 2.5e-3, where the pair constants take the FP64 form).
+@pytest.mark.parametrize("m,n", [(7, 256), (8, 257), (9, 1000), (33, 15887), (33, 15889)])
+def test_mixed_measure_at_the_edges_of_its_kernels(vl, h, m, n):
+    rng = np.random.default_rng(m + n)
+    E = rng.laplace(size=(m, n))
+    E[2:] += 0.3 * E[:-2]
+    E[1] = E[0] + 0.05 * rng.laplace(size=n)
+    Hx, Hr, D = _f64(m), _f64(m, m), _f64(m, m)
+    vl.vl_pairwise_measure(h, torch.from_numpy(E).cuda(), "mixed", Hx, Hr, D)
+    h.sync()
+    ref = oracle.pairwise_measure(oracle.standardize(E))
+    off = ~np.eye(m, dtype=bool)
+    want = np.where(off, ref["Er"], 0.0)
+    # the suite's bounds for the mixed path: 1e-5 of the entropy scale and of max |D|
+    assert np.abs(Hx.cpu().numpy() - ref["Ex"]).max() <= 1e-5 * max(1.42, np.abs(ref["Ex"]).max())
+    assert np.abs(Hr.cpu().numpy() - want).max() <= 1e-5 * max(1.42, np.abs(want).max())
+    assert np.abs(D.cpu().numpy() - ref["D"]).max() <= 1e-5 * np.abs(ref["D"]).max()
+
+
 def _order_fp64(D):
     """Algorithm 1 with running FP64 sums: the order, each step's relative gap, and
     how far that gap may be off: the sums start from pairs of 48 bits and take m
