@@ -16,8 +16,8 @@
 // All of them are bound by the number of FP64 instructions (1.6 per clock per SM,
 // conversions included): a row is read in as few passes as its statistics allow,
 // scalar divisions and roots are taken by one thread, conversions run on the
-// integer pipe.  m = 400, n = 2500: prep_lags 24 us (28 + 11 as two kernels with
-// a pass per window), measure_prep 35 us (33 + 19 as two).
+// integer pipe.  m = 400, n = 2500: prep_lags 26 us (28 + 11 as two kernels with a
+// pass per window), measure_prep 33 us (33 + 19 as two).
 #include <cmath>
 
 #include "fp64_bits.cuh"
@@ -31,48 +31,104 @@ namespace {
 
 constexpr int kStatMax = 256;  // threads of a row's CTA
 
-// Row i of X: its mean, the sums of its lag windows and a pass over the centred
+// Sum over t < kStatMax of val(t), by one warp, in block_sum's order; in all lanes.
+// Each level adds only the pairs that go on: two registers' halves change places
+// in the shuffle, so that 4, 2, then 1 register hold them.
+template <class Val>
+__device__ __forceinline__ double warp_tree(Val val) {
+  static_assert(kStatMax == 256, "eight warps' trees");
+  const int lane = threadIdx.x & 31;
+  double a[4];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    const int i = g * 32 + lane, t = (i >> 4) * 32 + (i & 15);
+    a[g] = val(t) + val(t + 16);
+  }
+  auto fold = [lane](double u, double v, int o) {
+    return ((lane & o) ? v : u) + __shfl_xor_sync(0xffffffffu, (lane & o) ? u : v, o);
+  };
+  double c = fold(fold(a[0], a[1], 8), fold(a[2], a[3], 8), 4);
+  // within a warp's sum 2 and 1, then between the warps (their index's bits 2, 1, 0
+  // are the lane's bits 2, 3, 4)
+#pragma unroll
+  for (int o : {2, 1, 4, 8, 16}) c += __shfl_xor_sync(0xffffffffu, c, o);
+  return c;
+}
+
+// Row i of X: its mean, the means of its lag windows and a pass over the centred
 // values: each(t, x_t - mean) for every t < n in the thread's order.
+// Window s = p - b is [s, s + n - p), its sum taken over threads that each add
+// every 256th sample from s + thread on, and then a tree.  (The order is fixed: an
+// ulp of a window mean flips the last bits of the normal equations and with them
+// FP32 roundings of the fitted lag matrices.)  Those samples are the ones that
+// thread + s adds in window 0, and at most one more at the end, so one pass serves
+// every window: w, the thread's samples below n - p; w1, the same without the
+// first, which stands for thread + s >= 256; the sample at the end apart.  m = 203,
+// n = 4001, p = 3: 3 FP64 instructions a sample for 9 with a pass per window, the
+// VAR fit 912 us for 930.
 template <class Each>
 __device__ __forceinline__ void centre_row(const double* __restrict__ x, int m, int n, int p,
-                                           double inv_n, double* red, double* __restrict__ mu_out,
+                                           double inv_n, double inv_eff, double* red,
+                                           double* __restrict__ mu_out,
                                            double* __restrict__ wbar, int* st, Each each) {
-  const int i = blockIdx.x;
+  const int i = blockIdx.x, tid = threadIdx.x;
   double s = 0.0;
   bool finite = true;
 #pragma unroll 4
-  for (int t = threadIdx.x; t < n; t += kStatMax) {
+  for (int t = tid; t < n; t += kStatMax) {
     const double v = x[t];
     finite &= is_finite(v);
     s += v;
   }
-  if (__syncthreads_or(!finite) && threadIdx.x == 0) set_status(st, VL_ERR_NONFINITE);
-  const double mu = block_sum(s, red, [inv_n](double t) { return t * inv_n; });
-  if (threadIdx.x == 0) mu_out[i] = mu;
-  double w = 0.0;
+  if (__syncthreads_or(!finite) && tid == 0) set_status(st, VL_ERR_NONFINITE);
+  const double mu = block_sum(s, red, [n, inv_n](double t) { return div_by(t, n, inv_n); });
+  if (tid == 0) mu_out[i] = mu;
+  const int n_eff = n - p;
+  __shared__ double w0s[kStatMax], w1s[kStatMax], ends[kStatMax];
+  double w = 0.0, w1 = 0.0, end = 0.0;
 #pragma unroll 4
-  for (int t = threadIdx.x; t < n; t += kStatMax) {
+  for (int t = tid; t < n; t += kStatMax) {
     const double d = x[t] - mu;
-    w += d;
+    if (t < n_eff) {
+      w += d;
+      if (tid < p && t != tid) w1 += d;
+    } else {
+      end = d;
+    }
     each(t, d);
   }
-  w = block_sum(w, red);
-  // window b = [p - b, n - b): the whole sum without its ends
-  for (int b = threadIdx.x; b <= p; b += blockDim.x) {
-    double e = 0.0;
-    for (int t = 0; t < p - b; ++t) e += x[t] - mu;
-    for (int t = n - b; t < n; ++t) e += x[t] - mu;
-    wbar[(int64_t)b * m + i] = (w - e) / (n - p);
+  w0s[tid] = w;
+  w1s[tid] = w1;
+  ends[tid] = end;
+  __syncthreads();
+  if (p < kStatMax) {
+    for (int sh = tid >> 5; sh <= p; sh += kStatMax / 32) {  // a warp per window
+      const double sum = warp_tree([&](int t) {
+        const int j = (t + sh) & (kStatMax - 1);
+        const int e = j + (n_eff - j + kStatMax - 1) / kStatMax * kStatMax;  // first >= n_eff
+        double v = t + sh < kStatMax ? w0s[j] : w1s[j];
+        if (e < n_eff + sh) v += ends[j];
+        return v;
+      });
+      if ((tid & 31) == 0) wbar[(int64_t)(p - sh) * m + i] = div_by(sum, n_eff, inv_eff);
+    }
+    return;
+  }
+  for (int b = 0; b <= p; ++b) {
+    w = 0.0;
+    for (int t = tid; t < n_eff; t += kStatMax) w += x[p - b + t] - mu;
+    w = block_sum(w, red);
+    if (tid == 0) wbar[(int64_t)b * m + i] = div_by(w, n_eff, inv_eff);
   }
 }
 
 __global__ void __launch_bounds__(kStatMax)
     var_prep_kernel(const double* __restrict__ X, int64_t ldx, int m, int n, int p, double inv_n,
-                    double* __restrict__ Xc, int64_t ldc, double* __restrict__ mu_out,
-                    double* __restrict__ wbar, int* st) {
+                    double inv_eff, double* __restrict__ Xc, int64_t ldc,
+                    double* __restrict__ mu_out, double* __restrict__ wbar, int* st) {
   __shared__ double red[2 * kStatMax];
   double* xc = Xc + blockIdx.x * ldc;
-  centre_row(X + blockIdx.x * ldx, m, n, p, inv_n, red, mu_out, wbar, st,
+  centre_row(X + blockIdx.x * ldx, m, n, p, inv_n, inv_eff, red, mu_out, wbar, st,
              [xc](int t, double d) { xc[t] = d; });
   for (int t = n + threadIdx.x; t < ldc; t += blockDim.x) xc[t] = 0.0;
 }
@@ -84,15 +140,16 @@ __global__ void __launch_bounds__(kStatMax)
 // of its windows, and each sample sliced once for all of them.
 __global__ void __launch_bounds__(kStatMax)
     prep_lags_kernel(const double* __restrict__ X, int64_t ldx, int m, int n, int p, double inv_n,
-                     float* __restrict__ Xc, int64_t ldc, double* __restrict__ mu_out,
-                     double* __restrict__ wbar, int Kpad, __nv_bfloat16* __restrict__ S,
-                     int64_t ldo, int64_t plane, int* __restrict__ exps, int* st) {
+                     double inv_eff, float* __restrict__ Xc, int64_t ldc,
+                     double* __restrict__ mu_out, double* __restrict__ wbar, int Kpad,
+                     __nv_bfloat16* __restrict__ S, int64_t ldo, int64_t plane,
+                     int* __restrict__ exps, int* st) {
   __shared__ double red[2 * kStatMax];
   __shared__ unsigned long long redu[32];
   const int k = blockIdx.x, n_eff = n - p;
   float* xc = Xc + k * ldc;
   uint32_t mx = 0;
-  centre_row(X + k * ldx, m, n, p, inv_n, red, mu_out, wbar, st, [&](int t, double d) {
+  centre_row(X + k * ldx, m, n, p, inv_n, inv_eff, red, mu_out, wbar, st, [&](int t, double d) {
     const float f = bits::to_float(d);
     mx = max(mx, __float_as_uint(f) & 0x7fffffffu);
     xc[t] = f;
@@ -222,7 +279,7 @@ __device__ __forceinline__ void row_stats(const double* __restrict__ e, int n, d
     s += v;
   }
   if (__syncthreads_or(!finite) && threadIdx.x == 0) set_status(st, VL_ERR_NONFINITE);
-  mu = block_sum(s, red, [inv_n](double t) { return t * inv_n; });
+  mu = block_fold(s, red, [inv_n](double t) { return t * inv_n; });
   double q = 0.0;
 #pragma unroll 4
   for (int t = threadIdx.x; t < n; t += kStatMax) {
@@ -230,7 +287,7 @@ __device__ __forceinline__ void row_stats(const double* __restrict__ e, int n, d
     q += d * d;
     each(d);
   }
-  isd = block_sum(q, red, [inv_n, st](double t) {
+  isd = block_fold(q, red, [inv_n, st](double t) {
     const double var = t * inv_n;
     if (var > 1e-300 || var != var) return rsqrt(var);
     set_status(st, VL_ERR_DEGENERATE);
@@ -393,14 +450,14 @@ __global__ void transpose_f32_kernel(const float* __restrict__ xs, int m, int n_
 void launch_var_prep(const double* X, int64_t ldx, int m, int n, int p, double* Xc, int64_t ldc,
                      double* mu, double* wbar, int* st, cudaStream_t s) {
   note_launch();
-  var_prep_kernel<<<m, kStatMax, 0, s>>>(X, ldx, m, n, p, 1.0 / n, Xc, ldc, mu, wbar, st);
+  var_prep_kernel<<<m, kStatMax, 0, s>>>(X, ldx, m, n, p, 1.0 / n, 1.0 / (n - p), Xc, ldc, mu, wbar, st);
 }
 
 void launch_prep_lags(const double* X, int64_t ldx, int m, int n, int p, float* Xc, int64_t ldc,
                       double* mu, double* wbar, int64_t Kpad, void* S, int64_t plane, int* exps,
                       int* st, cudaStream_t s) {
   note_launch();
-  prep_lags_kernel<<<m, kStatMax, 0, s>>>(X, ldx, m, n, p, 1.0 / n, Xc, ldc, mu, wbar, (int)Kpad,
+  prep_lags_kernel<<<m, kStatMax, 0, s>>>(X, ldx, m, n, p, 1.0 / n, 1.0 / (n - p), Xc, ldc, mu, wbar, (int)Kpad,
                                               static_cast<__nv_bfloat16*>(S), Kpad, plane, exps,
                                               st);
 }

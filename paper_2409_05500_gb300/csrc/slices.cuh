@@ -49,13 +49,17 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v
   return red[0];
 }
 
-// Sums over the block (a multiple of 64 threads) in FP64, in every thread.  An
-// FP64 instruction keeps a scheduler's FP64 unit for 64 clocks, so it is their
-// number that counts: the block folds through shared memory (each fold halves the
-// warps that add) down to one warp, whose last five steps are shuffles.  block_sum2:
-// two sums, the second's last warp beside the first's.  red: blockDim.x doubles
-// (twice that for two sums).  f is applied to the sum by one thread (a division
-// or root there costs one warp 600 to 1,000 clocks, not every warp).
+// Sums over the block (64 to 256 threads, a power of two) in FP64, in every
+// thread.  An FP64 instruction keeps a scheduler's FP64 unit for 64 clocks, so it
+// is their number that counts.  block_sum adds in the order of a shuffle tree in
+// each warp and one over the warps' sums, of which only the sums that go on are
+// formed: three levels folded through shared memory, the rest by the first warp.
+// (Where a mean decides how a sample rounds to FP32, its order stays fixed: an ulp
+// of it moves a coefficient by an ulp of FP32 now and then.)  block_fold and
+// block_sum2 (two sums, the second's last warp beside the first's) halve the block
+// instead, 0.5 us a sum faster.  red: 2 blockDim.x doubles.  f is applied to the
+// sum by one thread (a division or root there costs one warp 600 to 1,000 clocks,
+// not every warp).
 __device__ __forceinline__ double warp_sum_f64(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -63,6 +67,28 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
 }
 template <class F>
 __device__ __forceinline__ double block_sum(double v, double* red, F f) {
+  const int tid = threadIdx.x, n = blockDim.x;
+  double* r2 = red + n;
+  __syncthreads();
+  red[tid] = v;
+  __syncthreads();
+  // value (w, l) at w 2h + l: (w, l) + (w, l + h) goes to w h + l
+  if (tid < n / 2) r2[tid] = red[2 * tid - (tid & 15)] + red[2 * tid - (tid & 15) + 16];
+  __syncthreads();
+  if (tid < n / 4) red[tid] = r2[2 * tid - (tid & 7)] + r2[2 * tid - (tid & 7) + 8];
+  __syncthreads();
+  if (tid < 32) {
+    v = tid < n / 8 ? red[2 * tid - (tid & 3)] + red[2 * tid - (tid & 3) + 4] : 0.0;
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    for (int o = 16; o >= 4; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (tid == 0) r2[0] = f(v);
+  }
+  __syncthreads();
+  return r2[0];
+}
+template <class F>
+__device__ __forceinline__ double block_fold(double v, double* red, F f) {
   const int tid = threadIdx.x;
   __syncthreads();
   red[tid] = v;
@@ -77,6 +103,13 @@ __device__ __forceinline__ double block_sum(double v, double* red, F f) {
   }
   __syncthreads();
   return red[0];
+}
+// t / n, correctly rounded, from inv = 1 / n correctly rounded (Markstein 1990: a
+// quotient within an ulp, its exact remainder, one correction): three instructions
+// inline for a call into the division of 600 clocks and its instruction fetches.
+__device__ __forceinline__ double div_by(double t, int n, double inv) {
+  const double q = t * inv;
+  return fma(fma(-q, (double)n, t), inv, q);
 }
 __device__ __forceinline__ double block_sum(double v, double* red) {
   return block_sum(v, red, [](double t) { return t; });

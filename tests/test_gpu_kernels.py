@@ -140,3 +140,29 @@ def test_order_at_the_edges_of_its_searches(vl, h, m):
     assert np.array_equal(np.isinf(got), np.isinf(want_gap))
     fin = np.isfinite(want_gap)
     assert np.all(np.abs(got[fin] - want_gap[fin]) <= 1e-9 + slack[fin])
+
+
+# lag windows: fewer samples than a block has threads, one more, ends of windows
+# that fall to the first threads again, more lags than a warp and than a block.  A
+# trend makes every window's mean a different one.  Tolerances: FP64 normal
+# equations of condition up to 2e3, n 2.2e-16 each: 6.6e-10, taken as 1e-9; mixed
+# 1e-5 (FP32 rounding of the series, 6e-8, by a condition of up to 160).
+@pytest.mark.parametrize("m,n,p", [(3, 199, 1), (3, 256, 1), (3, 257, 2), (2, 259, 3),
+                                   (2, 300, 40), (2, 513, 60), (2, 1500, 255), (2, 1500, 256)])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_var_fit_with_different_window_means(vl, h, prec, m, n, p):
+    if prec == "mixed" and p > 60:
+        pytest.skip("condition beyond the tolerance's")
+    rng = np.random.default_rng(n + p)
+    X = rng.laplace(size=(m, n))
+    for t in range(1, n):
+        X[:, t] += 0.5 * X[:, t - 1]
+    X += np.linspace(2.0, 5.0, n)
+    M = _f64(p, m, m)
+    vl.vl_var_fit(h, torch.from_numpy(X).cuda(), p, prec, M, None)
+    h.sync()
+    Z = np.vstack([np.ones(n - p)] + [X[:, p - b:n - b] for b in range(1, p + 1)]).T
+    beta = np.linalg.lstsq(Z, X[:, p:].T, rcond=None)[0][1:]
+    want = beta.reshape(p, m, m).transpose(0, 2, 1)
+    tol = 1e-9 if prec == "fp64" else 1e-5
+    assert np.abs(M.cpu().numpy() - want).max() <= tol
