@@ -70,7 +70,7 @@ struct DeviceGuard {
 // handle's own; a batch gives every stream of its pool one of these.
 struct Exec {
   vl_handle h;
-  cudaStream_t s;
+  Lane s;
   int* st;
   void** ws;       // workspace pointer owned by the handle
   size_t* ws_cap;  // and its capacity
@@ -175,7 +175,7 @@ vl_status var_fit_impl(Exec& x, const double* X, int64_t ldx, int m, int n, int 
   if (s != VL_OK || x.measure) return s;
   if (!E) E = Ew;
   Ctx cx = make_ctx(x, part, part_cap);
-  cudaStream_t st = x.s;
+  Lane st = x.s;
   if constexpr (sizeof(T) == 4) {
     // W W^T on the tensor cores: the lag windows sliced once, the symmetric
     // q x q product; its rows m.. (the Z rows) are G
@@ -243,7 +243,7 @@ struct CovOut {
 template <class T>
 vl_status cov_and_stats(const Ctx& cx, const double* E, int64_t lde, int m, int n,
                         const CovOut& o, void* scratch) {
-  cudaStream_t st = cx.s;
+  Lane st = cx.s;
   if constexpr (sizeof(T) == 4) {
     const int64_t kp = tg_kpad(n), plane = (int64_t)m * kp;
     char* S = static_cast<char*>(scratch);
@@ -313,7 +313,7 @@ vl_status pairwise_impl(Exec& x, const double* E, int64_t lde, int m, int n, dou
   if (!D) D = D_w;
   vl_handle h = x.h;
   Ctx cx = make_ctx(x, gpart, part_cap);
-  cudaStream_t st = x.s;
+  Lane st = x.s;
   if constexpr (sizeof(T) == 4) {
     o.xt = xt;
     o.m_pad = pl.m_pad;
@@ -368,7 +368,7 @@ vl_status fit_b_impl(Exec& x, const double* E, int64_t lde, int m, int n,
   });
   if (s != VL_OK || x.measure) return s;
   Ctx cx = make_ctx(x, gpart, part_cap);
-  cudaStream_t st = x.s;
+  Lane st = x.s;
   const double* C = C_in;
   if (!C) {
     if (cov_and_stats<T>(cx, E, lde, m, n, o, scratch) != VL_OK)
@@ -748,7 +748,7 @@ vl_status batched_mixed(vl_handle h, const vl_instance* inst, const std::vector<
   fork();
   for (size_t j = 0; j < idx.size(); ++j) {
     PoolSlot& ps = h->pool[j % S];
-    Exec x{h, ps.stream, dstat + idx[j], &ps.ws, &ps.ws_cap, false, 0};
+    Exec x{h, Lane(ps.stream, false), dstat + idx[j], &ps.ws, &ps.ws_cap, false, 0};
     s = batch_prep(x, inst[idx[j]], B[j]);
     if (s != VL_OK) break;
   }
@@ -792,7 +792,7 @@ vl_status batched_mixed(vl_handle h, const vl_instance* inst, const std::vector<
   fork();
   for (size_t j = 0; j < idx.size(); ++j) {
     PoolSlot& ps = h->pool[j % S];
-    Exec x{h, ps.stream, dstat + idx[j], &ps.ws, &ps.ws_cap, false, 0};
+    Exec x{h, Lane(ps.stream, false), dstat + idx[j], &ps.ws, &ps.ws_cap, false, 0};
     s = batch_finish(x, inst[idx[j]], B[j], certified);
     if (s != VL_OK) break;
   }
@@ -909,7 +909,7 @@ vl_status batched_impl(vl_handle h, const vl_instance* inst, int count, vl_preci
       const int k = idx[t];
       PoolSlot& ps = h->pool[t % S];
       const vl_instance& I = inst[k];
-      Exec x{h, ps.stream, h->bstatus + k, &ps.ws, &ps.ws_cap, false, 0};
+      Exec x{h, Lane(ps.stream, false), h->bstatus + k, &ps.ws, &ps.ws_cap, false, 0};
       double* E = static_cast<double*>(ps.buf);
       double* C = E + (size_t)I.m * (I.n - I.p);
       double* D = I.D ? I.D : C + (size_t)I.m * I.m;

@@ -39,6 +39,7 @@ __device__ __forceinline__ unsigned long long splitmix64_mix(unsigned long long 
 __global__ void __launch_bounds__(kBootThreads) boot_resample_kernel(
     const double* __restrict__ X, int64_t ldx, int m, int n, int block_len,
     unsigned long long seed, long long b0, double* __restrict__ out) {
+  pdl_begin(X, out);
   const int t = blockIdx.x * kBootThreads + threadIdx.x;
   if (t >= n) return;
   const unsigned long long b = (unsigned long long)(b0 + blockIdx.z);
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(kBootThreads) boot_resample_kernel(
 // sets VL_ERR_ARG and is skipped.
 __global__ void boot_inverse_kernel(const int32_t* __restrict__ order, int m,
                                     int32_t* __restrict__ pos, int* st) {
+  pdl_begin(order, pos, st);
   const int32_t* o = order + (int64_t)blockIdx.x * m;
   int32_t* q = pos + (int64_t)blockIdx.x * m;
   for (int k = threadIdx.x; k < m; k += blockDim.x) {
@@ -72,6 +74,7 @@ __global__ void boot_inverse_kernel(const int32_t* __restrict__ order, int m,
 __global__ void __launch_bounds__(kBootThreads) boot_count_kernel(
     const double* __restrict__ B0, const int32_t* __restrict__ pos, int m, int nb,
     double threshold, double* __restrict__ edge, double* __restrict__ before) {
+  pdl_begin(B0, pos, edge, before);
   const int64_t mm = (int64_t)m * m;
   const int64_t e = (int64_t)blockIdx.x * kBootThreads + threadIdx.x;
   if (e >= mm) return;
@@ -87,6 +90,7 @@ __global__ void __launch_bounds__(kBootThreads) boot_count_kernel(
 
 __global__ void boot_normalize_kernel(double* __restrict__ edge, double* __restrict__ before,
                                       int64_t mm, double count) {
+  pdl_begin(edge, before);
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < mm;
        e += (int64_t)gridDim.x * blockDim.x) {
     edge[e] = edge[e] / count;
@@ -98,32 +102,28 @@ __global__ void boot_normalize_kernel(double* __restrict__ edge, double* __restr
 
 void launch_boot_resample(const double* X, int64_t ldx, int m, int n, int block_len,
                           unsigned long long seed, long long b0, int nb, double* out,
-                          cudaStream_t s) {
+                          Lane s) {
   constexpr int kMaxZ = 65535;  // grid.z limit
   for (int z0 = 0; z0 < nb; z0 += kMaxZ) {
-    note_launch();
     dim3 grid((n + kBootThreads - 1) / kBootThreads, (m + kBootRows - 1) / kBootRows,
               std::min(kMaxZ, nb - z0));
-    boot_resample_kernel<<<grid, kBootThreads, 0, s>>>(X, ldx, m, n, block_len, seed, b0 + z0,
-                                                       out + (int64_t)z0 * m * n);
+    launch(boot_resample_kernel, grid, kBootThreads, 0, s, X, ldx, m, n, block_len, seed, b0 + z0,
+           out + (int64_t)z0 * m * n);
   }
 }
 
 void launch_boot_count(const int32_t* order, const double* B0, int m, int nb, double threshold,
-                       int32_t* pos, double* edge, double* before, int* st, cudaStream_t s) {
-  note_launch();
-  boot_inverse_kernel<<<nb, 256, 0, s>>>(order, m, pos, st);
-  note_launch();
+                       int32_t* pos, double* edge, double* before, int* st, Lane s) {
+  launch(boot_inverse_kernel, nb, 256, 0, s, order, m, pos, st);
   const int64_t mm = (int64_t)m * m;
-  boot_count_kernel<<<(unsigned)((mm + kBootThreads - 1) / kBootThreads), kBootThreads, 0, s>>>(
-      B0, pos, m, nb, threshold, edge, before);
+  launch(boot_count_kernel, (unsigned)((mm + kBootThreads - 1) / kBootThreads), kBootThreads, 0, s,
+         B0, pos, m, nb, threshold, edge, before);
 }
 
-void launch_boot_normalize(double* edge, double* before, int m, int count, cudaStream_t s) {
-  note_launch();
+void launch_boot_normalize(double* edge, double* before, int m, int count, Lane s) {
   const int64_t mm = (int64_t)m * m;
   const int blocks = (int)std::min<int64_t>((mm + 255) / 256, 4096);
-  boot_normalize_kernel<<<blocks, 256, 0, s>>>(edge, before, mm, (double)count);
+  launch(boot_normalize_kernel, blocks, 256, 0, s, edge, before, mm, (double)count);
 }
 
 }  // namespace vl

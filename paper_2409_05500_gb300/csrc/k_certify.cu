@@ -81,6 +81,7 @@ __device__ __forceinline__ double block_sum_d(double v, double* red) {
 // and the control words of round 0.
 __global__ void cert_init_kernel(const double* __restrict__ D, int m, int* ctrl,
                                  unsigned long long* dmax_bits) {
+  pdl_begin(D, ctrl, dmax_bits);
   __shared__ double red[32];
   double v = 0.0;
   const int64_t tot = (int64_t)m * m;
@@ -114,6 +115,7 @@ __global__ void cert_round_kernel(const int32_t* __restrict__ order, int m, int 
                                   int* __restrict__ ccount, const float2* __restrict__ spick,
                                   const unsigned long long* __restrict__ dmax_bits,
                                   float* __restrict__ thr) {
+  pdl_begin(order, ctrl, pos, flag, ccount, spick, dmax_bits, thr);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < m) {
     pos[order[t]] = t;
@@ -165,6 +167,7 @@ __global__ void __launch_bounds__(32)
                      const float* __restrict__ thr, int m, int* ctrl,
                      const unsigned long long* __restrict__ dmax_bits, int* __restrict__ flag,
                      int* __restrict__ ccount, int* __restrict__ cand) {
+  pdl_begin(pt, sh0, sl0, order, pos, thr, ctrl, dmax_bits, flag, ccount, cand);
   extern __shared__ int ord_s[];  // m order entries, then m thresholds
   float* thr_s = reinterpret_cast<float*>(ord_s + m);
   if (!ctrl[C_ACTIVE]) return;
@@ -227,6 +230,7 @@ __global__ void __launch_bounds__(RTH)
                      const int* __restrict__ cand, unsigned* __restrict__ need,
                      const unsigned* __restrict__ done, int2* __restrict__ pairs,
                      int* __restrict__ stats) {
+  pdl_begin(D, order, pos, ctrl, dmax_bits, flag, ccount, cand, need, done, pairs, stats);
   const int k = blockIdx.x;
   const double pos_thr = CERT_POS * __longlong_as_double((long long)*dmax_bits);
   if (!ctrl[C_ACTIVE] || k < ctrl[C_K0] || !flag[k]) return;
@@ -271,6 +275,7 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 __global__ void __launch_bounds__(RTH)
     cert_stats_kernel(const double* __restrict__ E, int64_t lde, int m, int n, const int* ctrl,
                       float2* __restrict__ xs, double* __restrict__ hx) {
+  pdl_begin(E, ctrl, xs, hx);
   __shared__ double red[32];
   __shared__ float2 tab[32];
   if (!ctrl[C_ACTIVE] || !ctrl[C_ANY] || ctrl[C_HXREADY]) return;
@@ -309,6 +314,7 @@ __global__ void __launch_bounds__(RTH)
                       const double* __restrict__ hx, const int2* __restrict__ pairs,
                       double* __restrict__ D64, unsigned* __restrict__ done,
                       int* __restrict__ stats) {
+  pdl_begin(xs, ctrl, hx, pairs, D64, done, stats);
   __shared__ float2 tab[32];
   if (!ctrl[C_ACTIVE] || !ctrl[C_ANY]) return;
   if (threadIdx.x < 32) tab[threadIdx.x] = df::kExp2Frac[threadIdx.x];
@@ -364,6 +370,7 @@ __global__ void __launch_bounds__(RTH)
                        int* ctrl, const int* __restrict__ flag, const int* __restrict__ ccount,
                        const int* __restrict__ cand, const double* __restrict__ D64,
                        const unsigned* __restrict__ done, int* __restrict__ pick) {
+  pdl_begin(order, pos, ctrl, flag, ccount, cand, D64, done, pick);
   __shared__ double red[32];
   __shared__ double sc[CMAX + 1];
   const int k = blockIdx.x;
@@ -411,6 +418,7 @@ __global__ void __launch_bounds__(STH)
                        const float* __restrict__ sl0, int m, int32_t* __restrict__ order,
                        const int* __restrict__ pos, const int* __restrict__ pick,
                        const int* ctrl, float2* __restrict__ spick, int* __restrict__ stats) {
+  pdl_begin(pt, sh0, sl0, order, pos, pick, ctrl, spick, stats);
   if (!ctrl[C_ACTIVE]) return;
   const int ks = ctrl[C_FIRST];
   if (ks >= m) return;
@@ -447,6 +455,7 @@ __global__ void __launch_bounds__(STH)
 
 // Steps after a pick changed in the last round were not verified again.
 __global__ void cert_tail_kernel(int m, const int* ctrl, int* stats) {
+  pdl_begin(ctrl, stats);
   if (ctrl[C_ACTIVE] && ctrl[C_FIRST] < m) atomicAdd(&stats[3], 1);
 }
 
@@ -506,46 +515,36 @@ float2* certify_spick(void* cert_ws, int m) { return cert_layout(cert_ws, m, 0).
 
 void launch_certify(const double* D, const double* E, int64_t lde, int m, int n, void* order_ws,
                     void* cert_ws, int32_t* order, int32_t* stats_out, int num_sms,
-                    cudaStream_t s) {
+                    Lane s) {
   const OrderWs ow = order_ws_layout(order_ws, m);
   CertWs w = cert_layout(cert_ws, m, n);
   // the control words, counters and bitsets start at zero (they are laid out
   // first, contiguously)
   cudaMemsetAsync(w.ctrl, 0, reinterpret_cast<char*>(w.pos) - reinterpret_cast<char*>(w.ctrl), s);
   const int gb = (m + 255) / 256;
-  note_launch();
-  cert_init_kernel<<<std::min(1024, std::max(1, (int)(((size_t)m * m + 255) / 256))), 256, 0, s>>>(
-      D, m, w.ctrl, w.dmax);
+  launch(cert_init_kernel, std::min(1024, std::max(1, (int)(((size_t)m * m + 255) / 256))), 256, 0,
+         s, D, m, w.ctrl, w.dmax);
   const auto resume = m <= STH       ? cert_resume_kernel<1>
                       : m <= 2 * STH ? cert_resume_kernel<2>
                       : m <= 4 * STH ? cert_resume_kernel<4>
                       : m <= 8 * STH ? cert_resume_kernel<8>
                                      : cert_resume_kernel<16>;
   for (int r = 0; r < CERT_ROUNDS; ++r) {
-    note_launch();
-    cert_round_kernel<<<gb, 256, 0, s>>>(order, m, r, w.ctrl, w.pos, w.flag, w.ccount, w.spick,
-                                         w.dmax, w.thr);
-    note_launch();
-    cert_flag_kernel<<<(m + 31) / 32, 32, 8 * (size_t)m, s>>>(ow.pt, ow.sh, ow.sl, order, w.pos,
-                                                   w.thr, m, w.ctrl, w.dmax, w.flag, w.ccount,
-                                                   w.cand);
-    note_launch();
-    cert_mark_kernel<<<m, RTH, 0, s>>>(D, order, w.pos, m, w.ctrl, w.dmax, w.flag, w.ccount,
-                                      w.cand, w.need, w.done, w.pairs, w.stats);
-    note_launch();
-    cert_stats_kernel<<<m, RTH, 0, s>>>(E, lde, m, n, w.ctrl, w.xs, w.hx);
-    note_launch();
-    cert_pairs_kernel<<<4 * num_sms, RTH, 0, s>>>(w.xs, m, n, w.ctrl, w.hx, w.pairs, w.D64,
-                                                  w.done, w.stats);
-    note_launch();
-    cert_decide_kernel<<<m, RTH, 0, s>>>(order, w.pos, m, w.ctrl, w.flag, w.ccount, w.cand,
-                                        w.D64, w.done, w.pick);
-    note_launch();
-    resume<<<1, STH, 0, s>>>(ow.pt, ow.sh, ow.sl, m, order, w.pos, w.pick, w.ctrl, w.spick,
-                             w.stats);
+    launch(cert_round_kernel, gb, 256, 0, s, order, m, r, w.ctrl, w.pos, w.flag, w.ccount, w.spick,
+           w.dmax, w.thr);
+    launch(cert_flag_kernel, (m + 31) / 32, 32, 8 * (size_t)m, s, ow.pt, ow.sh, ow.sl, order,
+           w.pos, w.thr, m, w.ctrl, w.dmax, w.flag, w.ccount, w.cand);
+    launch(cert_mark_kernel, m, RTH, 0, s, D, order, w.pos, m, w.ctrl, w.dmax, w.flag, w.ccount,
+           w.cand, w.need, w.done, w.pairs, w.stats);
+    launch(cert_stats_kernel, m, RTH, 0, s, E, lde, m, n, w.ctrl, w.xs, w.hx);
+    launch(cert_pairs_kernel, 4 * num_sms, RTH, 0, s, w.xs, m, n, w.ctrl, w.hx, w.pairs, w.D64,
+           w.done, w.stats);
+    launch(cert_decide_kernel, m, RTH, 0, s, order, w.pos, m, w.ctrl, w.flag, w.ccount, w.cand,
+           w.D64, w.done, w.pick);
+    launch(resume, 1, STH, 0, s, ow.pt, ow.sh, ow.sl, m, order, w.pos, w.pick, w.ctrl, w.spick,
+           w.stats);
   }
-  note_launch();
-  cert_tail_kernel<<<1, 1, 0, s>>>(m, w.ctrl, w.stats);
+  launch(cert_tail_kernel, 1, 1, 0, s, m, w.ctrl, w.stats);
   if (stats_out)
     cudaMemcpyAsync(stats_out, w.stats, 4 * sizeof(int), cudaMemcpyDeviceToDevice, s);
 }

@@ -637,6 +637,7 @@ __global__ void __launch_bounds__(CTH, 1)
     chol_cluster_kernel(float* __restrict__ A, int64_t lda, int n, float* __restrict__ dinv,
                         const double* __restrict__ diag0, float rel_tol, float* scratch, int own,
                         int* st) {
+  pdl_wait(diag0);  // all else is written here too
   extern __shared__ __align__(16) float cc_smem[];
   const int nblk = (n + CB - 1) / CB, W = (int)cluster_size() - 1, rank = (int)cluster_rank();
   const size_t tiles = (size_t)(nblk * (nblk + 1) / 2) * CB * CB;
@@ -669,7 +670,7 @@ Shape cluster_shape(int n) {
 // small or the cluster not launched (the caller then uses another path).
 bool launch_chol_cluster(float* A, int64_t lda, int n, float* dinv, const double* diag0,
                          float rel_tol, float* scratch, size_t scratch_cap, int* st,
-                         cudaStream_t s) {
+                         Lane s) {
   if (n < 1 || n > CL_NMAX) return false;
   const int nblk = (n + CB - 1) / CB;
   if (nblk > 3 && scratch_floats(nblk) > scratch_cap) return false;
@@ -688,13 +689,14 @@ bool launch_chol_cluster(float* A, int64_t lda, int n, float* dinv, const double
   cfg.blockDim = dim3(CTH, 1, 1);
   cfg.dynamicSmemBytes = h.smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = h.cl;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  at[1] = pdl_attribute();
+  cfg.numAttrs = s.overlap ? 2 : 1;
   note_launch();
   if (cudaLaunchKernelEx(&cfg, chol_cluster_kernel, A, lda, n, dinv, diag0, rel_tol, scratch,
                          h.own, st) !=

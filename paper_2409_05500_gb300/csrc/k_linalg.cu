@@ -84,6 +84,7 @@ __global__ void __launch_bounds__(NTH) gemm_kernel(int M, int N, int K, int kchu
                                                    View<T> Bl, double beta, TC* __restrict__ C,
                                                    int64_t ldc, int mode,
                                                    double* __restrict__ part) {
+  pdl_begin(C, part);
   constexpr int BM = 16 * TMt, BN = 16 * TNt;
   constexpr int NOP = SPLIT ? 2 : 1;
   const int r0 = blockIdx.y * BM, c0 = blockIdx.x * BN;
@@ -228,6 +229,7 @@ template <class TC>
 __global__ void splitk_reduce_f32_kernel(const float* __restrict__ part, int ksplit, int M,
                                          int N, double beta, TC* __restrict__ C, int64_t ldc,
                                          int mode) {
+  pdl_begin(part, C);
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)M * N) return;
   int r = (int)(idx / N), c = (int)(idx % N);
@@ -252,6 +254,7 @@ __global__ void splitk_reduce_f32_kernel(const float* __restrict__ part, int ksp
 template <class TC>
 __global__ void splitk_reduce_kernel(const double* __restrict__ part, int ksplit, int M, int N,
                                      double beta, TC* __restrict__ C, int64_t ldc, int mode) {
+  pdl_begin(part, C);
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)M * N) return;
   int r = (int)(idx / N), c = (int)(idx % N);
@@ -310,6 +313,7 @@ __global__ void __launch_bounds__(NTH) chol_diag_kernel(T* __restrict__ A, int64
                                                         T* __restrict__ dinv,
                                                         const double* __restrict__ diag0,
                                                         double rel_tol, int* st) {
+  pdl_wait(diag0);  // all else is written here too
   extern __shared__ __align__(16) unsigned char chol_smem[];
   T* L = reinterpret_cast<T*>(chol_smem);  // entry (i, k) at i CROW + (k & 3) CLS + k / 4
   __shared__ __align__(16) T colj[2][CHOL_NB];
@@ -438,19 +442,11 @@ constexpr int SBP = SB + 4;  // panel row stride in shared memory (16-byte align
 constexpr int SINGLE_MAX = 512;
 constexpr int STH = 512;
 
-__device__ __forceinline__ unsigned long long gtimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-// prof (optional, NULL in the library): three globaltimer stamps per block
-// column (after the diagonal block, the panel and the trailing update).
 __global__ void __launch_bounds__(STH) chol_single_kernel(float* __restrict__ A, int64_t lda,
                                                           int n, float* __restrict__ dinv,
                                                           const double* __restrict__ diag0,
-                                                          float rel_tol, int* st,
-                                                          unsigned long long* prof = nullptr) {
+                                                          float rel_tol, int* st) {
+  pdl_begin(A, dinv, diag0, st);
   extern __shared__ __align__(16) float cs_smem[];
   const int nblk = (n + SB - 1) / SB;
   float* P = cs_smem;                      // [max(n, SB)][SBP] panel; rows 0..31 also
@@ -532,7 +528,6 @@ __global__ void __launch_bounds__(STH) chol_single_kernel(float* __restrict__ A,
         if (r < nb && lane <= r) A[(int64_t)(k0 + r) * lda + k0 + lane] = P[(size_t)r * SBP + lane];
     }
     __syncthreads();
-    if (prof && tid == 0) prof[3 * b] = gtimer();
     // panel rows below the block: P[i][c] = sum_{q <= c} A[i][k0+q] Linv[c][q]
     const int r0 = k0 + SB;
     for (int i0 = r0 + 4 * warp; i0 < n; i0 += 4 * (STH / 32)) {  // four rows per warp
@@ -556,7 +551,6 @@ __global__ void __launch_bounds__(STH) chol_single_kernel(float* __restrict__ A,
       }
     }
     __syncthreads();
-    if (prof && tid == 0) prof[3 * b + 1] = gtimer();
     // trailing update, lower triangle, 32 x 32 tiles over rows/cols >= r0
     const int nt = (n - r0 + SB - 1) / SB;
     const int ntiles = nt * (nt + 1) / 2;
@@ -599,7 +593,6 @@ __global__ void __launch_bounds__(STH) chol_single_kernel(float* __restrict__ A,
       }
     }
     __syncthreads();
-    if (prof && tid == 0) prof[3 * b + 2] = gtimer();
   }
   if (tid == 0 && bad) set_status(st, VL_ERR_RANK);
   // 64 x 64 diagonal-block inverses for the blocked solves
@@ -678,6 +671,7 @@ __global__ void __launch_bounds__(NTH) trsm_cols_kernel(const T* __restrict__ L,
                                                         const T* __restrict__ dinv, int n,
                                                         T* __restrict__ R, int64_t ldr, int nrhs,
                                                         int backward) {
+  pdl_begin(L, dinv, R);
   extern __shared__ __align__(16) unsigned char trsm_smem[];
   T* Lbuf = reinterpret_cast<T*>(trsm_smem);          // [2][64][LSW]
   T* Dbuf = Lbuf + 2 * CHOL_NB * LSW;                  // [64][LSW]  inverse block
@@ -786,6 +780,7 @@ size_t trsm_smem_bytes() {
 template <class TI, class TO>
 __global__ void convert_kernel(const TI* __restrict__ in, int64_t ldi, TO* __restrict__ out,
                                int64_t ldo, int rows, int cols) {
+  pdl_begin(in, out);
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)rows * cols) return;
   int r = (int)(idx / cols), c = (int)(idx % cols);
@@ -795,12 +790,14 @@ __global__ void convert_kernel(const TI* __restrict__ in, int64_t ldi, TO* __res
 template <class T>
 __global__ void save_diag_kernel(const T* __restrict__ A, int64_t lda, int n,
                                  double* __restrict__ d) {
+  pdl_begin(A, d);
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) d[i] = (double)A[(int64_t)i * lda + i];
 }
 
 template <class T>
 __global__ void set_identity_kernel(T* A, int64_t lda, int n) {
+  pdl_begin(A);
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)n * n) return;
   int r = (int)(idx / n), c = (int)(idx % n);
@@ -832,18 +829,16 @@ void gemm_launch(const Ctx& cx, int M, int N, int K, double alpha, View<T> A, Vi
   int kchunk = ks > 1 ? (((K + ks - 1) / ks + 31) / 32) * 32 : std::max(K, 1);
   ks = ks > 1 ? (K + kchunk - 1) / kchunk : 1;
   dim3 grid(gn, gm, ks);
-  note_launch();
-  gemm_kernel<T, TC, TMt, TNt, SPLIT><<<grid, NTH, 0, cx.s>>>(
-      M, N, K, kchunk, alpha, A, Al, B, Bl, beta, C, ldc, mode, ks > 1 ? cx.part : nullptr);
+  launch(gemm_kernel<T, TC, TMt, TNt, SPLIT>, grid, NTH, 0, cx.s, M, N, K, kchunk, alpha, A, Al, B,
+         Bl, beta, C, ldc, mode, ks > 1 ? cx.part : nullptr);
   if (ks > 1) {
     int64_t tot = (int64_t)M * N;
-    note_launch();
     if constexpr (!SPLIT && sizeof(T) == 4)
-      splitk_reduce_f32_kernel<TC><<<(unsigned)((tot + 255) / 256), 256, 0, cx.s>>>(
-          reinterpret_cast<const float*>(cx.part), ks, M, N, beta, C, ldc, mode);
+      launch(splitk_reduce_f32_kernel<TC>, (unsigned)((tot + 255) / 256), 256, 0, cx.s,
+             reinterpret_cast<const float*>(cx.part), ks, M, N, beta, C, ldc, mode);
     else
-      splitk_reduce_kernel<TC><<<(unsigned)((tot + 255) / 256), 256, 0, cx.s>>>(
-          cx.part, ks, M, N, beta, C, ldc, mode);
+      launch(splitk_reduce_kernel<TC>, (unsigned)((tot + 255) / 256), 256, 0, cx.s, cx.part, ks, M,
+             N, beta, C, ldc, mode);
   }
 }
 
@@ -907,10 +902,9 @@ template <class T>
 void chol_blocked(const Ctx& cx, T* A, int64_t lda, int n, T* dinv, double* diag0,
                   double pivot_floor) {
   const int NB = CHOL_NB;
-  cudaStream_t s = cx.s;
+  Lane s = cx.s;
   const double rel_tol = pivot_floor > 0 ? pivot_floor : (sizeof(T) == 4 ? 1e-6 : 1e-12);
-  note_launch();
-  save_diag_kernel<T><<<(n + 255) / 256, 256, 0, s>>>(A, lda, n, diag0);
+  launch(save_diag_kernel<T>, (n + 255) / 256, 256, 0, s, A, lda, n, diag0);
   if constexpr (sizeof(T) == 4) {
     if (n <= SINGLE_MAX) {
       if (launch_chol_cluster(A, lda, n, dinv, diag0, (float)rel_tol,
@@ -923,9 +917,8 @@ void chol_blocked(const Ctx& cx, T* A, int64_t lda, int n, T* dinv, double* diag
                              (int)smem1);
         attr1 = true;
       }
-      note_launch();
-      chol_single_kernel<<<1, STH, chol_single_smem(n), s>>>(A, lda, n, dinv, diag0,
-                                                            (float)rel_tol, cx.st);
+      launch(chol_single_kernel, 1, STH, chol_single_smem(n), s, A, lda, n, dinv, diag0,
+             (float)rel_tol, cx.st);
       return;
     }
   }
@@ -939,9 +932,8 @@ void chol_blocked(const Ctx& cx, T* A, int64_t lda, int n, T* dinv, double* diag
   for (int k0 = 0; k0 < n; k0 += NB) {
     const int nb = std::min(NB, n - k0);
     T* dblk = dinv + (int64_t)(k0 / NB) * NB * NB;
-    note_launch();
-    chol_diag_kernel<T><<<1, NTH, smem, s>>>(A + (int64_t)k0 * lda + k0, lda, nb, dblk,
-                                             diag0 + k0, rel_tol, cx.st);
+    launch(chol_diag_kernel<T>, 1, NTH, smem, s, A + (int64_t)k0 * lda + k0, lda, nb, dblk, diag0 +
+           k0, rel_tol, cx.st);
     const int rest = n - k0 - nb;
     if (rest <= 0) break;
     // panel: L[i, k0:k0+nb] = A[i, k0:k0+nb] * Linv_kk^T
@@ -969,9 +961,8 @@ void chol_solve_blocked(const Ctx& cx, const T* L, int64_t lda, const T* dinv, i
                          (int)smem);
     attr_set = true;
   }
-  note_launch();
-  trsm_cols_kernel<T><<<(nrhs + SC - 1) / SC, NTH, smem, cx.s>>>(L, lda, dinv, n, R, ldr, nrhs,
-                                                                 backward ? 1 : 0);
+  launch(trsm_cols_kernel<T>, (nrhs + SC - 1) / SC, NTH, smem, cx.s, L, lda, dinv, n, R, ldr, nrhs,
+         backward ? 1 : 0);
 }
 template void chol_solve_blocked<float>(const Ctx&, const float*, int64_t, const float*, int,
                                         float*, int64_t, int, bool);
@@ -980,27 +971,25 @@ template void chol_solve_blocked<double>(const Ctx&, const double*, int64_t, con
 
 template <class TI, class TO>
 void launch_convert(const TI* in, int64_t ldi, TO* out, int64_t ldo, int rows, int cols,
-                    cudaStream_t s) {
+                    Lane s) {
   int64_t tot = (int64_t)rows * cols;
   if (tot <= 0) return;
-  note_launch();
-  convert_kernel<TI, TO><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(in, ldi, out, ldo, rows,
-                                                                      cols);
+  launch(convert_kernel<TI, TO>, (unsigned)((tot + 255) / 256), 256, 0, s, in, ldi, out, ldo, rows,
+         cols);
 }
 template void launch_convert<double, float>(const double*, int64_t, float*, int64_t, int, int,
-                                            cudaStream_t);
+                                            Lane);
 template void launch_convert<float, double>(const float*, int64_t, double*, int64_t, int, int,
-                                            cudaStream_t);
+                                            Lane);
 template void launch_convert<double, double>(const double*, int64_t, double*, int64_t, int, int,
-                                             cudaStream_t);
+                                             Lane);
 
 template <class T>
-void launch_set_identity(T* A, int64_t lda, int n, cudaStream_t s) {
+void launch_set_identity(T* A, int64_t lda, int n, Lane s) {
   int64_t tot = (int64_t)n * n;
-  note_launch();
-  set_identity_kernel<T><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(A, lda, n);
+  launch(set_identity_kernel<T>, (unsigned)((tot + 255) / 256), 256, 0, s, A, lda, n);
 }
-template void launch_set_identity<float>(float*, int64_t, int, cudaStream_t);
-template void launch_set_identity<double>(double*, int64_t, int, cudaStream_t);
+template void launch_set_identity<float>(float*, int64_t, int, Lane);
+template void launch_set_identity<double>(double*, int64_t, int, Lane);
 
 }  // namespace vl

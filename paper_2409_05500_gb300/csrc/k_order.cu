@@ -31,6 +31,7 @@ static_assert(VL_MAX_M <= 4096, "the search key holds the variable index in 12 b
 
 // Pt[c * m + i] = min(0, D[i * m + c])^2 as a double-float pair.
 __global__ void pt_kernel(const double* __restrict__ D, int m, float2* __restrict__ pt, int* st) {
+  pdl_begin(D, pt, st);
   __shared__ double tile[32][33];
   const int c0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -58,6 +59,7 @@ __global__ void pt_kernel(const double* __restrict__ D, int m, float2* __restric
 // S_i = sum_{j != i} min(0, D_ij)^2 in FP64, one warp per row, fixed order.
 __global__ void rowsum_kernel(const double* __restrict__ D, int m, float* __restrict__ sh,
                               float* __restrict__ sl) {
+  pdl_begin(D, sh, sl);
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (i >= m) return;
@@ -167,6 +169,7 @@ __global__ void __launch_bounds__(OC_TH) order_local_kernel(const float2* __rest
                                                             const float* __restrict__ sl0, int m,
                                                             int32_t* __restrict__ order,
                                                             float2* __restrict__ spick) {
+  pdl_wait(pt, sh0, sl0, order, spick);
   extern __shared__ __align__(16) float2 oc_rows[];
   stage_rows(pt, m, 0, m, oc_rows);
   __syncthreads();
@@ -200,6 +203,7 @@ __global__ void __launch_bounds__(OC_TH) order_cluster_kernel(const float2* __re
                                                               const float* __restrict__ sl0, int m,
                                                               int32_t* __restrict__ order,
                                                               float2* __restrict__ spick) {
+  pdl_wait(pt, sh0, sl0, order, spick);
   extern __shared__ __align__(16) float2 oc_rows[];
   unsigned rank;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
@@ -238,7 +242,7 @@ __global__ void __launch_bounds__(OC_TH) order_cluster_kernel(const float2* __re
 // caller then runs order_kernel).
 template <int NW>
 bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, float2* spick,
-                          cudaStream_t s) {
+                          Lane s) {
   static bool attr = false;
   if (!attr) {
     if (cudaFuncSetAttribute(order_cluster_kernel<NW>,
@@ -254,13 +258,14 @@ bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, float2* spick
   cfg.blockDim = dim3(OC_TH, 1, 1);
   cfg.dynamicSmemBytes = oc_smem(m);
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = OC_CTAS;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  at[1] = pdl_attribute();
+  cfg.numAttrs = s.overlap ? 2 : 1;
   note_launch();
   if (cudaLaunchKernelEx(&cfg, order_cluster_kernel<NW>, (const float2*)w.pt,
                          (const float*)w.sh, (const float*)w.sl, m, order, spick) !=
@@ -272,16 +277,15 @@ bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, float2* spick
 }
 
 template <int NW>
-void launch_order_local(const OrderWs& w, int m, int32_t* order, float2* spick, cudaStream_t s) {
+void launch_order_local(const OrderWs& w, int m, int32_t* order, float2* spick, Lane s) {
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(order_local_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          OL_MAX_M * OL_MAX_M * (int)sizeof(float2));
     attr = true;
   }
-  note_launch();
-  order_local_kernel<NW><<<1, OC_TH, (size_t)m * m * sizeof(float2), s>>>(w.pt, w.sh, w.sl, m,
-                                                                         order, spick);
+  launch(order_local_kernel<NW>, 1, OC_TH, (size_t)m * m * sizeof(float2), s, w.pt, w.sh, w.sl, m,
+         order, spick);
 }
 
 // Gaps after the search, from the order: variable i replays its score S_i =
@@ -300,6 +304,7 @@ __global__ void __launch_bounds__(GAP_TH)
     gap_scores_kernel(const float2* __restrict__ pt, const float* __restrict__ sh0,
                       const float* __restrict__ sl0, const int32_t* __restrict__ order, int m,
                       double* __restrict__ s1, unsigned long long* __restrict__ s2) {
+  pdl_begin(pt, sh0, sl0, order, s1, s2);
   constexpr int PER = GAP_V * GAP_T / GAP_TH;
   __shared__ double ps[GAP_T][GAP_V];  // P_i,order[k], then the scores before step k
   __shared__ int pos[GAP_V];           // the step of i's own pick, once reached
@@ -363,6 +368,7 @@ __global__ void __launch_bounds__(GAP_TH)
 
 __global__ void gap_kernel(const double* __restrict__ s1, const unsigned long long* __restrict__ s2,
                            int m, double* __restrict__ gap) {
+  pdl_begin(s1, s2, gap);
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= m) return;
   if (s2[k] == ~0ull) {
@@ -388,14 +394,12 @@ OrderWs order_ws_layout(void* ws, int m) {
 }
 
 void launch_order_gaps(void* ws, int m, const int32_t* order, double* gap,
-                       cudaStream_t s) {
+                       Lane s) {
   const OrderWs w = order_ws_layout(ws, m);
   cudaMemsetAsync(w.s2, 0xff, (size_t)m * sizeof(unsigned long long), s);
-  note_launch();
-  gap_scores_kernel<<<(m + GAP_V - 1) / GAP_V, GAP_TH, 0, s>>>(w.pt, w.sh, w.sl, order, m,
-                                                                   w.s1, w.s2);
-  note_launch();
-  gap_kernel<<<(m + 255) / 256, 256, 0, s>>>(w.s1, w.s2, m, gap);
+  launch(gap_scores_kernel, (m + GAP_V - 1) / GAP_V, GAP_TH, 0, s, w.pt, w.sh, w.sl, order, m,
+         w.s1, w.s2);
+  launch(gap_kernel, (m + 255) / 256, 256, 0, s, w.s1, w.s2, m, gap);
 }
 
 size_t order_ws_bytes(int m) {
@@ -404,13 +408,11 @@ size_t order_ws_bytes(int m) {
 }
 
 void launch_causal_order(const double* D, int m, void* ws, int32_t* order, double* gap, int* st,
-                         cudaStream_t s, float2* spick) {
+                         Lane s, float2* spick) {
   const OrderWs w = order_ws_layout(ws, m);
   dim3 grid((m + 31) / 32, (m + 31) / 32), block(32, 8);
-  note_launch();
-  pt_kernel<<<grid, block, 0, s>>>(D, m, w.pt, st);
-  note_launch();
-  rowsum_kernel<<<(m + 7) / 8, 256, 0, s>>>(D, m, w.sh, w.sl);
+  launch(pt_kernel, grid, block, 0, s, D, m, w.pt, st);
+  launch(rowsum_kernel, (m + 7) / 8, 256, 0, s, D, m, w.sh, w.sl);
   const bool cluster = m > OL_MAX_M && m <= OC_MAX_M &&
                        (m <= 256 ? launch_order_cluster<8>(w, m, order, spick, s)
                                  : launch_order_cluster<16>(w, m, order, spick, s));
@@ -423,15 +425,15 @@ void launch_causal_order(const double* D, int m, void* ws, int32_t* order, doubl
   } else if (m <= OL_MAX_M) {
     launch_order_local<8>(w, m, order, spick, s);
   } else if (!cluster) {
-    note_launch();
+    const Lane alone(s, false);  // order_kernel has no pdl_wait: 1.5 us of 250 or more
     if (m <= 2 * STH)
-      order_kernel<2><<<1, STH, 0, s>>>(w.pt, w.sh, w.sl, m, order, spick);
+      launch(order_kernel<2>, 1, STH, 0, alone, w.pt, w.sh, w.sl, m, order, spick);
     else if (m <= 4 * STH)
-      order_kernel<4><<<1, STH, 0, s>>>(w.pt, w.sh, w.sl, m, order, spick);
+      launch(order_kernel<4>, 1, STH, 0, alone, w.pt, w.sh, w.sl, m, order, spick);
     else if (m <= 8 * STH)
-      order_kernel<8><<<1, STH, 0, s>>>(w.pt, w.sh, w.sl, m, order, spick);
+      launch(order_kernel<8>, 1, STH, 0, alone, w.pt, w.sh, w.sl, m, order, spick);
     else
-      order_kernel<16><<<1, STH, 0, s>>>(w.pt, w.sh, w.sl, m, order, spick);
+      launch(order_kernel<16>, 1, STH, 0, alone, w.pt, w.sh, w.sl, m, order, spick);
   }
   if (gap) launch_order_gaps(ws, m, order, gap, s);
 }

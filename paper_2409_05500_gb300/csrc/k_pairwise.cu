@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(TB / MTI * 16, MINB)
     pairwise_f32_kernel(const float* __restrict__ xt, int m, int m_pad, int T, int n_run,
                         int tps, const float* __restrict__ rho32,
                         const float* __restrict__ c32, float* __restrict__ part) {
+  pdl_begin(xt, rho32, c32, part);
   pairwise_f32_item<MTI, TTS>(blockIdx.x, blockIdx.y, xt, m, m_pad, T, n_run, tps, rho32, c32,
                               part);
 }
@@ -291,6 +292,7 @@ template <int MTI, int TTS, int MINB>
 __global__ void __launch_bounds__(TB / MTI * 16, MINB)
     pairwise_f32_list_kernel(const PairJob* __restrict__ jobs, const int4* __restrict__ items,
                              int nitems) {
+  pdl_begin(jobs, items);
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
     const int4 w = items[it];
     const PairJob& j = jobs[w.x];
@@ -327,6 +329,7 @@ __global__ void __launch_bounds__(FX_TH)
     pairwise_f64_kernel(const double* __restrict__ xt, int m, int m_pad, int n_real, int tps,
                         const double* __restrict__ rho64, const double* __restrict__ c64,
                         double* __restrict__ part) {
+  pdl_begin(xt, rho64, c64, part);
   __shared__ fx::u64 te[fx::EXP_N], tl[fx::LOG_N];
   __shared__ fx::u32 tr[fx::LOG_N];
   const fx::Tab T{te, tl, tr};
@@ -364,6 +367,7 @@ __global__ void __launch_bounds__(FX_TH)
 __global__ void pair_consts64_kernel(const double* __restrict__ C, int m,
                                      double* __restrict__ rho64, double* __restrict__ c64,
                                      int* st) {
+  pdl_begin(C, rho64, c64, st);
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int a = (int)(idx / m), b = (int)(idx % m);
   if (idx >= (int64_t)m * m || b <= a) return;
@@ -387,6 +391,7 @@ __global__ void pair_consts64_kernel(const double* __restrict__ C, int m,
 __global__ void pair_consts_kernel(const double* __restrict__ C, const double* __restrict__ w,
                                    int m, float* __restrict__ rho32, float* __restrict__ c32,
                                    int* st) {
+  pdl_begin(C, w, rho32, c32, st);
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int a = (int)(idx / m), b = (int)(idx % m);
   if (idx >= (int64_t)m * m || b <= a) return;  // the pairwise kernel reads i < j
@@ -482,6 +487,7 @@ __global__ void __launch_bounds__(2 * FT * FT)
     measure_finalize_kernel(const void* __restrict__ part, int m, int splits, double inv_n,
                             const double* __restrict__ hx, double* __restrict__ Hx,
                             double* __restrict__ Hr, double* __restrict__ D) {
+  pdl_begin(part, hx, Hx, Hr, D);
   __shared__ double hs[2][FT][FT + 1];
   int I, J;
   tile_coords(blockIdx.x, (m + FT - 1) / FT, I, J);
@@ -580,22 +586,20 @@ PairPlan plan_pairwise(int m, int n, int num_sms, bool fp64) {
 }
 
 void launch_pair_consts(const double* C, const double* w, int m, float* rho32, float* c32,
-                        int* st, cudaStream_t s) {
+                        int* st, Lane s) {
   int64_t tot = (int64_t)m * m;
-  note_launch();
-  pair_consts_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(C, w, m, rho32, c32, st);
+  launch(pair_consts_kernel, (unsigned)((tot + 255) / 256), 256, 0, s, C, w, m, rho32, c32, st);
 }
 
 void launch_pair_consts64(const double* C, int m, double* rho64, double* c64, int* st,
-                          cudaStream_t s) {
+                          Lane s) {
   int64_t tot = (int64_t)m * m;
-  note_launch();
-  pair_consts64_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(C, m, rho64, c64, st);
+  launch(pair_consts64_kernel, (unsigned)((tot + 255) / 256), 256, 0, s, C, m, rho64, c64, st);
 }
 
 template <int MTI, int TTS, int MINB>
 void launch_pairwise_f32_cfg(const float* xt, const PairPlan& pl, const float* rho32,
-                             const float* c32, float* part, cudaStream_t s) {
+                             const float* c32, float* part, Lane s) {
   const int n_run = ((pl.n + KRUN - 1) / KRUN) * KRUN;
   dim3 grid(pl.tiles, pl.splits);
   const size_t smem = sizeof(float) * 3 * TTS * 2 * TB;  // three stages of TTS x 64 samples
@@ -605,13 +609,12 @@ void launch_pairwise_f32_cfg(const float* xt, const PairPlan& pl, const float* r
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr_set = true;
   }
-  note_launch();
-  pairwise_f32_kernel<MTI, TTS, MINB><<<grid, TB / MTI * 16, smem, s>>>(
-      xt, pl.m, pl.m_pad, pl.m_pad / TB, n_run, pl.t_per_split, rho32, c32, part);
+  launch(pairwise_f32_kernel<MTI, TTS, MINB>, grid, TB / MTI * 16, smem, s, xt, pl.m, pl.m_pad,
+         pl.m_pad / TB, n_run, pl.t_per_split, rho32, c32, part);
 }
 
 void launch_pairwise_f32(const float* xt, const PairPlan& pl, const float* rho32,
-                         const float* c32, float* part, cudaStream_t s) {
+                         const float* c32, float* part, Lane s) {
   launch_pairwise_f32_cfg<F32_MTI, F32_TTS, F32_MINB>(xt, pl, rho32, c32, part, s);
 }
 
@@ -631,7 +634,7 @@ PairJob make_pair_job(const float* xt, const PairPlan& pl, const float* rho32, c
 }
 
 void launch_pairwise_f32_list(const PairJob* jobs, const int4* items, int nitems, int grid,
-                              cudaStream_t s) {
+                              Lane s) {
   constexpr int MTI = F32_MTI, TTS = F32_TTS, MINB = F32_MINB;
   const size_t smem = sizeof(float) * 3 * TTS * 2 * TB;
   static bool attr_set = false;
@@ -640,26 +643,23 @@ void launch_pairwise_f32_list(const PairJob* jobs, const int4* items, int nitems
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr_set = true;
   }
-  note_launch();
-  pairwise_f32_list_kernel<MTI, TTS, MINB><<<std::max(1, std::min(grid, nitems)), TB / MTI * 16,
-                                             smem, s>>>(jobs, items, nitems);
+  launch(pairwise_f32_list_kernel<MTI, TTS, MINB>, std::max(1, std::min(grid, nitems)), TB / MTI *
+         16, smem, s, jobs, items, nitems);
 }
 
 void launch_pairwise_f64(const double* xt, const PairPlan& pl, const double* rho64,
-                         const double* c64, double* part, cudaStream_t s) {
+                         const double* c64, double* part, Lane s) {
   const int64_t pairs = (int64_t)pl.m * (pl.m - 1) / 2;
   dim3 grid((unsigned)((pairs + FX_TH - 1) / FX_TH), pl.splits);
-  note_launch();
-  pairwise_f64_kernel<<<grid, FX_TH, 0, s>>>(xt, pl.m, pl.m_pad, pl.n, pl.t_per_split, rho64,
-                                             c64, part);
+  launch(pairwise_f64_kernel, grid, FX_TH, 0, s, xt, pl.m, pl.m_pad, pl.n, pl.t_per_split, rho64,
+         c64, part);
 }
 
 void launch_measure_finalize(const void* part, const PairPlan& pl, const double* hx, double* Hx,
-                             double* Hr, double* D, bool fp32_parts, cudaStream_t s) {
+                             double* Hr, double* D, bool fp32_parts, Lane s) {
   const unsigned T = (pl.m + FT - 1) / FT;
-  note_launch();
-  (fp32_parts ? measure_finalize_kernel<true> : measure_finalize_kernel<false>)
-      <<<T * (T + 1) / 2, 2 * FT * FT, 0, s>>>(part, pl.m, pl.splits, 1.0 / pl.n, hx, Hx, Hr, D);
+  launch(fp32_parts ? measure_finalize_kernel<true> : measure_finalize_kernel<false>, T * (T + 1) /
+         2, 2 * FT * FT, 0, s, part, pl.m, pl.splits, 1.0 / pl.n, hx, Hx, Hr, D);
 }
 
 }  // namespace vl

@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(RTH, 4)
     refine_residual_kernel(const float* __restrict__ nhi, const float* __restrict__ nlo, int m,
                            int mp, const float* __restrict__ beta0, int kchunk,
                            float2* __restrict__ part) {
+  pdl_begin(nhi, nlo, beta0, part);
   __shared__ float Ah[RK][RT + 1], Al[RK][RT + 1];
   __shared__ __align__(8) float Bs[RK][RT];
   const int q = m + mp;
@@ -99,6 +100,7 @@ __global__ void __launch_bounds__(RTH, 4)
 __global__ void refine_reduce_kernel(const float* __restrict__ nhi, const float* __restrict__ nlo,
                                      int m, int mp, const float2* __restrict__ part, int splits,
                                      float* __restrict__ r) {
+  pdl_begin(nhi, nlo, part, r);
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)mp * m) return;
   const int a = (int)(idx / m), i = (int)(idx % m);
@@ -124,6 +126,7 @@ __global__ void refine_reduce_kernel(const float* __restrict__ nhi, const float*
 // beta0 replaced by its FP32 rounding (for the residuals of the VAR).
 __global__ void refine_apply_kernel(float* __restrict__ beta, const float* __restrict__ delta,
                                     int m, int p, double* __restrict__ M) {
+  pdl_begin(beta, delta, M);
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)p * m * m) return;
   const int a = (int)(idx / m), i = (int)(idx % m);  // a = tau m + k (0-based tau)
@@ -144,23 +147,21 @@ int refine_splits(int m, int p, int num_sms) {
 }
 
 void launch_refine_residual(const float* nhi, const float* nlo, int m, int p, const float* beta0,
-                            float* r, float2* part, int num_sms, cudaStream_t s) {
+                            float* r, float2* part, int num_sms, Lane s) {
   const int mp = m * p, splits = refine_splits(m, p, num_sms);
   const int kchunk = ((mp + splits - 1) / splits + RK - 1) / RK * RK;
   const int nz = (mp + kchunk - 1) / kchunk;
   dim3 grid((m + RT - 1) / RT, (mp + RT - 1) / RT, nz);
-  note_launch();
-  refine_residual_kernel<<<grid, RTH, 0, s>>>(nhi, nlo, m, mp, beta0, kchunk, part);
+  launch(refine_residual_kernel, grid, RTH, 0, s, nhi, nlo, m, mp, beta0, kchunk, part);
   const int64_t tot = (int64_t)mp * m;
-  note_launch();
-  refine_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(nhi, nlo, m, mp, part, nz, r);
+  launch(refine_reduce_kernel, (unsigned)((tot + 255) / 256), 256, 0, s, nhi, nlo, m, mp, part, nz,
+         r);
 }
 
 void launch_refine_apply(float* beta, const float* delta, int m, int p, double* M,
-                         cudaStream_t s) {
+                         Lane s) {
   const int64_t tot = (int64_t)p * m * m;
-  note_launch();
-  refine_apply_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(beta, delta, m, p, M);
+  launch(refine_apply_kernel, (unsigned)((tot + 255) / 256), 256, 0, s, beta, delta, m, p, M);
 }
 
 }  // namespace vl

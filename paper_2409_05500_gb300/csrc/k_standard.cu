@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(SC_WARPS * 32)
                           unsigned* __restrict__ counter, const int32_t* __restrict__ idx,
                           int32_t* __restrict__ order, double* __restrict__ gap, int k,
                           int* __restrict__ pick, int* st) {
+  pdl_begin(D, S, counter, idx, order, gap, pick, st);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int a = blockIdx.x * SC_WARPS + warp;
   if (a < u) {
@@ -120,6 +121,7 @@ __global__ void __launch_bounds__(RF_TH)
                       const int32_t* __restrict__ idx, double* __restrict__ Wn, int64_t ldn,
                       int32_t* __restrict__ idx_next, int32_t* __restrict__ order,
                       double* __restrict__ gap, int k) {
+  pdl_begin(W, C, pick, idx, Wn, idx_next, order, gap);
   const int pk = *pick;
   const int an = blockIdx.y;
   const int a = an + (an >= pk ? 1 : 0);
@@ -146,19 +148,17 @@ __global__ void __launch_bounds__(RF_TH)
 
 void launch_std_score_pick(const double* D, int u, double* S, unsigned* counter,
                            const int32_t* idx, int32_t* order, double* gap, int k, int* pick,
-                           int* st, cudaStream_t s) {
-  note_launch();
-  std_score_pick_kernel<<<(u + SC_WARPS - 1) / SC_WARPS, SC_WARPS * 32, 0, s>>>(
-      D, u, S, counter, idx, order, gap, k, pick, st);
+                           int* st, Lane s) {
+  launch(std_score_pick_kernel, (u + SC_WARPS - 1) / SC_WARPS, SC_WARPS * 32, 0, s, D, u, S,
+         counter, idx, order, gap, k, pick, st);
 }
 
 void launch_std_refine(const double* W, int64_t ldw, int u, int n, const double* C,
                        const int* pick, const int32_t* idx, double* Wn, int64_t ldn,
-                       int32_t* idx_next, int32_t* order, double* gap, int k, cudaStream_t s) {
+                       int32_t* idx_next, int32_t* order, double* gap, int k, Lane s) {
   const int chunks = std::min(8, std::max(1, (n + 4 * RF_TH - 1) / (4 * RF_TH)));
-  note_launch();
-  std_refine_kernel<<<dim3(chunks, u - 1), RF_TH, 0, s>>>(W, ldw, u, n, C, pick, idx, Wn, ldn,
-                                                          idx_next, order, gap, k);
+  launch(std_refine_kernel, dim3(chunks, u - 1), RF_TH, 0, s, W, ldw, u, n, C, pick, idx, Wn, ldn,
+         idx_next, order, gap, k);
 }
 
 }  // namespace vl

@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kStatMax)
     var_prep_kernel(const double* __restrict__ X, int64_t ldx, int m, int n, int p, double inv_n,
                     double inv_eff, double* __restrict__ Xc, int64_t ldc,
                     double* __restrict__ mu_out, double* __restrict__ wbar, int* st) {
+  pdl_begin(X, Xc, mu_out, wbar, st);
   __shared__ double red[2 * kStatMax];
   double* xc = Xc + blockIdx.x * ldc;
   centre_row(X + blockIdx.x * ldx, m, n, p, inv_n, inv_eff, red, mu_out, wbar, st,
@@ -144,6 +145,7 @@ __global__ void __launch_bounds__(kStatMax)
                      double* __restrict__ mu_out, double* __restrict__ wbar, int Kpad,
                      __nv_bfloat16* __restrict__ S, int64_t ldo, int64_t plane,
                      int* __restrict__ exps, int* st) {
+  pdl_begin(X, Xc, mu_out, wbar, S, exps, st);
   __shared__ double red[2 * kStatMax];
   __shared__ unsigned long long redu[32];
   const int k = blockIdx.x, n_eff = n - p;
@@ -191,6 +193,7 @@ __global__ void var_normal_eq_kernel(const double* __restrict__ G, int m, int p,
                                      const double* __restrict__ wbar, T* __restrict__ Gzz,
                                      T* __restrict__ Gzy, float* __restrict__ nhi,
                                      float* __restrict__ nlo) {
+  pdl_begin(G, wbar, Gzz, Gzy, nhi, nlo);
   const int mp = m * p, q = m * (p + 1);
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)mp * q) return;
@@ -209,6 +212,7 @@ __global__ void var_normal_eq_kernel(const double* __restrict__ G, int m, int p,
 
 template <class T>
 __global__ void var_coef_kernel(const T* __restrict__ beta, int m, int p, double* __restrict__ M) {
+  pdl_begin(beta, M);
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)p * m * m) return;
   const int tau = (int)(idx / ((int64_t)m * m));
@@ -225,6 +229,7 @@ template <class T>
 __global__ void __launch_bounds__(CST_TH)
     var_cst_kernel(const T* __restrict__ beta, int m, int p, const double* __restrict__ wbar,
                    double* __restrict__ cst) {
+  pdl_begin(beta, wbar, cst);
   __shared__ double red[CST_TH / 32][CST_C];
   const int i = blockIdx.x * CST_C + threadIdx.x % CST_C;
   double c = 0.0;
@@ -250,6 +255,7 @@ __global__ void var_resid_init_kernel(const double* __restrict__ X, int64_t ldx,
                                       const double* __restrict__ mu,
                                       const double* __restrict__ cst, double* __restrict__ E,
                                       int64_t lde) {
+  pdl_begin(X, mu, cst, E);
   const int i = blockIdx.y;
   const double off = mu[i] + cst[i];
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_eff; t += gridDim.x * blockDim.x)
@@ -309,6 +315,7 @@ __global__ void __launch_bounds__(kStatMax)
     standardize_kernel(const double* __restrict__ E, int64_t lde, int n, double inv_n,
                        double* __restrict__ mu_out, double* __restrict__ isd_out,
                        double* __restrict__ hx, int* st) {
+  pdl_begin(E, mu_out, isd_out, hx, st);
   __shared__ double red[2 * kStatMax];
   __shared__ fx::u64 te[fx::EXP_N], tl[fx::LOG_N];
   __shared__ fx::u32 tr[fx::LOG_N];
@@ -347,6 +354,7 @@ __global__ void __launch_bounds__(kStatMax)
                         __nv_bfloat16* __restrict__ S, int64_t plane, int* __restrict__ exps,
                         float* __restrict__ xs, float* __restrict__ xt, int m_pad, int n_pad,
                         double* __restrict__ hx, int* st) {
+  pdl_begin(E, S, exps, xs, xt, hx, st);
   __shared__ double red[2 * kStatMax];
   __shared__ unsigned long long redu[32];
   const int i = blockIdx.x;
@@ -404,6 +412,7 @@ __global__ void __launch_bounds__(kStatMax)
 __global__ void center64_kernel(const double* __restrict__ E, int64_t lde, int n,
                                 const double* __restrict__ mu, double* __restrict__ out,
                                 int64_t ldc) {
+  pdl_begin(E, mu, out);
   const int i = blockIdx.y;
   const double mi = mu[i];
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ldc;
@@ -416,6 +425,7 @@ __global__ void transpose_std_kernel(const double* __restrict__ E, int64_t lde, 
                                      const double* __restrict__ mu,
                                      const double* __restrict__ isd, double* __restrict__ xt,
                                      int m_pad, int n_pad) {
+  pdl_begin(E, mu, isd, xt);
   __shared__ double tile[32][33];
   const int t0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
@@ -434,6 +444,7 @@ __global__ void transpose_std_kernel(const double* __restrict__ E, int64_t lde, 
 // multiples of 32.
 __global__ void transpose_f32_kernel(const float* __restrict__ xs, int m, int n_pad,
                                      float* __restrict__ xt, int m_pad) {
+  pdl_begin(xs, xt);
   __shared__ float tile[32][33];
   const int t0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
@@ -448,67 +459,60 @@ __global__ void transpose_f32_kernel(const float* __restrict__ xs, int m, int n_
 }  // namespace
 
 void launch_var_prep(const double* X, int64_t ldx, int m, int n, int p, double* Xc, int64_t ldc,
-                     double* mu, double* wbar, int* st, cudaStream_t s) {
-  note_launch();
-  var_prep_kernel<<<m, kStatMax, 0, s>>>(X, ldx, m, n, p, 1.0 / n, 1.0 / (n - p), Xc, ldc, mu, wbar, st);
+                     double* mu, double* wbar, int* st, Lane s) {
+  launch(var_prep_kernel, m, kStatMax, 0, s, X, ldx, m, n, p, 1.0 / n,
+         1.0 / (n - p), Xc, ldc, mu, wbar, st);
 }
 
 void launch_prep_lags(const double* X, int64_t ldx, int m, int n, int p, float* Xc, int64_t ldc,
                       double* mu, double* wbar, int64_t Kpad, void* S, int64_t plane, int* exps,
-                      int* st, cudaStream_t s) {
-  note_launch();
-  prep_lags_kernel<<<m, kStatMax, 0, s>>>(X, ldx, m, n, p, 1.0 / n, 1.0 / (n - p), Xc, ldc, mu, wbar, (int)Kpad,
-                                              static_cast<__nv_bfloat16*>(S), Kpad, plane, exps,
-                                              st);
+                      int* st, Lane s) {
+  launch(prep_lags_kernel, m, kStatMax, 0, s, X, ldx, m, n, p, 1.0 / n,
+         1.0 / (n - p), Xc, ldc, mu, wbar,
+         (int)Kpad, static_cast<__nv_bfloat16*>(S), Kpad, plane, exps, st);
 }
 
 template <class T>
 void launch_var_normal_eq(const double* G, int m, int p, int n_eff, const double* wbar, T* Gzz,
-                          T* Gzy, cudaStream_t s, float* nhi, float* nlo) {
+                          T* Gzy, Lane s, float* nhi, float* nlo) {
   const int mp = m * p;
   const int64_t tot = (int64_t)mp * (mp + m);
-  note_launch();
-  var_normal_eq_kernel<T><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(G, m, p, n_eff, wbar,
-                                                                        Gzz, Gzy, nhi, nlo);
+  launch(var_normal_eq_kernel<T>, (unsigned)((tot + 255) / 256), 256, 0, s, G, m, p, n_eff, wbar,
+         Gzz, Gzy, nhi, nlo);
 }
 template void launch_var_normal_eq<float>(const double*, int, int, int, const double*, float*,
-                                          float*, cudaStream_t, float*, float*);
+                                          float*, Lane, float*, float*);
 template void launch_var_normal_eq<double>(const double*, int, int, int, const double*,
-                                           double*, double*, cudaStream_t, float*, float*);
+                                           double*, double*, Lane, float*, float*);
 
 template <class T>
 void launch_var_coef(const T* beta, int m, int p, const double* wbar, double* M, double* cst,
-                     cudaStream_t s) {
+                     Lane s) {
   const int64_t tot = (int64_t)p * m * m;
-  note_launch();
-  var_coef_kernel<T><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(beta, m, p, M);
-  note_launch();
-  var_cst_kernel<T><<<(m + CST_C - 1) / CST_C, CST_TH, 0, s>>>(beta, m, p, wbar, cst);
+  launch(var_coef_kernel<T>, (unsigned)((tot + 255) / 256), 256, 0, s, beta, m, p, M);
+  launch(var_cst_kernel<T>, (m + CST_C - 1) / CST_C, CST_TH, 0, s, beta, m, p, wbar, cst);
 }
 template void launch_var_coef<float>(const float*, int, int, const double*, double*, double*,
-                                     cudaStream_t);
+                                     Lane);
 
 template <class T>
-void launch_var_cst(const T* beta, int m, int p, const double* wbar, double* cst, cudaStream_t s) {
-  note_launch();
-  var_cst_kernel<T><<<(m + CST_C - 1) / CST_C, CST_TH, 0, s>>>(beta, m, p, wbar, cst);
+void launch_var_cst(const T* beta, int m, int p, const double* wbar, double* cst, Lane s) {
+  launch(var_cst_kernel<T>, (m + CST_C - 1) / CST_C, CST_TH, 0, s, beta, m, p, wbar, cst);
 }
-template void launch_var_cst<float>(const float*, int, int, const double*, double*, cudaStream_t);
+template void launch_var_cst<float>(const float*, int, int, const double*, double*, Lane);
 template void launch_var_coef<double>(const double*, int, int, const double*, double*, double*,
-                                      cudaStream_t);
+                                      Lane);
 
 void launch_var_resid_init(const double* X, int64_t ldx, int m, int n, int p, const double* mu,
-                           const double* cst, double* E, int64_t lde, cudaStream_t s) {
+                           const double* cst, double* E, int64_t lde, Lane s) {
   const int n_eff = n - p;
   dim3 grid((unsigned)((n_eff + 255) / 256 < 64 ? (n_eff + 255) / 256 : 64), m);
-  note_launch();
-  var_resid_init_kernel<<<grid, 256, 0, s>>>(X, ldx, n_eff, p, mu, cst, E, lde);
+  launch(var_resid_init_kernel, grid, 256, 0, s, X, ldx, n_eff, p, mu, cst, E, lde);
 }
 
 void launch_standardize(const double* E, int64_t lde, int m, int n, double* mu, double* inv_sd,
-                        double* hx, int* st, cudaStream_t s) {
-  note_launch();
-  standardize_kernel<<<m, kStatMax, 0, s>>>(E, lde, n, 1.0 / n, mu, inv_sd, hx, st);
+                        double* hx, int* st, Lane s) {
+  launch(standardize_kernel, m, kStatMax, 0, s, E, lde, n, 1.0 / n, mu, inv_sd, hx, st);
 }
 
 // The standardized rows go straight to their time-major places while that is
@@ -520,37 +524,33 @@ bool measure_prep_needs_rows(int m, int n) { return (int64_t)m * n > kDirectMax;
 
 void launch_measure_prep(const double* E, int64_t lde, int m, int n, int64_t Kpad, void* S,
                          int64_t plane, int* exps, float* xs, float* xt, int m_pad, int n_pad,
-                         double* hx, int* st, cudaStream_t s) {
+                         double* hx, int* st, Lane s) {
   __nv_bfloat16* Sb = static_cast<__nv_bfloat16*>(S);
-  note_launch();
   if (!xt) {
-    measure_prep_kernel<false><<<m, kStatMax, 0, s>>>(E, lde, m, n, 1.0 / n, (int)Kpad, Sb, plane, exps,
-                                                          nullptr, nullptr, 0, 0, nullptr, st);
+    launch(measure_prep_kernel<false>, m, kStatMax, 0, s, E, lde, m, n, 1.0 / n, (int)Kpad, Sb,
+           plane, exps, nullptr, nullptr, 0, 0, nullptr, st);
     return;
   }
   const bool rows = measure_prep_needs_rows(m, n);
-  measure_prep_kernel<true><<<rows ? m : m_pad, kStatMax, 0, s>>>(
-      E, lde, m, n, 1.0 / n, (int)Kpad, Sb, plane, exps, rows ? xs : nullptr, xt, m_pad, n_pad, hx, st);
+  launch(measure_prep_kernel<true>, rows ? m : m_pad, kStatMax, 0, s, E, lde, m, n, 1.0 / n,
+         (int)Kpad, Sb, plane, exps, rows ? xs : nullptr, xt, m_pad, n_pad, hx, st);
   if (rows) {
-    note_launch();
-    transpose_f32_kernel<<<dim3(n_pad / 32, m_pad / 32), dim3(32, 8), 0, s>>>(xs, m, n_pad, xt,
-                                                                             m_pad);
+    launch(transpose_f32_kernel, dim3(n_pad / 32, m_pad / 32), dim3(32, 8), 0, s, xs, m, n_pad, xt,
+           m_pad);
   }
 }
 
 void launch_center64(const double* E, int64_t lde, int m, int n, const double* mu, double* out,
-                     int64_t ldc, cudaStream_t s) {
+                     int64_t ldc, Lane s) {
   dim3 grid((unsigned)((ldc + 255) / 256 < 64 ? (ldc + 255) / 256 : 64), m);
-  note_launch();
-  center64_kernel<<<grid, 256, 0, s>>>(E, lde, n, mu, out, ldc);
+  launch(center64_kernel, grid, 256, 0, s, E, lde, n, mu, out, ldc);
 }
 
 void launch_transpose_std(const double* E, int64_t lde, int m, int n, const double* mu,
                           const double* inv_sd, double* xt, int m_pad, int n_pad,
-                          cudaStream_t s) {
+                          Lane s) {
   dim3 grid((n_pad + 31) / 32, (m_pad + 31) / 32), block(32, 8);
-  note_launch();
-  transpose_std_kernel<<<grid, block, 0, s>>>(E, lde, m, n, mu, inv_sd, xt, m_pad, n_pad);
+  launch(transpose_std_kernel, grid, block, 0, s, E, lde, m, n, mu, inv_sd, xt, m_pad, n_pad);
 }
 
 namespace {
@@ -558,6 +558,7 @@ namespace {
 // One CTA: 2 sum ln L[i][i] in FP64 (a fixed-order block reduction).
 __global__ void logdet_value_kernel(const double* __restrict__ L, int64_t ldl, int m,
                                     double penalty, double* __restrict__ value, int* st) {
+  pdl_begin(L, value, st);
   __shared__ double red[2 * kStatMax];
   double s = 0.0;
   bool bad = false;
@@ -576,6 +577,7 @@ __global__ void logdet_value_kernel(const double* __restrict__ L, int64_t ldl, i
 
 __global__ void argmin_p_kernel(const double* __restrict__ values, int p_max,
                                 int32_t* __restrict__ p_best) {
+  pdl_begin(values, p_best);
   int best = 0;
   for (int i = 1; i < p_max; ++i)
     if (values[i] < values[best]) best = i;
@@ -585,14 +587,12 @@ __global__ void argmin_p_kernel(const double* __restrict__ values, int p_max,
 }  // namespace
 
 void launch_logdet_value(const double* L, int64_t ldl, int m, double penalty, double* value,
-                         int* st, cudaStream_t s) {
-  note_launch();
-  logdet_value_kernel<<<1, kStatMax, 0, s>>>(L, ldl, m, penalty, value, st);
+                         int* st, Lane s) {
+  launch(logdet_value_kernel, 1, kStatMax, 0, s, L, ldl, m, penalty, value, st);
 }
 
-void launch_argmin_p(const double* values, int p_max, int32_t* p_best, cudaStream_t s) {
-  note_launch();
-  argmin_p_kernel<<<1, 1, 0, s>>>(values, p_max, p_best);
+void launch_argmin_p(const double* values, int p_max, int32_t* p_best, Lane s) {
+  launch(argmin_p_kernel, 1, 1, 0, s, values, p_max, p_best);
 }
 
 }  // namespace vl

@@ -80,6 +80,7 @@ static_assert(TG_SEG * TG_K * 3 * 128 * 128 < (1 << 24), "a level sum must stay 
 __global__ void slice_time_kernel(const float* __restrict__ Xc, int64_t ldc, int m, int n,
                                   int kp, const int* __restrict__ vexp,
                                   __nv_bfloat16* __restrict__ St, int64_t plane) {
+  pdl_begin(Xc, vexp, St);
   __shared__ float tile[32][33];
   const int s0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
@@ -105,6 +106,7 @@ __global__ void slice_time_kernel(const float* __restrict__ Xc, int64_t ldc, int
 __global__ void slice_beta_kernel(const float* __restrict__ beta, int m, int p, int kp,
                                   const int* __restrict__ vexp, __nv_bfloat16* __restrict__ Sb,
                                   int64_t plane, int* __restrict__ aexp) {
+  pdl_begin(beta, vexp, Sb, aexp);
   __shared__ unsigned long long red[32];
   const int i = blockIdx.x, K = p * kp;
   unsigned long long mx = 0;
@@ -135,6 +137,7 @@ __global__ void resid_apply_kernel(const double* __restrict__ X, int64_t ldx, in
                                    int p, const double* __restrict__ mu,
                                    const double* __restrict__ cst, const float2* __restrict__ part,
                                    const int* __restrict__ aexp, double* __restrict__ E) {
+  pdl_begin(X, mu, cst, part, aexp, E);
   const int i = blockIdx.y;
   const double off = mu[i] + cst[i];
   const double scale = bits::pow2(aexp[i] - 14);
@@ -205,6 +208,7 @@ __device__ __forceinline__ void tg_tile(int q, const TgParams& P, int& I, int& J
 __global__ void __launch_bounds__(TG_THREADS, 1)
     tcgram_kernel(const __grid_constant__ CUtensorMap mapA,
                   const __grid_constant__ CUtensorMap mapB, TgParams P) {
+  pdl_begin();
   extern __shared__ unsigned char tg_raw[];
   // 1024-byte aligned base for the swizzled tiles
   unsigned char* smem = tg_raw + ((1024 - (tc::smem_u32(tg_raw) & 1023)) & 1023);
@@ -448,6 +452,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
 __global__ void tg_reduce_sym_kernel(const float2* __restrict__ part, int splits, int N,
                                      const int* __restrict__ exps, double* __restrict__ C,
                                      int64_t ldc, double* __restrict__ w) {
+  pdl_begin(part, exps, C, w);
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)N * N) return;
   const int i = (int)(idx / N), j = (int)(idx % N);
@@ -545,11 +550,9 @@ bool launch_tcgram_sym(const Ctx& cx, const void* S, int N, int Kpad, int64_t ld
   splits = (P.nkb + P.kb_per_split - 1) / P.kb_per_split;
   P.part = reinterpret_cast<float2*>(cx.part);
   P.st = cx.st;
-  note_launch();
-  tcgram_kernel<<<dim3(tiles, splits), TG_THREADS, TG_SMEM, cx.s>>>(mA, mB, P);
-  note_launch();
-  tg_reduce_sym_kernel<<<(unsigned)((per + 255) / 256), 256, 0, cx.s>>>(P.part, splits, N, exps,
-                                                                       C, ldc, w);
+  launch(tcgram_kernel, dim3(tiles, splits), TG_THREADS, TG_SMEM, cx.s, mA, mB, P);
+  launch(tg_reduce_sym_kernel, (unsigned)((per + 255) / 256), 256, 0, cx.s, P.part, splits, N,
+         exps, C, ldc, w);
   return true;
 }
 
@@ -565,12 +568,10 @@ bool launch_tc_var_resid(const Ctx& cx, const float* Xc, int64_t ldc, const doub
   const int kp = (int)tg_kpad(m), n_eff = n - p, K = p * kp;
   const int64_t plane_t = (int64_t)n * kp, plane_b = (int64_t)m * K;
   if ((size_t)m * n_eff > cx.part_cap) return false;
-  note_launch();
-  slice_time_kernel<<<dim3((n + 31) / 32, kp / 32), dim3(32, 8), 0, cx.s>>>(
-      Xc, ldc, m, n, kp, vexp, static_cast<__nv_bfloat16*>(St), plane_t);
-  note_launch();
-  slice_beta_kernel<<<m, 256, 0, cx.s>>>(beta, m, p, kp, vexp, static_cast<__nv_bfloat16*>(Sb),
-                                          plane_b, aexp);
+  launch(slice_time_kernel, dim3((n + 31) / 32, kp / 32), dim3(32, 8), 0, cx.s, Xc, ldc, m, n, kp,
+         vexp, static_cast<__nv_bfloat16*>(St), plane_t);
+  launch(slice_beta_kernel, m, 256, 0, cx.s, beta, m, p, kp, vexp, static_cast<__nv_bfloat16*>(Sb),
+         plane_b, aexp);
   CUtensorMap mA, mB;
   if (!make_slice_map(&mA, Sb, K, m, K, plane_b, TG_M) ||
       !make_slice_map(&mB, St, kp, n, kp, plane_t, TG_N))
@@ -596,11 +597,9 @@ bool launch_tc_var_resid(const Ctx& cx, const float* Xc, int64_t ldc, const doub
   P.lag_p = p;
   P.part = reinterpret_cast<float2*>(cx.part);
   P.st = cx.st;
-  note_launch();
-  tcgram_kernel<<<dim3(tiles, 1), TG_THREADS, TG_SMEM, cx.s>>>(mA, mB, P);
-  note_launch();
-  resid_apply_kernel<<<dim3((n_eff + 255) / 256 < 16 ? (n_eff + 255) / 256 : 16, m), 256, 0,
-                       cx.s>>>(X, ldx, m, n_eff, p, mu, cst, P.part, aexp, E);
+  launch(tcgram_kernel, dim3(tiles, 1), TG_THREADS, TG_SMEM, cx.s, mA, mB, P);
+  launch(resid_apply_kernel, dim3((n_eff + 255) / 256 < 16 ? (n_eff + 255) / 256 : 16, m), 256, 0,
+         cx.s, X, ldx, m, n_eff, p, mu, cst, P.part, aexp, E);
   return true;
 }
 

@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(TTH) trsm_ring_kernel(const T* __restrict__ L,
                                                         const T* __restrict__ dinv, int n,
                                                         T* __restrict__ R, int64_t ldr, int nrhs,
                                                         int npass, int vec) {
+  pdl_begin();  // L and dinv are read by cp.async only; R is written here too
   constexpr int NS = Ring<T>::NS, LS = Ring<T>::LS;
   constexpr int EPC = 16 / sizeof(T);  // elements per 16-byte chunk
   extern __shared__ __align__(16) unsigned char trsm_ring_smem[];
@@ -280,7 +281,7 @@ size_t ring_smem(int n) {
 
 template <class T>
 bool launch_trsm_ring(const T* L, int64_t lda, const T* dinv, int n, T* R, int64_t ldr, int nrhs,
-                      bool backward, cudaStream_t s) {
+                      bool backward, Lane s) {
   if (n < 1 || n > TNMAX || nrhs < 1) return false;
   static bool attr = false;
   if (!attr) {
@@ -293,14 +294,13 @@ bool launch_trsm_ring(const T* L, int64_t lda, const T* dinv, int n, T* R, int64
   }
   const int vec = ((uintptr_t)L % 16 == 0) && ((uintptr_t)dinv % 16 == 0) &&
                   ((lda * (int64_t)sizeof(T)) % 16 == 0);
-  note_launch();
-  trsm_ring_kernel<T><<<(nrhs + TSC - 1) / TSC, TTH, ring_smem<T>(n), s>>>(
-      L, lda, dinv, n, R, ldr, nrhs, backward ? 2 : 1, vec);
+  launch(trsm_ring_kernel<T>, (nrhs + TSC - 1) / TSC, TTH, ring_smem<T>(n), s, L, lda, dinv, n, R,
+         ldr, nrhs, backward ? 2 : 1, vec);
   return true;
 }
 template bool launch_trsm_ring<float>(const float*, int64_t, const float*, int, float*, int64_t,
-                                      int, bool, cudaStream_t);
+                                      int, bool, Lane);
 template bool launch_trsm_ring<double>(const double*, int64_t, const double*, int, double*,
-                                       int64_t, int, bool, cudaStream_t);
+                                       int64_t, int, bool, Lane);
 
 }  // namespace vl
