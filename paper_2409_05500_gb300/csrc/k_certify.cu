@@ -304,11 +304,18 @@ __global__ void __launch_bounds__(RTH)
   if (threadIdx.x == 0) hx[i] = entropy_from_moments(sa / n - LN2, sb / n);
 }
 
-// 3b. Re-evaluation of the queued pairs, one warp per pair (a, b): rho =
-// mean(x_a x_b) of the standardized rows, the moments of both standardized
-// residuals u = (x_a - rho x_b) / sqrt(1 - rho^2) and v (roles swapped) in
-// double-float, their sums and entropies in FP64, and D_ab = -D_ba into the
-// cache D64.
+// 3b. Re-evaluation of the queued pairs (a, b): rho = mean(x_a x_b) of the
+// standardized rows, the moments of both standardized residuals u = (x_a -
+// rho x_b) / sqrt(1 - rho^2) and v (roles swapped) in double-float, their sums
+// and entropies in FP64, and D_ab = -D_ba into the cache D64.
+//
+// A lane's samples are one dependent chain, so few pairs of long series leave most
+// warps idle: G = 1, 2, 4 or 8 warps of a CTA share a pair, as many as the queue
+// leaves free, with at least PAIR_MIN samples a lane (the five sums over the warps
+// cost a pair about that much).  m = 120, n = 10000, three rounds: 122 us for 486
+// with one warp a pair; m = 100, n = 999: 8.9 us a round for 16.5 (PAIR_MIN = 16,
+// which leaves these at one warp: 19).
+constexpr int PAIR_MIN = 4;
 __global__ void __launch_bounds__(RTH)
     cert_pairs_kernel(const float2* __restrict__ xs, int m, int n, const int* ctrl,
                       const double* __restrict__ hx, const int2* __restrict__ pairs,
@@ -316,41 +323,60 @@ __global__ void __launch_bounds__(RTH)
                       int* __restrict__ stats) {
   pdl_begin(xs, ctrl, hx, pairs, D64, done, stats);
   __shared__ float2 tab[32];
+  __shared__ double part[5][RTH / 32];
   if (!ctrl[C_ACTIVE] || !ctrl[C_ANY]) return;
   if (threadIdx.x < 32) tab[threadIdx.x] = df::kExp2Frac[threadIdx.x];
   __syncthreads();
   const int np = ctrl[C_NPAIRS];
-  const int lane = threadIdx.x & 31;
-  const int nwarps = gridDim.x * (blockDim.x >> 5);
-  for (int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < np; w += nwarps) {
-    const int2 pr = pairs[w];
+  constexpr int WARPS = RTH / 32;
+  int G = 1;
+  while (G < WARPS && 2 * G * np <= (int)gridDim.x * WARPS && n >= 2 * G * 32 * PAIR_MIN) G *= 2;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g0 = wid & ~(G - 1);                         // first warp of the pair's
+  const int first = lane + 32 * (wid - g0), step = 32 * G;
+  // sums over the pair's warps, the same in each of them
+  auto over_warps = [&](double v, int k) {
+    v = warp_sum_d(v);
+    if (G == 1) return v;
+    if (lane == 0) part[k][wid] = v;
+    __syncthreads();
+    double t = part[k][g0];
+    for (int q = 1; q < G; ++q) t += part[k][g0 + q];
+    return t;
+  };
+  // every warp of a CTA goes round as often as its first pair does (barriers)
+  for (int w0 = blockIdx.x * (WARPS / G); w0 < np; w0 += gridDim.x * (WARPS / G)) {
+    const int w = w0 + wid / G;
+    const int2 pr = pairs[min(w, np - 1)];
     const int a = pr.x, b = pr.y;
     const float2* xa = xs + (int64_t)a * n;
     const float2* xb = xs + (int64_t)b * n;
+    const int len = w < np ? n : 0;
     df::F2 c{0.0f, 0.0f};
-    for (int t = lane; t < n; t += 32) {
+    for (int t = first; t < len; t += step) {
       const float2 p = xa[t], q = xb[t];
       c = df::add(c, df::mul(df::F2{p.x, p.y}, df::F2{q.x, q.y}));
     }
-    const double rho = warp_sum_d(df::to_double(c)) / n;
-    double dab = 0.0;
-    if (1.0 - rho * rho >= DEGENERATE_1MR2) {
-      const df::F2 r = df::from_double(rho);
-      const df::F2 sc = df::from_double(1.0 / sqrt(1.0 - rho * rho));
-      df::F2 au{0.0f, 0.0f}, bu{0.0f, 0.0f}, av{0.0f, 0.0f}, bv{0.0f, 0.0f};
-      for (int t = lane; t < n; t += 32) {
-        const float2 p = xa[t], q = xb[t];
-        const df::F2 fa{p.x, p.y}, fb{q.x, q.y};
-        moments_df(df::mul(sc, df::add(fa, df::neg(df::mul(r, fb)))), au, bu, tab);
-        moments_df(df::mul(sc, df::add(fb, df::neg(df::mul(r, fa)))), av, bv, tab);
-      }
-      const double sau = warp_sum_d(df::to_double(au)), sbu = warp_sum_d(df::to_double(bu));
-      const double sav = warp_sum_d(df::to_double(av)), sbv = warp_sum_d(df::to_double(bv));
-      const double hab = entropy_from_moments(sau / n - LN2, sbu / n);  // H(r_{a<-b})
-      const double hba = entropy_from_moments(sav / n - LN2, sbv / n);  // H(r_{b<-a})
-      dab = hx[b] + hab - hx[a] - hba;
+    const double rho = over_warps(df::to_double(c), 0) / n;
+    const bool good = 1.0 - rho * rho >= DEGENERATE_1MR2;
+    const df::F2 r = df::from_double(rho);
+    const df::F2 sc = df::from_double(good ? 1.0 / sqrt(1.0 - rho * rho) : 0.0);
+    df::F2 au{0.0f, 0.0f}, bu{0.0f, 0.0f}, av{0.0f, 0.0f}, bv{0.0f, 0.0f};
+    for (int t = first; t < (good ? len : 0); t += step) {
+      const float2 p = xa[t], q = xb[t];
+      const df::F2 fa{p.x, p.y}, fb{q.x, q.y};
+      moments_df(df::mul(sc, df::add(fa, df::neg(df::mul(r, fb)))), au, bu, tab);
+      moments_df(df::mul(sc, df::add(fb, df::neg(df::mul(r, fa)))), av, bv, tab);
     }
-    if (lane == 0) {
+    const double sau = over_warps(df::to_double(au), 1), sbu = over_warps(df::to_double(bu), 2);
+    const double sav = over_warps(df::to_double(av), 3), sbv = over_warps(df::to_double(bv), 4);
+    if (first == 0 && w < np) {
+      double dab = 0.0;
+      if (good) {
+        const double hab = entropy_from_moments(sau / n - LN2, sbu / n);  // H(r_{a<-b})
+        const double hba = entropy_from_moments(sav / n - LN2, sbv / n);  // H(r_{b<-a})
+        dab = hx[b] + hab - hx[a] - hba;
+      }
       D64[(int64_t)a * m + b] = dab;
       D64[(int64_t)b * m + a] = -dab;
       const int64_t bit = (int64_t)a * m + b;

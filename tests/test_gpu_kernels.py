@@ -166,3 +166,33 @@ def test_var_fit_with_different_window_means(vl, h, prec, m, n, p):
     want = beta.reshape(p, m, m).transpose(0, 2, 1)
     tol = 1e-9 if prec == "fp64" else 1e-5
     assert np.abs(M.cpu().numpy() - want).max() <= tol
+
+
+# the re-evaluated pairs of a certified ordering by one warp, two, four and eight:
+# series just below and at the lengths where their number changes, odd ones among
+# them.  The planted near tie is decided as by the exact measure, nothing left open.
+@pytest.mark.parametrize("n", [121, 255, 256, 511, 512, 1023, 1024, 3001])
+def test_certified_pairs_at_the_lengths_of_their_splits(vl, h, n):
+    from test_gpu_parity import _planted_near_tie
+    for seed in range(50):  # a tie whose planting swaps the two picks alone
+        rng = np.random.default_rng(1000 * n + seed)
+        E = rng.laplace(size=(12, n))
+        for i in range(1, 12):
+            E[i] += 0.6 * E[(i * 7) % i] + 0.4 * E[i - 1]
+        D = np.asarray(oracle.pairwise_measure(oracle.standardize(E))["D"])
+        od = oracle.order_heuristic(D)
+        ref = [int(c) for c in od["order"]]
+        Dp, k, a, b = _planted_near_tie(D, od["order"], od["steps"])
+        swapped = ref[:k] + [b, a] + ref[k + 2:]
+        if [int(c) for c in oracle.order_heuristic(Dp)["order"]] == swapped:
+            break
+    else:
+        pytest.fail("no such series")
+    order = torch.empty(12, dtype=torch.int32, device="cuda")
+    stats = torch.zeros(4, dtype=torch.int32, device="cuda")
+    vl.vl_causal_order_certified(h, torch.from_numpy(Dp).cuda(), torch.from_numpy(E).cuda(), order,
+                                 None, stats)
+    h.sync()
+    assert [int(c) for c in order.cpu().numpy()] == ref
+    st = [int(v) for v in stats.cpu().numpy()]
+    assert st[1] >= 1 and st[2] >= 1 and st[3] == 0, st
