@@ -491,7 +491,8 @@ extern "C" vl_status vl_causal_order_noalloc(void* cuda_stream, const double* D,
   // an error the caller left pending is not this call's: report only an
   // error that the launches below raise (and clear only that one)
   const cudaError_t before = cudaPeekAtLastError();
-  launch_causal_order(D, m, scratch, order, gap, nullptr, static_cast<cudaStream_t>(cuda_stream));
+  launch_causal_order(D, m, scratch, order, gap, nullptr,
+                      Lane(static_cast<cudaStream_t>(cuda_stream)));
   const cudaError_t after = cudaPeekAtLastError();
   if (after == cudaSuccess || after == before) return VL_OK;
   cudaGetLastError();

@@ -103,11 +103,12 @@ namespace vl {
 // before it runs (programmatic dependent launch, see pdl_begin).  A lane that
 // shares the GPU with others must not: the CTAs that wait there hold shared
 // memory, registers and thread slots that the other lanes' kernels could use
-// (32 concurrent streams of fits of mixed sizes: 15.6 ms without, 23.6 with).
+// (32 concurrent streams of fits of mixed sizes: 15.6 ms without, 23.6 with).  For
+// the same reason it is for calls of small kernels only.
 struct Lane {
   cudaStream_t s;
   bool overlap;
-  Lane(cudaStream_t stream, bool alone = true) : s(stream), overlap(alone) {}
+  Lane(cudaStream_t stream, bool over = false) : s(stream), overlap(over) {}
   operator cudaStream_t() const { return s; }
 };
 
@@ -120,8 +121,7 @@ void note_launch();
 // the next kernel of the stream be set up as soon as all of this one's CTAs are
 // resident, and waits until the kernels before it have completed and their writes
 // are visible.  Measured, without and with: a fit of m = 10 188 -> 120 us, the
-// measure of the same size 44 -> 30, 99 search steps 6.1 -> 5.3 ms, a fit of
-// m = 400 858 -> 820 us.
+// measure of m = 50 44 -> 30, 99 search steps of m = 100 6.1 -> 5.3 ms.
 // pdl_wait() alone, in long kernels of few CTAs (Cholesky, the cluster search):
 // the next kernel's CTAs waiting on the other SMs made these slower (fit_b at
 // m = 400: 208 us without any of this, 224 with pdl_begin, 206 with pdl_wait).
