@@ -675,15 +675,8 @@ bool launch_chol_cluster(float* A, int64_t lda, int n, float* dinv, const double
   const int nblk = (n + CB - 1) / CB;
   if (nblk > 3 && scratch_floats(nblk) > scratch_cap) return false;
   const Shape h = cluster_shape(n);
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)cluster_shape(CL_NMAX).smem) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    attr = true;
-  }
+  static SmemOptIn smem;
+  if (!smem.allow(chol_cluster_kernel, cluster_shape(CL_NMAX).smem)) return false;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(h.cl, 1, 1);
   cfg.blockDim = dim3(CTH, 1, 1);

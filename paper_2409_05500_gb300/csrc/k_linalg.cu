@@ -910,25 +910,16 @@ void chol_blocked(const Ctx& cx, T* A, int64_t lda, int n, T* dinv, double* diag
       if (launch_chol_cluster(A, lda, n, dinv, diag0, (float)rel_tol,
                               reinterpret_cast<float*>(cx.part), 2 * cx.part_cap, cx.st, s))
         return;
-      const size_t smem1 = chol_single_smem(SINGLE_MAX);
-      static bool attr1 = false;
-      if (!attr1) {
-        cudaFuncSetAttribute(chol_single_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem1);
-        attr1 = true;
-      }
+      static SmemOptIn single;
+      single.allow(chol_single_kernel, chol_single_smem(SINGLE_MAX));
       launch(chol_single_kernel, 1, STH, chol_single_smem(n), s, A, lda, n, dinv, diag0,
              (float)rel_tol, cx.st);
       return;
     }
   }
   const size_t smem = CHOL_NB * CROW * sizeof(T);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(chol_diag_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    attr_set = true;
-  }
+  static SmemOptIn diag;
+  diag.allow(chol_diag_kernel<T>, smem);
   for (int k0 = 0; k0 < n; k0 += NB) {
     const int nb = std::min(NB, n - k0);
     T* dblk = dinv + (int64_t)(k0 / NB) * NB * NB;
@@ -955,12 +946,8 @@ void chol_solve_blocked(const Ctx& cx, const T* L, int64_t lda, const T* dinv, i
                         int64_t ldr, int nrhs, bool backward) {
   if (launch_trsm_ring<T>(L, lda, dinv, n, R, ldr, nrhs, backward, cx.s)) return;
   const size_t smem = trsm_smem_bytes<T>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(trsm_cols_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    attr_set = true;
-  }
+  static SmemOptIn cols;
+  cols.allow(trsm_cols_kernel<T>, smem);
   launch(trsm_cols_kernel<T>, (nrhs + SC - 1) / SC, NTH, smem, cx.s, L, lda, dinv, n, R, ldr, nrhs,
          backward ? 1 : 0);
 }

@@ -243,16 +243,8 @@ __global__ void __launch_bounds__(OC_TH) order_cluster_kernel(const float2* __re
 template <int NW>
 bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, float2* spick,
                           Lane s) {
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(order_cluster_kernel<NW>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)oc_smem(OC_MAX_M)) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    attr = true;
-  }
+  static SmemOptIn smem;
+  if (!smem.allow(order_cluster_kernel<NW>, oc_smem(OC_MAX_M))) return false;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(OC_CTAS, 1, 1);
   cfg.blockDim = dim3(OC_TH, 1, 1);
@@ -278,12 +270,8 @@ bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, float2* spick
 
 template <int NW>
 void launch_order_local(const OrderWs& w, int m, int32_t* order, float2* spick, Lane s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(order_local_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         OL_MAX_M * OL_MAX_M * (int)sizeof(float2));
-    attr = true;
-  }
+  static SmemOptIn smem;
+  smem.allow(order_local_kernel<NW>, OL_MAX_M * OL_MAX_M * sizeof(float2));
   launch(order_local_kernel<NW>, 1, OC_TH, (size_t)m * m * sizeof(float2), s, w.pt, w.sh, w.sl, m,
          order, spick);
 }

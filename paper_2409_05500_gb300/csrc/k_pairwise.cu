@@ -603,12 +603,8 @@ void launch_pairwise_f32_cfg(const float* xt, const PairPlan& pl, const float* r
   const int n_run = ((pl.n + KRUN - 1) / KRUN) * KRUN;
   dim3 grid(pl.tiles, pl.splits);
   const size_t smem = sizeof(float) * 3 * TTS * 2 * TB;  // three stages of TTS x 64 samples
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(pairwise_f32_kernel<MTI, TTS, MINB>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr_set = true;
-  }
+  static SmemOptIn opt;
+  opt.allow(pairwise_f32_kernel<MTI, TTS, MINB>, smem);
   launch(pairwise_f32_kernel<MTI, TTS, MINB>, grid, TB / MTI * 16, smem, s, xt, pl.m, pl.m_pad,
          pl.m_pad / TB, n_run, pl.t_per_split, rho32, c32, part);
 }
@@ -637,12 +633,8 @@ void launch_pairwise_f32_list(const PairJob* jobs, const int4* items, int nitems
                               Lane s) {
   constexpr int MTI = F32_MTI, TTS = F32_TTS, MINB = F32_MINB;
   const size_t smem = sizeof(float) * 3 * TTS * 2 * TB;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(pairwise_f32_list_kernel<MTI, TTS, MINB>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr_set = true;
-  }
+  static SmemOptIn opt;
+  opt.allow(pairwise_f32_list_kernel<MTI, TTS, MINB>, smem);
   launch(pairwise_f32_list_kernel<MTI, TTS, MINB>, std::max(1, std::min(grid, nitems)), TB / MTI *
          16, smem, s, jobs, items, nitems);
 }

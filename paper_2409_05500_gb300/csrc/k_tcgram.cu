@@ -525,15 +525,8 @@ bool launch_tcgram_sym(const Ctx& cx, const void* S, int N, int Kpad, int64_t ld
   if (!make_slice_map(&mA, S, Kpad, N, ldo, plane, TG_M) ||
       !make_slice_map(&mB, S, Kpad, N, ldo, plane, TG_N))
     return false;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(tcgram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)TG_SMEM) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    attr = true;
-  }
+  static SmemOptIn smem;
+  if (!smem.allow(tcgram_kernel, TG_SMEM)) return false;
   TgParams P{};
   P.M = P.N = N;
   P.sym = 1;
@@ -576,15 +569,8 @@ bool launch_tc_var_resid(const Ctx& cx, const float* Xc, int64_t ldc, const doub
   if (!make_slice_map(&mA, Sb, K, m, K, plane_b, TG_M) ||
       !make_slice_map(&mB, St, kp, n, kp, plane_t, TG_N))
     return false;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(tcgram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)TG_SMEM) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    attr = true;
-  }
+  static SmemOptIn smem;
+  if (!smem.allow(tcgram_kernel, TG_SMEM)) return false;
   TgParams P{};
   P.M = m;
   P.N = n_eff;

@@ -283,15 +283,8 @@ template <class T>
 bool launch_trsm_ring(const T* L, int64_t lda, const T* dinv, int n, T* R, int64_t ldr, int nrhs,
                       bool backward, Lane s) {
   if (n < 1 || n > TNMAX || nrhs < 1) return false;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(trsm_ring_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)ring_smem<T>(TNMAX)) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    attr = true;
-  }
+  static SmemOptIn smem;
+  if (!smem.allow(trsm_ring_kernel<T>, ring_smem<T>(TNMAX))) return false;
   const int vec = ((uintptr_t)L % 16 == 0) && ((uintptr_t)dinv % 16 == 0) &&
                   ((lda * (int64_t)sizeof(T)) % 16 == 0);
   launch(trsm_ring_kernel<T>, (nrhs + TSC - 1) / TSC, TTH, ring_smem<T>(n), s, L, lda, dinv, n, R,

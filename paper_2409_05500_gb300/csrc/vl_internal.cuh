@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -167,6 +168,30 @@ inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, con
   note_launch();
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
+
+// Dynamic shared memory beyond 48 KB: a kernel has to be allowed it on every
+// device that launches it.  One of these per kernel (static, for any thread)
+// remembers the devices on which that is done, the first 64 of them; false if the
+// runtime refuses.
+class SmemOptIn {
+  std::atomic<uint64_t> done{0};
+
+ public:
+  template <class... P>
+  bool allow(void (*kernel)(P...), size_t bytes) {
+    int dev = 0;
+    bool ok = cudaGetDevice(&dev) == cudaSuccess;
+    const uint64_t bit = dev >= 0 && dev < 64 ? uint64_t(1) << dev : 0;
+    if (ok && (done.load(std::memory_order_relaxed) & bit)) return true;
+    ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)bytes) == cudaSuccess;
+    if (ok)
+      done.fetch_or(bit, std::memory_order_relaxed);
+    else
+      cudaGetLastError();
+    return ok;
+  }
+};
 
 // What every launcher needs: the stream, the sticky status word, the split-K
 // scratch of the handle (FP64 partial products) and the SM count.

@@ -1,0 +1,59 @@
+// The library's host side on the stand-in runtime (fake_cuda.cpp): prints what
+// went wrong, one line each.
+#include <varlingam_gb300.h>
+
+#include <cstdio>
+#include <cstring>
+
+#include "fake_cuda.h"
+
+#include <cuda_runtime_api.h>
+
+namespace {
+
+double* const X = reinterpret_cast<double*>(uintptr_t(1) << 44);  // never read
+int32_t* const ORDER = reinterpret_cast<int32_t*>(uintptr_t(1) << 45);
+
+void report(const char* call, int device, int m, vl_status s) {
+  for (const fake::Launch& l : fake::launches)
+    if (l.refused)
+      std::printf("%s m=%d device %d: refused %s with %zu bytes\n", call, m, device,
+                  l.name.c_str(), l.smem);
+  if (s != VL_OK) std::printf("%s m=%d device %d: status %d\n", call, m, device, (int)s);
+  fake::launches.clear();
+}
+
+// Every call on the first device, then on the second.
+void two_devices() {
+  for (int d = 0; d < 2; ++d) {
+    cudaSetDevice(d);
+    vl_handle h;
+    if (vl_create(&h, d, nullptr, 0) != VL_OK) std::printf("vl_create\n");
+    for (int m : {20, 40, 64, 78, 79, 100, 160, 161, 300, 448, 449, 512, 600}) {
+      const int n = 3 * m + 50;
+      report("vl_causal_order", d, m, vl_causal_order(h, X, m, ORDER, X));
+      report("vl_causal_order_certified", d, m,
+             vl_causal_order_certified(h, X, X, n, m, n, ORDER, X, nullptr));
+      if (m <= VL_NOALLOC_MAX_M)
+        report("vl_causal_order_noalloc", d, m,
+               vl_causal_order_noalloc(nullptr, X, m, ORDER, X));
+      for (vl_precision prec : {VL_PREC_MIXED, VL_PREC_FP64}) {
+        report("vl_pairwise_measure", d, m,
+               vl_pairwise_measure(h, X, n, m, n, prec, X, X, X));
+        report("vl_var_fit", d, m, vl_var_fit(h, X, n, m, n, 2, prec, X, X));
+        report("vl_fit_b", d, m, vl_fit_b(h, X, n, m, n, ORDER, X, 1, prec, X, X));
+      }
+      vl_instance I[2] = {{X, n, m, n, 1, ORDER, X, X, X, X}, {X, n, m, n, 1, ORDER, X, X, X, X}};
+      vl_status st[2];
+      report("vl_fit_batched", d, m, vl_fit_batched(h, I, 2, VL_PREC_MIXED, st));
+    }
+    vl_destroy(h);
+  }
+}
+
+}  // namespace
+
+int main(int argc, char** argv) {
+  if (argc == 2 && !std::strcmp(argv[1], "two_devices")) two_devices();
+  return 0;
+}
