@@ -409,11 +409,18 @@ vl_status fit_b_impl(Exec& x, const double* E, int64_t lde, int m, int n,
   return check_launch(x.h, "vl_fit_b");
 }
 
+// The search was not launched: whatever would follow must not use the order.
+vl_status not_launched(vl_handle h, const char* what) {
+  const vl_status s = check_launch(h, what);
+  return s != VL_OK ? s : fail(h, VL_ERR_CUDA, std::string(what) + ": search not launched");
+}
+
 vl_status order_impl(Exec& x, const double* D, int m, int32_t* order, double* gap) {
   char* ows;
   vl_status s = with_workspace(x, [&](Arena& a) { ows = a.take<char>(order_ws_bytes(m)); });
   if (s != VL_OK || x.measure) return s;
-  launch_causal_order(D, m, ows, order, gap, x.st, x.s);
+  if (!launch_causal_order(D, m, ows, order, gap, x.st, x.s))
+    return not_launched(x.h, "vl_causal_order");
   return check_launch(x.h, "vl_causal_order");
 }
 
@@ -427,7 +434,8 @@ vl_status order_certified_impl(Exec& x, const double* D, const double* E, int64_
     cws = a.take<char>(certify_ws_bytes(m, n));
   });
   if (s != VL_OK || x.measure) return s;
-  launch_causal_order(D, m, ows, order, nullptr, x.st, x.s, certify_spick(cws, m));
+  if (!launch_causal_order(D, m, ows, order, nullptr, x.st, x.s, certify_spick(cws, m)))
+    return not_launched(x.h, "vl_causal_order_certified");
   launch_certify(D, E, lde, m, n, ows, cws, order, stats, x.h->num_sms, x.s);
   if (gap) launch_order_gaps(ows, m, order, gap, x.s);
   return check_launch(x.h, "vl_causal_order_certified");

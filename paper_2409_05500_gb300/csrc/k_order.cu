@@ -268,12 +268,17 @@ bool launch_order_cluster(const OrderWs& w, int m, int32_t* order, float2* spick
   return true;
 }
 
+// Launch the search in one CTA's shared memory; false as above.
 template <int NW>
-void launch_order_local(const OrderWs& w, int m, int32_t* order, float2* spick, Lane s) {
+bool launch_order_local(const OrderWs& w, int m, int32_t* order, float2* spick, Lane s) {
   static SmemOptIn smem;
-  smem.allow(order_local_kernel<NW>, OL_MAX_M * OL_MAX_M * sizeof(float2));
-  launch(order_local_kernel<NW>, 1, OC_TH, (size_t)m * m * sizeof(float2), s, w.pt, w.sh, w.sl, m,
-         order, spick);
+  if (!smem.allow(order_local_kernel<NW>, OL_MAX_M * OL_MAX_M * sizeof(float2))) return false;
+  if (launch(order_local_kernel<NW>, 1, OC_TH, (size_t)m * m * sizeof(float2), s, w.pt, w.sh, w.sl,
+             m, order, spick) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return true;
 }
 
 // Gaps after the search, from the order: variable i replays its score S_i =
@@ -395,35 +400,36 @@ size_t order_ws_bytes(int m) {
          (size_t)m * sizeof(float4) + 1024;
 }
 
-void launch_causal_order(const double* D, int m, void* ws, int32_t* order, double* gap, int* st,
+bool launch_causal_order(const double* D, int m, void* ws, int32_t* order, double* gap, int* st,
                          Lane s, float2* spick) {
   const OrderWs w = order_ws_layout(ws, m);
   dim3 grid((m + 31) / 32, (m + 31) / 32), block(32, 8);
   launch(pt_kernel, grid, block, 0, s, D, m, w.pt, st);
   launch(rowsum_kernel, (m + 7) / 8, 256, 0, s, D, m, w.sh, w.sl);
-  const bool cluster = m > OL_MAX_M && m <= OC_MAX_M &&
-                       (m <= 256 ? launch_order_cluster<8>(w, m, order, spick, s)
-                                 : launch_order_cluster<16>(w, m, order, spick, s));
-  if (m <= 32) {
-    launch_order_local<1>(w, m, order, spick, s);
-  } else if (m <= 64) {
-    launch_order_local<2>(w, m, order, spick, s);
-  } else if (m <= 128) {
-    launch_order_local<4>(w, m, order, spick, s);
-  } else if (m <= OL_MAX_M) {
-    launch_order_local<8>(w, m, order, spick, s);
-  } else if (!cluster) {
+  bool done = false;
+  if (m <= 32)
+    done = launch_order_local<1>(w, m, order, spick, s);
+  else if (m <= 64)
+    done = launch_order_local<2>(w, m, order, spick, s);
+  else if (m <= 128)
+    done = launch_order_local<4>(w, m, order, spick, s);
+  else if (m <= OL_MAX_M)
+    done = launch_order_local<8>(w, m, order, spick, s);
+  else if (m <= 256)
+    done = launch_order_cluster<8>(w, m, order, spick, s);
+  else if (m <= OC_MAX_M)
+    done = launch_order_cluster<16>(w, m, order, spick, s);
+  if (!done) {
     const Lane alone(s, false);  // order_kernel has no pdl_wait: 1.5 us of 250 or more
-    if (m <= 2 * STH)
-      launch(order_kernel<2>, 1, STH, 0, alone, w.pt, w.sh, w.sl, m, order, spick);
-    else if (m <= 4 * STH)
-      launch(order_kernel<4>, 1, STH, 0, alone, w.pt, w.sh, w.sl, m, order, spick);
-    else if (m <= 8 * STH)
-      launch(order_kernel<8>, 1, STH, 0, alone, w.pt, w.sh, w.sl, m, order, spick);
-    else
-      launch(order_kernel<16>, 1, STH, 0, alone, w.pt, w.sh, w.sl, m, order, spick);
+    const auto search = m <= 2 * STH   ? order_kernel<2>
+                        : m <= 4 * STH ? order_kernel<4>
+                        : m <= 8 * STH ? order_kernel<8>
+                                       : order_kernel<16>;
+    if (launch(search, 1, STH, 0, alone, w.pt, w.sh, w.sl, m, order, spick) != cudaSuccess)
+      return false;
   }
   if (gap) launch_order_gaps(ws, m, order, gap, s);
+  return true;
 }
 
 }  // namespace vl
@@ -479,10 +485,10 @@ extern "C" vl_status vl_causal_order_noalloc(void* cuda_stream, const double* D,
   // an error the caller left pending is not this call's: report only an
   // error that the launches below raise (and clear only that one)
   const cudaError_t before = cudaPeekAtLastError();
-  launch_causal_order(D, m, scratch, order, gap, nullptr,
-                      Lane(static_cast<cudaStream_t>(cuda_stream)));
+  const bool launched = launch_causal_order(D, m, scratch, order, gap, nullptr,
+                                            Lane(static_cast<cudaStream_t>(cuda_stream)));
   const cudaError_t after = cudaPeekAtLastError();
-  if (after == cudaSuccess || after == before) return VL_OK;
+  if (launched && (after == cudaSuccess || after == before)) return VL_OK;
   cudaGetLastError();
   return VL_ERR_CUDA;
 }

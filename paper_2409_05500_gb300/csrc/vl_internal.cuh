@@ -155,8 +155,8 @@ inline cudaLaunchAttribute pdl_attribute() {
   return a;
 }
 template <class... P, class... A>
-inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, const Lane& s,
-                   A&&... args) {
+inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, const Lane& s,
+                          A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -166,7 +166,7 @@ inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, con
   cfg.attrs = at;
   cfg.numAttrs = s.overlap ? 1 : 0;
   note_launch();
-  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 // Dynamic shared memory beyond 48 KB: a kernel has to be allowed it on every
@@ -365,7 +365,9 @@ size_t order_ws_bytes(int m);
 void launch_order_gaps(void* ws, int m, const int32_t* order, double* gap, Lane s);
 // spick (optional): the winning score of every step as a double-float pair,
 // for the certification of near ties (k_certify.cu).
-void launch_causal_order(const double* D, int m, void* ws, int32_t* order, double* gap, int* st,
+// False if no search could be launched: `order` is then not written, and must not
+// be used as an index by a later launch (check_launch has the error).
+bool launch_causal_order(const double* D, int m, void* ws, int32_t* order, double* gap, int* st,
                          Lane s, float2* spick = nullptr);
 
 // Tensor-core exact-slice Gram products (k_tcgram.cu).  Operands are three

@@ -51,9 +51,41 @@ void two_devices() {
   }
 }
 
+// A search that cannot be launched: another takes its place; without any, the
+// call fails and nothing that would use the order as an index is launched.
+void no_search() {
+  vl_handle h;
+  if (vl_create(&h, 0, nullptr, 0) != VL_OK) std::printf("vl_create\n");
+  for (int m : {50, 160, 300}) {
+    const int n = 3 * m + 50;
+    const vl_instance I{X, n, m, n, 1, ORDER, X, X, X, X};
+    fake::refuse = {"order_local_kernel", "order_cluster_kernel"};
+    vl_status s = vl_causal_order(h, X, m, ORDER, X);
+    if (s != VL_OK || !fake::launched("order_kernel")) std::printf("m=%d: no other search\n", m);
+    s = vl_causal_order_noalloc(nullptr, X, m, ORDER, X);
+    if (s != VL_OK) std::printf("m=%d: no other search without allocation\n", m);
+    fake::refuse.push_back("order_kernel");
+    for (int call = 0; call < 5; ++call) {
+      fake::launches.clear();
+      vl_status st = VL_OK;
+      if (call == 0) s = vl_causal_order(h, X, m, ORDER, X);
+      if (call == 1) s = vl_causal_order_noalloc(nullptr, X, m, ORDER, X);
+      if (call == 2) s = vl_causal_order_certified(h, X, X, n, m, n, ORDER, X, nullptr);
+      if (call == 3) s = vl_fit(h, X, n, m, n, 1, VL_PREC_MIXED, X, ORDER, X, X, X);
+      if (call == 4) s = vl_fit_batched(h, &I, 1, VL_PREC_MIXED_CERTIFIED, &st);
+      if (s != VL_ERR_CUDA) std::printf("m=%d call %d: status %d\n", m, call, (int)s);
+      for (const char* k : {"gap_scores_kernel", "cert_", "permute_cov_kernel"})
+        if (fake::launched(k)) std::printf("m=%d call %d: %s without an order\n", m, call, k);
+    }
+    fake::refuse.clear();
+  }
+  vl_destroy(h);
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
   if (argc == 2 && !std::strcmp(argv[1], "two_devices")) two_devices();
+  if (argc == 2 && !std::strcmp(argv[1], "no_search")) no_search();
   return 0;
 }

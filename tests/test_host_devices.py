@@ -1,7 +1,8 @@
 """The library's host side without a GPU: its objects linked with a stand-in for
 the CUDA runtime (tests/c/fake_cuda) that keeps, for every device, how much
 dynamic shared memory a kernel may use there, and refuses launches beyond it.
-Every call runs on two devices of one process, one after the other."""
+Every call runs on two devices of one process, one after the other, and with
+searches whose launch fails."""
 import glob
 import importlib.util
 import os
@@ -34,7 +35,7 @@ def host_check(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("what", ["two_devices"])
+@pytest.mark.parametrize("what", ["two_devices", "no_search"])
 def test_host_side(host_check, what):
     out = subprocess.run([host_check, what], check=True, capture_output=True, text=True).stdout
     assert out == ""
