@@ -271,7 +271,9 @@ __device__ __forceinline__ void kahan_f(float& S, float& C, float x) {
 
 // Mean, then 1/std (0 for a constant row) of row e; each(d) sees every centred
 // value between the two.  Sets the status word for rows that are not finite or
-// constant and goes on (a row that is not finite leaves NaN everywhere).
+// constant and goes on (a row that is not finite leaves NaN everywhere).  The mean
+// is the sum in block_sum's order, divided: n copies of a number with an exact sum
+// have that number as their mean, and a variance of exactly 0.
 template <class Each>
 __device__ __forceinline__ void row_stats(const double* __restrict__ e, int n, double inv_n,
                                           double* red, int* st, double& mu, double& isd,
@@ -285,7 +287,7 @@ __device__ __forceinline__ void row_stats(const double* __restrict__ e, int n, d
     s += v;
   }
   if (__syncthreads_or(!finite) && threadIdx.x == 0) set_status(st, VL_ERR_NONFINITE);
-  mu = block_fold(s, red, [inv_n](double t) { return t * inv_n; });
+  mu = block_sum(s, red, [n, inv_n](double t) { return div_by(t, n, inv_n); });
   double q = 0.0;
 #pragma unroll 4
   for (int t = threadIdx.x; t < n; t += kStatMax) {
