@@ -137,7 +137,7 @@ __global__ void resid_apply_kernel(const double* __restrict__ X, int64_t ldx, in
                                    int p, const double* __restrict__ mu,
                                    const double* __restrict__ cst, const float2* __restrict__ part,
                                    const int* __restrict__ aexp, double* __restrict__ E) {
-  pdl_begin(X, mu, cst, part, aexp, E);
+  pdl_wait(X, mu, cst, part, aexp, E);
   const int i = blockIdx.y;
   const double off = mu[i] + cst[i];
   const double scale = bits::pow2(aexp[i] - 14);
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1)
 __global__ void tg_reduce_sym_kernel(const float2* __restrict__ part, int splits, int N,
                                      const int* __restrict__ exps, double* __restrict__ C,
                                      int64_t ldc, double* __restrict__ w) {
-  pdl_begin(part, exps, C, w);
+  pdl_wait(part, exps, C, w);
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)N * N) return;
   const int i = (int)(idx / N), j = (int)(idx % N);

@@ -125,7 +125,12 @@ void note_launch();
 // measure of m = 50 44 -> 30, 99 search steps of m = 100 6.1 -> 5.3 ms.
 // pdl_wait() alone, in long kernels of few CTAs (Cholesky, the cluster search):
 // the next kernel's CTAs waiting on the other SMs made these slower (fit_b at
-// m = 400: 208 us without any of this, 224 with pdl_begin, 206 with pdl_wait).
+// m = 400: 208 us without any of this, 224 with pdl_begin, 206 with pdl_wait), and
+// in the pairwise kernel for the same reason.  Also in the last kernel of each
+// tensor-core product: a kernel that releases before its own wait lets launches run
+// ahead by several kernels, whose CTAs then decide where the others find room
+// (VAR fit of m = 20, n = 13000, p = 3 164 us without any of this, 260 with
+// pdl_begin there, 132 so; m = 30, n = 5000, p = 1 108, 111 and 74).
 // Every kernel given to launch() on an overlapping lane MUST call one of the two
 // before it touches global memory, with every pointer parameter that it reads
 // but does not write: a load through a const __restrict__ parameter counts as
