@@ -41,12 +41,12 @@ cudaError_t set(cudaError_t e) {
   return e;
 }
 
-cudaError_t do_launch(const void* func, size_t smem) {
+cudaError_t do_launch(const void* func, size_t smem, bool overlap = false) {
   const std::string& name = names()[func];
   const auto a = allowed.find({device, func});
   bool refused = smem > (a == allowed.end() ? SMEM_DEFAULT : a->second);
   for (const std::string& r : fake::refuse) refused |= name.find(r) != std::string::npos;
-  fake::launches.push_back({name, device, smem, refused});
+  fake::launches.push_back({name, device, smem, overlap, refused});
   return set(refused ? cudaErrorInvalidValue : cudaSuccess);
 }
 
@@ -90,7 +90,11 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t smem, 
   return do_launch(reinterpret_cast<const void*>(k), smem);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* func, void**) {
-  return do_launch(func, c->dynamicSmemBytes);
+  bool overlap = false;
+  for (unsigned k = 0; k < c->numAttrs; ++k)
+    overlap |= c->attrs[k].id == cudaLaunchAttributeProgrammaticStreamSerialization &&
+               c->attrs[k].val.programmaticStreamSerializationAllowed;
+  return do_launch(func, c->dynamicSmemBytes, overlap);
 }
 cudaError_t cudaFuncSetAttribute(const void* func, cudaFuncAttribute a, int v) {
   if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {

@@ -12,6 +12,7 @@ struct Launch {
   std::string name;  // mangled
   int device;
   size_t smem;
+  bool overlap;  // may be set up while its predecessor runs
   bool refused;
 };
 extern std::vector<Launch> launches;

@@ -82,10 +82,45 @@ void no_search() {
   vl_destroy(h);
 }
 
+// Which calls' launches overlap: mixed ones up to m n = 2^18, FP64 ones up to
+// m^2 n = 2^20, never a batch's.
+void overlap() {
+  vl_handle h;
+  if (vl_create(&h, 0, nullptr, 0) != VL_OK) std::printf("vl_create\n");
+  const struct {
+    int m, n;
+    bool mixed, fp64;
+  } sizes[] = {{10, 1000, true, true},   {16, 4096, true, true},  {16, 4097, true, false},
+               {50, 1000, true, false},  {64, 4096, true, false}, {64, 4097, false, false},
+               {100, 2600, true, false}, {400, 2500, false, false}};
+  for (const auto& z : sizes)
+    for (vl_precision prec : {VL_PREC_MIXED, VL_PREC_FP64}) {
+      const bool want = prec == VL_PREC_MIXED ? z.mixed : z.fp64;
+      for (int call = 0; call < 7; ++call) {
+        const vl_instance I{X, z.n, z.m, z.n, 1, ORDER, X, X, X, X};
+        vl_status st;
+        fake::launches.clear();
+        if (call == 0) vl_var_fit(h, X, z.n, z.m, z.n, 1, prec, X, X);
+        if (call == 1) vl_pairwise_measure(h, X, z.n, z.m, z.n, prec, X, X, X);
+        if (call == 2) vl_causal_order_standard(h, X, z.n, z.m, z.n, prec, ORDER, X);
+        if (call == 3) vl_fit_b(h, X, z.n, z.m, z.n, ORDER, X, 1, prec, X, X);
+        if (call == 4) vl_fit(h, X, z.n, z.m, z.n, 1, prec, X, ORDER, X, X, X);
+        if (call == 5) vl_var_select(h, X, z.n, z.m, z.n, 2, VL_IC_BIC, prec, X, ORDER);
+        if (call == 6) vl_fit_batched(h, &I, 1, prec, &st);
+        bool any = false;
+        for (const fake::Launch& l : fake::launches) any |= l.overlap;
+        if (any != (want && call != 6))
+          std::printf("call %d m=%d n=%d precision %d: overlap %d\n", call, z.m, z.n, (int)prec, any);
+      }
+    }
+  vl_destroy(h);
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
   if (argc == 2 && !std::strcmp(argv[1], "two_devices")) two_devices();
   if (argc == 2 && !std::strcmp(argv[1], "no_search")) no_search();
+  if (argc == 2 && !std::strcmp(argv[1], "overlap")) overlap();
   return 0;
 }

@@ -2,7 +2,7 @@
 the CUDA runtime (tests/c/fake_cuda) that keeps, for every device, how much
 dynamic shared memory a kernel may use there, and refuses launches beyond it.
 Every call runs on two devices of one process, one after the other, and with
-searches whose launch fails."""
+searches whose launch fails; and which calls' launches overlap."""
 import glob
 import importlib.util
 import os
@@ -35,7 +35,7 @@ def host_check(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("what", ["two_devices", "no_search"])
+@pytest.mark.parametrize("what", ["two_devices", "no_search", "overlap"])
 def test_host_side(host_check, what):
     out = subprocess.run([host_check, what], check=True, capture_output=True, text=True).stdout
     assert out == ""
