@@ -1,11 +1,11 @@
 // Small dense linear algebra on the CUDA cores: a tiled GEMM over strided
-// views, a compensated hi/lo split product for covariances, and a blocked
-// Cholesky factorisation with blocked triangular solves built from them.
+// views and a blocked Cholesky factorisation with blocked triangular solves built
+// from it.
 //
-// Precision: with T = float every product is an FP32 FMA; partial sums are
-// flushed every `kFlush` steps of k into a double-float (hi, lo) accumulator
-// (TwoSum), so the error does not grow with K.  With T = double everything is
-// FP64.  Split-K partials are combined in FP64 in a fixed order (deterministic).
+// Precision: with T = float every product is an FP32 FMA over slices of 512 steps of
+// k (longer only where their partials outgrow the scratch), added as a double-float
+// (hi, lo) pair (TwoSum).  With T = double everything is FP64.  The order of the
+// partials is fixed (deterministic).
 #include <algorithm>
 
 #include "vl_internal.cuh"
@@ -72,55 +72,37 @@ struct StageLoader {
   }
 };
 
-// mode: 0 = full, 1 = lower (c <= r), 2 = upper (c >= r, mirrored into C[c, r]).
+// lower: only the entries c <= r.
 // C[r, c] = alpha * sum_k A(r, k) B(c, k) + beta * C[r, c], or, with split-K
 // (gridDim.z > 1), slice z's partial into part[z][r][c].  The next k-stage is
 // loaded into registers while the current one is consumed (double buffer).
-// SPLIT: A and B come as (hi, lo) FP32 pairs; each step adds hi*hi + hi*lo +
-// lo*hi and the FP32 sum is flushed every 32 steps into a double-float pair.
-template <class T, class TC, int TMt, int TNt, bool SPLIT>
+template <class T, class TC, int TMt, int TNt>
 __global__ void __launch_bounds__(NTH) gemm_kernel(int M, int N, int K, int kchunk,
-                                                   double alpha, View<T> A, View<T> Al, View<T> B,
-                                                   View<T> Bl, double beta, TC* __restrict__ C,
-                                                   int64_t ldc, int mode,
+                                                   double alpha, View<T> A, View<T> B, double beta,
+                                                   TC* __restrict__ C, int64_t ldc, bool lower,
                                                    double* __restrict__ part) {
   pdl_begin(C, part);
   constexpr int BM = 16 * TMt, BN = 16 * TNt;
-  constexpr int NOP = SPLIT ? 2 : 1;
   const int r0 = blockIdx.y * BM, c0 = blockIdx.x * BN;
-  if (mode == 1 && c0 > r0 + BM - 1) return;
-  if (mode == 2 && r0 > c0 + BN - 1) return;
-  __shared__ __align__(16) T As[2][NOP][KC * (BM + 4)];
-  __shared__ __align__(16) T Bs[2][NOP][KC * (BN + 4)];
+  if (lower && c0 > r0 + BM - 1) return;
+  __shared__ __align__(16) T As[2][KC * (BM + 4)];
+  __shared__ __align__(16) T Bs[2][KC * (BN + 4)];
   const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
   const int kbeg = blockIdx.z * kchunk;
   const int kend = min(K, kbeg + kchunk);
   T acc[TMt][TNt];
-  float hi[SPLIT ? TMt : 1][SPLIT ? TNt : 1], lo[SPLIT ? TMt : 1][SPLIT ? TNt : 1];
 #pragma unroll
   for (int a = 0; a < TMt; ++a)
 #pragma unroll
     for (int b = 0; b < TNt; ++b) acc[a][b] = T(0);
-  if constexpr (SPLIT) {
-#pragma unroll
-    for (int a = 0; a < TMt; ++a)
-#pragma unroll
-      for (int b = 0; b < TNt; ++b) hi[a][b] = lo[a][b] = 0.f;
-  }
-  StageLoader<T, BM> la, lal;
-  StageLoader<T, BN> lb, lbl;
+  StageLoader<T, BM> la;
+  StageLoader<T, BN> lb;
   const int nst = kend > kbeg ? (kend - kbeg + KC - 1) / KC : 0;
   if (nst > 0) {
     la.load(A, r0, M, kbeg, kend);
     lb.load(B, c0, N, kbeg, kend);
-    la.store(As[0][0], A.ks);
-    lb.store(Bs[0][0], B.ks);
-    if constexpr (SPLIT) {
-      lal.load(Al, r0, M, kbeg, kend);
-      lbl.load(Bl, c0, N, kbeg, kend);
-      lal.store(As[0][NOP - 1], Al.ks);
-      lbl.store(Bs[0][NOP - 1], Bl.ks);
-    }
+    la.store(As[0], A.ks);
+    lb.store(Bs[0], B.ks);
   }
   __syncthreads();
   for (int t = 0; t < nst; ++t) {
@@ -130,56 +112,22 @@ __global__ void __launch_bounds__(NTH) gemm_kernel(int M, int N, int K, int kchu
       const int k1 = kbeg + (t + 1) * KC;
       la.load(A, r0, M, k1, kend);
       lb.load(B, c0, N, k1, kend);
-      if constexpr (SPLIT) {
-        lal.load(Al, r0, M, k1, kend);
-        lbl.load(Bl, c0, N, k1, kend);
-      }
     }
 #pragma unroll
     for (int kk = 0; kk < KC; ++kk) {
       T a[TMt], b[TNt];
 #pragma unroll
-      for (int q = 0; q < TMt; ++q) a[q] = As[buf][0][kk * (BM + 4) + ty * TMt + q];
+      for (int q = 0; q < TMt; ++q) a[q] = As[buf][kk * (BM + 4) + ty * TMt + q];
 #pragma unroll
-      for (int q = 0; q < TNt; ++q) b[q] = Bs[buf][0][kk * (BN + 4) + tx * TNt + q];
-      if constexpr (SPLIT) {
-        T al[TMt], bl[TNt];
+      for (int q = 0; q < TNt; ++q) b[q] = Bs[buf][kk * (BN + 4) + tx * TNt + q];
 #pragma unroll
-        for (int q = 0; q < TMt; ++q) al[q] = As[buf][NOP - 1][kk * (BM + 4) + ty * TMt + q];
+      for (int x = 0; x < TMt; ++x)
 #pragma unroll
-        for (int q = 0; q < TNt; ++q) bl[q] = Bs[buf][NOP - 1][kk * (BN + 4) + tx * TNt + q];
-#pragma unroll
-        for (int x = 0; x < TMt; ++x)
-#pragma unroll
-          for (int y = 0; y < TNt; ++y) {
-            T tt = fma(a[x], bl[y], al[x] * b[y]);
-            acc[x][y] = fma(a[x], b[y], acc[x][y] + tt);
-          }
-      } else {
-#pragma unroll
-        for (int x = 0; x < TMt; ++x)
-#pragma unroll
-          for (int y = 0; y < TNt; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
-      }
-    }
-    if constexpr (SPLIT) {
-      if ((t & 3) == 3) {  // every 32 steps of k
-#pragma unroll
-        for (int x = 0; x < TMt; ++x)
-#pragma unroll
-          for (int y = 0; y < TNt; ++y) {
-            two_sum_acc(hi[x][y], lo[x][y], (float)acc[x][y]);
-            acc[x][y] = T(0);
-          }
-      }
+        for (int y = 0; y < TNt; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
     }
     if (more) {
-      la.store(As[buf ^ 1][0], A.ks);
-      lb.store(Bs[buf ^ 1][0], B.ks);
-      if constexpr (SPLIT) {
-        lal.store(As[buf ^ 1][NOP - 1], Al.ks);
-        lbl.store(Bs[buf ^ 1][NOP - 1], Bl.ks);
-      }
+      la.store(As[buf ^ 1], A.ks);
+      lb.store(Bs[buf ^ 1], B.ks);
     }
     __syncthreads();
   }
@@ -189,9 +137,8 @@ __global__ void __launch_bounds__(NTH) gemm_kernel(int M, int N, int K, int kchu
     for (int y = 0; y < TNt; ++y) {
       const int r = r0 + ty * TMt + x, c = c0 + tx * TNt + y;
       if (r >= M || c >= N) continue;
-      if (mode == 1 && c > r) continue;
-      if (mode == 2 && c < r) continue;
-      if constexpr (!SPLIT && sizeof(T) == 4) {
+      if (lower && c > r) continue;
+      if constexpr (sizeof(T) == 4) {
         // all-FP32 epilogue (FP64 conversions run at 1/64 rate on this part):
         // split-K slices leave FP32 partials, reduced by splitk_reduce_f32
         if (part) {
@@ -203,22 +150,15 @@ __global__ void __launch_bounds__(NTH) gemm_kernel(int M, int N, int K, int kchu
           float v = (float)alpha * acc[x][y];
           if (beta != 0.0) v = fmaf((float)beta, C[(int64_t)r * ldc + c], v);
           C[(int64_t)r * ldc + c] = v;
-          if (mode == 2 && c != r) C[(int64_t)c * ldc + r] = v;
           continue;
         }
       }
-      double v;
-      if constexpr (SPLIT)
-        v = ((double)hi[x][y] + (double)lo[x][y]) + (double)acc[x][y];
-      else
-        v = (double)acc[x][y];
-      v *= alpha;
+      double v = (double)acc[x][y] * alpha;
       if (part) {
         part[((int64_t)blockIdx.z * M + r) * N + c] = v;
       } else {
         if (beta != 0.0) v += beta * (double)C[(int64_t)r * ldc + c];
         C[(int64_t)r * ldc + c] = (TC)v;
-        if (mode == 2 && c != r) C[(int64_t)c * ldc + r] = (TC)v;
       }
     }
 }
@@ -228,13 +168,12 @@ __global__ void __launch_bounds__(NTH) gemm_kernel(int M, int N, int K, int kchu
 template <class TC>
 __global__ void splitk_reduce_f32_kernel(const float* __restrict__ part, int ksplit, int M,
                                          int N, double beta, TC* __restrict__ C, int64_t ldc,
-                                         int mode) {
+                                         bool lower) {
   pdl_begin(part, C);
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)M * N) return;
   int r = (int)(idx / N), c = (int)(idx % N);
-  if (mode == 1 && c > r) return;
-  if (mode == 2 && c < r) return;
+  if (lower && c > r) return;
   float hi = 0.f, lo = 0.f;
   for (int z = 0; z < ksplit; ++z) two_sum_acc(hi, lo, part[((int64_t)z * M + r) * N + c]);
   TC v;
@@ -248,23 +187,20 @@ __global__ void splitk_reduce_f32_kernel(const float* __restrict__ part, int ksp
     v = d;
   }
   C[(int64_t)r * ldc + c] = v;
-  if (mode == 2 && c != r) C[(int64_t)c * ldc + r] = v;
 }
 
 template <class TC>
 __global__ void splitk_reduce_kernel(const double* __restrict__ part, int ksplit, int M, int N,
-                                     double beta, TC* __restrict__ C, int64_t ldc, int mode) {
+                                     double beta, TC* __restrict__ C, int64_t ldc, bool lower) {
   pdl_begin(part, C);
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)M * N) return;
   int r = (int)(idx / N), c = (int)(idx % N);
-  if (mode == 1 && c > r) return;
-  if (mode == 2 && c < r) return;
+  if (lower && c > r) return;
   double v = 0.0;
   for (int z = 0; z < ksplit; ++z) v += part[((int64_t)z * M + r) * N + c];
   if (beta != 0.0) v += beta * (double)C[(int64_t)r * ldc + c];
   C[(int64_t)r * ldc + c] = (TC)v;
-  if (mode == 2 && c != r) C[(int64_t)c * ldc + r] = (TC)v;
 }
 
 // ---- Cholesky of one nb x nb diagonal block, plus the inverse of the factor.
@@ -814,31 +750,30 @@ int pick_ksplit(int tiles, int K, int num_sms, int max_chunk) {
   return std::min(ks, 64);
 }
 
-template <class T, class TC, int TMt, int TNt, bool SPLIT>
-void gemm_launch(const Ctx& cx, int M, int N, int K, double alpha, View<T> A, View<T> Al,
-                 View<T> B, View<T> Bl, double beta, TC* C, int64_t ldc, int mode,
-                 int max_chunk) {
+template <class T, class TC, int TMt, int TNt>
+void gemm_launch(const Ctx& cx, int M, int N, int K, double alpha, View<T> A, View<T> B,
+                 double beta, TC* C, int64_t ldc, bool lower, int max_chunk) {
   if (M <= 0 || N <= 0) return;
   constexpr int BM = 16 * TMt, BN = 16 * TNt;
   const int gm = (M + BM - 1) / BM, gn = (N + BN - 1) / BN;
   int tiles = gm * gn;
-  if (mode != 0) tiles = (tiles + std::min(gm, gn)) / 2;
+  if (lower) tiles = (tiles + std::min(gm, gn)) / 2;
   int ks = pick_ksplit(tiles, K, cx.num_sms, max_chunk);
   if (ks > 1 && (!cx.part || (size_t)ks * M * N > cx.part_cap))
     ks = cx.part ? std::max(1, (int)std::min<size_t>(ks, cx.part_cap / ((size_t)M * N))) : 1;
   int kchunk = ks > 1 ? (((K + ks - 1) / ks + 31) / 32) * 32 : std::max(K, 1);
   ks = ks > 1 ? (K + kchunk - 1) / kchunk : 1;
   dim3 grid(gn, gm, ks);
-  launch(gemm_kernel<T, TC, TMt, TNt, SPLIT>, grid, NTH, 0, cx.s, M, N, K, kchunk, alpha, A, Al, B,
-         Bl, beta, C, ldc, mode, ks > 1 ? cx.part : nullptr);
+  launch(gemm_kernel<T, TC, TMt, TNt>, grid, NTH, 0, cx.s, M, N, K, kchunk, alpha, A, B, beta, C,
+         ldc, lower, ks > 1 ? cx.part : nullptr);
   if (ks > 1) {
     int64_t tot = (int64_t)M * N;
-    if constexpr (!SPLIT && sizeof(T) == 4)
+    if constexpr (sizeof(T) == 4)
       launch(splitk_reduce_f32_kernel<TC>, (unsigned)((tot + 255) / 256), 256, 0, cx.s,
-             reinterpret_cast<const float*>(cx.part), ks, M, N, beta, C, ldc, mode);
+             reinterpret_cast<const float*>(cx.part), ks, M, N, beta, C, ldc, lower);
     else
       launch(splitk_reduce_kernel<TC>, (unsigned)((tot + 255) / 256), 256, 0, cx.s, cx.part, ks, M,
-             N, beta, C, ldc, mode);
+             N, beta, C, ldc, lower);
   }
 }
 
@@ -858,24 +793,22 @@ size_t gemm_part_need(int M, int N, int K) {
 template <class T, class TC>
 void launch_gemm(const Ctx& cx, int M, int N, int K, double alpha, View<T> A, View<T> B,
                  double beta, TC* C, int64_t ldc, bool lower_only) {
-  const int mode = lower_only ? 1 : 0;
   if constexpr (sizeof(T) == 4) {
     // largest micro-tile whose padded work stays within 10% of the best
     if ((int64_t)M * N >= 256 * 256) {
       const double w8 = tile_waste(M, N, 128, 128), w5 = tile_waste(M, N, 80, 80);
       const double w4 = tile_waste(M, N, 64, 64);
       if (w8 <= 1.1 * std::min(w5, w4))
-        gemm_launch<T, TC, 8, 8, false>(cx, M, N, K, alpha, A, A, B, B, beta, C, ldc, mode, 512);
+        gemm_launch<T, TC, 8, 8>(cx, M, N, K, alpha, A, B, beta, C, ldc, lower_only, 512);
       else if (w5 <= 1.1 * w4)
-        gemm_launch<T, TC, 5, 5, false>(cx, M, N, K, alpha, A, A, B, B, beta, C, ldc, mode, 512);
+        gemm_launch<T, TC, 5, 5>(cx, M, N, K, alpha, A, B, beta, C, ldc, lower_only, 512);
       else
-        gemm_launch<T, TC, 4, 4, false>(cx, M, N, K, alpha, A, A, B, B, beta, C, ldc, mode, 512);
+        gemm_launch<T, TC, 4, 4>(cx, M, N, K, alpha, A, B, beta, C, ldc, lower_only, 512);
     } else {
-      gemm_launch<T, TC, 4, 4, false>(cx, M, N, K, alpha, A, A, B, B, beta, C, ldc, mode, 512);
+      gemm_launch<T, TC, 4, 4>(cx, M, N, K, alpha, A, B, beta, C, ldc, lower_only, 512);
     }
   } else {
-    gemm_launch<T, TC, 4, 4, false>(cx, M, N, K, alpha, A, A, B, B, beta, C, ldc, mode,
-                                    1 << 30);
+    gemm_launch<T, TC, 4, 4>(cx, M, N, K, alpha, A, B, beta, C, ldc, lower_only, 1 << 30);
   }
 }
 template void launch_gemm<float, float>(const Ctx&, int, int, int, double, View<float>,
@@ -884,19 +817,6 @@ template void launch_gemm<float, double>(const Ctx&, int, int, int, double, View
                                          View<float>, double, double*, int64_t, bool);
 template void launch_gemm<double, double>(const Ctx&, int, int, int, double, View<double>,
                                           View<double>, double, double*, int64_t, bool);
-
-void launch_gemm_split(const Ctx& cx, int M, int N, int K, View<float> Ahi, View<float> Alo,
-                       View<float> Bhi, View<float> Blo, double* C, int64_t ldc,
-                       bool upper_only) {
-  // a 32 x 32 tile when the whole product fits one: a 64 x 64 tile would
-  // spend three quarters of its arithmetic on padding
-  if (std::max(M, N) <= 32)
-    gemm_launch<float, double, 2, 2, true>(cx, M, N, K, 1.0, Ahi, Alo, Bhi, Blo, 0.0, C, ldc,
-                                           upper_only ? 2 : 0, 1 << 30);
-  else
-    gemm_launch<float, double, 4, 4, true>(cx, M, N, K, 1.0, Ahi, Alo, Bhi, Blo, 0.0, C, ldc,
-                                           upper_only ? 2 : 0, 1 << 30);
-}
 
 template <class T>
 void chol_blocked(const Ctx& cx, T* A, int64_t lda, int n, T* dinv, double* diag0,

@@ -38,7 +38,6 @@ namespace vl {
 namespace {
 
 constexpr int TB = 32;        // variables per tile side
-constexpr int TT = 128;       // samples per shared-memory stage
 constexpr int KRUN = 16;      // samples per product/Kahan run (product <= 2^16)
 constexpr float KAPPA = 2.8853900817779268f;       // 2 log2(e)
 constexpr float GAUSS_K = -0.08664339756999316f;   // -1 / (8 log2 e)

@@ -274,8 +274,8 @@ void launch_transpose_std(const double* E, int64_t lde, int m, int n, const doub
 
 // Dense linear algebra (k_linalg.cu).  A "view" addresses element (r, k) at
 // base[r * rs + k * ks].  gemm computes C[r, c] = alpha * sum_k A(r,k) B(c,k)
-// + beta * C[r, c] for r < M, c < N (C row-major, ldc), accumulating in T
-// with a double-float flush every `flush` steps of k when T is float.
+// + beta * C[r, c] for r < M, c < N (C row-major, ldc), accumulating in T, when T
+// is float over slices of k that are added as double-float pairs.
 template <class T>
 struct View {
   const T* base;
@@ -284,9 +284,6 @@ struct View {
 template <class T, class TC>
 void launch_gemm(const Ctx& c, int M, int N, int K, double alpha, View<T> A, View<T> B,
                  double beta, TC* C, int64_t ldc, bool lower_only);
-void launch_gemm_split(const Ctx& c, int M, int N, int K, View<float> Ahi, View<float> Alo,
-                       View<float> Bhi, View<float> Blo, double* C, int64_t ldc,
-                       bool upper_only);
 // Split-K scratch (doubles) the GEMMs of an (M x N) product may use.
 size_t gemm_part_need(int M, int N, int K);
 // Cholesky of the n x n SPD matrix A (T, row-major, lda, lower part used) in
