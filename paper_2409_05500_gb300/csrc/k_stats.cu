@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kStatMax)
   __shared__ fx::u64 te[fx::EXP_N], tl[fx::LOG_N];
   __shared__ fx::u32 tr[fx::LOG_N];
   const fx::Tab tab{te, tl, tr};
-  fx::fill_tables(te, tl, tr);
+  if (hx) fx::fill_tables(te, tl, tr);
   const int i = blockIdx.x;
   const double* e = E + (int64_t)i * lde;
   double mu, isd;
