@@ -79,24 +79,18 @@ struct Exec {
 };
 
 // Launches of a call on m x n samples overlap (Lane) while its kernels are so
-// small that the time between them counts.
-//  - Mixed: the kernels grow with the samples.  Measured on a stream without and
-//    with: m n = 1e4 a fit 188 -> 110 us, 1e5 99 search steps 6.1 -> 4.6 ms, 2.6e5
-//    measures of m = 20 to 1600 between 133 -> 122 and 328 -> 311; 8e5 to 1e6 within
-//    3 % either way, but a fit of m = 400 replayed as a graph 791 -> 823 us and the
-//    iterative search of that size 44.6 -> 60.6 ms.
-//  - FP64: products and pairs take most of a call, and their kernels lose more from
-//    the CTAs that wait beside them than the launches cost.  m^2 n = 1.5e5 a measure
-//    168 -> 151 us, 9e5 a fit 863 -> 841, 1e6 a VAR fit 1587 -> 1582, but 2.5e6 one
-//    478 -> 707, 5e6 a measure 508 -> 737, 4e7 (p = 2) a fit 4500 -> 5800.
+// small that the time between them counts.  Measured on a stream without and
+// with: m n = 1e4 a fit 188 -> 110 us, an FP64 one of m = 30, n = 1000 862 -> 807, 1e5
+// 99 search steps 6.1 -> 4.6 ms, 2.6e5 measures of m = 20 to 1600 between 133 -> 122 and
+// 328 -> 311; 8e5 to 1e6 within 3 % either way, but a fit of m = 400 replayed as a graph
+// 791 -> 823 us and the iterative search of that size 44.6 -> 60.6 ms.
 // What else the caller runs is not known here.  Fits of m = 50, n = 5000 on the
 // caller's own streams, a fit without and with: two streams of calls 151 -> 125 us,
 // of replayed graphs 113 -> 123; eight of calls from as many threads 62 -> 64, of
 // graphs 46 -> 59; m = 10, n = 1000 the same or faster everywhere.
-constexpr int64_t OVERLAP_MAX = 1 << 18, OVERLAP_MAX_FP64 = 1 << 20;
-Exec handle_exec(vl_handle h, int64_t m, int64_t n, bool fp64 = false) {
-  const bool overlap = m * n <= OVERLAP_MAX && (!fp64 || m * m * n <= OVERLAP_MAX_FP64);
-  return Exec{h, Lane(h->stream, overlap), h->status, &h->ws, &h->ws_cap, false, 0};
+constexpr int64_t OVERLAP_MAX = 1 << 18;
+Exec handle_exec(vl_handle h, int64_t m, int64_t n) {
+  return Exec{h, Lane(h->stream, m * n <= OVERLAP_MAX), h->status, &h->ws, &h->ws_cap, false, 0};
 }
 
 vl_status grow(vl_handle h, void** ws, size_t* cap, size_t bytes, cudaStream_t s) {
@@ -1090,7 +1084,7 @@ vl_status vl_var_fit(vl_handle h, const double* X, int64_t ldx, int m, int n, in
   if ((int64_t)n - p <= (int64_t)m * p + 1)
     return fail(h, VL_ERR_RANK, "vl_var_fit: n - p <= m p + 1, the VAR has no unique fit");
   DeviceGuard g(h->device);
-  Exec x = handle_exec(h, m, n, prec == VL_PREC_FP64);
+  Exec x = handle_exec(h, m, n);
   return prec != VL_PREC_FP64 ? var_fit_impl<float>(x, X, ldx, m, n, p, M, E)
                                : var_fit_impl<double>(x, X, ldx, m, n, p, M, E);
 }
@@ -1111,7 +1105,7 @@ vl_status vl_var_select(vl_handle h, const double* X, int64_t ldx, int m, int n,
                 "vl_var_select: n - p_max <= m (p_max + 1), the residual covariance of the "
                 "largest VAR cannot be of full rank");
   DeviceGuard g(h->device);
-  Exec x = handle_exec(h, m, n, prec == VL_PREC_FP64);
+  Exec x = handle_exec(h, m, n);
   // the candidates' coefficients and residuals (reused from p to p)
   const size_t mb = (size_t)p_max * m * m, eb = (size_t)m * T;
   vl_status s = grow(h, &h->selbuf, &h->selbuf_cap, sizeof(double) * (mb + eb) + 512, x.s);
@@ -1157,7 +1151,7 @@ vl_status vl_pairwise_measure(vl_handle h, const double* E, int64_t lde, int m, 
   if (m < 2 || n_eff < 2 || m > VL_MAX_M || lde < n_eff)
     return fail(h, VL_ERR_SHAPE, "vl_pairwise_measure: need 2 <= m <= VL_MAX_M, n_eff >= 2, lde >= n_eff");
   DeviceGuard g(h->device);
-  Exec x = handle_exec(h, m, n_eff, prec == VL_PREC_FP64);
+  Exec x = handle_exec(h, m, n_eff);
   return prec != VL_PREC_FP64 ? pairwise_impl<float>(x, E, lde, m, n_eff, Hx, Hr, D, nullptr)
                                : pairwise_impl<double>(x, E, lde, m, n_eff, Hx, Hr, D, nullptr);
 }
@@ -1195,7 +1189,7 @@ vl_status vl_causal_order_standard(vl_handle h, const double* E, int64_t lde, in
     return fail(h, VL_ERR_SHAPE,
                 "vl_causal_order_standard: need 2 <= m <= VL_MAX_M, n_eff >= 2, lde >= n_eff");
   DeviceGuard g(h->device);
-  Exec x = handle_exec(h, m, n_eff, prec == VL_PREC_FP64);
+  Exec x = handle_exec(h, m, n_eff);
   return prec != VL_PREC_FP64 ? order_standard_impl<float>(x, E, lde, m, n_eff, order, gap)
                                : order_standard_impl<double>(x, E, lde, m, n_eff, order, gap);
 }
@@ -1210,7 +1204,7 @@ vl_status vl_fit_b(vl_handle h, const double* E, int64_t lde, int m, int n_eff,
     return fail(h, VL_ERR_SHAPE, "vl_fit_b: bad sizes");
   if (validate_prec(h, prec) != VL_OK) return VL_ERR_ARG;
   DeviceGuard g(h->device);
-  Exec x = handle_exec(h, m, n_eff, prec != VL_PREC_MIXED);
+  Exec x = handle_exec(h, m, n_eff);
   return prec == VL_PREC_MIXED
              ? fit_b_impl<float>(x, E, lde, m, n_eff, order, M, p, B0, Btau, nullptr)
              : fit_b_impl<double>(x, E, lde, m, n_eff, order, M, p, B0, Btau, nullptr);
@@ -1231,7 +1225,7 @@ vl_status vl_fit(vl_handle h, const double* X, int64_t ldx, int m, int n, int p,
   double* E = static_cast<double*>(h->sbuf);
   double* C = E + m * ne;
   if (!D) D = C + mm;
-  Exec x = handle_exec(h, m, n, prec == VL_PREC_FP64);
+  Exec x = handle_exec(h, m, n);
   return prec != VL_PREC_FP64 ? fit_one<float>(x, I, E, C, D, prec == VL_PREC_MIXED_CERTIFIED)
                                : fit_one<double>(x, I, E, C, D);
 }

@@ -764,8 +764,15 @@ void gemm_launch(const Ctx& cx, int M, int N, int K, double alpha, View<T> A, Vi
   int kchunk = ks > 1 ? (((K + ks - 1) / ks + 31) / 32) * 32 : std::max(K, 1);
   ks = ks > 1 ? (K + kchunk - 1) / kchunk : 1;
   dim3 grid(gn, gm, ks);
-  launch(gemm_kernel<T, TC, TMt, TNt>, grid, NTH, 0, cx.s, M, N, K, kchunk, alpha, A, B, beta, C,
-         ldc, lower, ks > 1 ? cx.part : nullptr);
+  // An FP64 product has about two CTAs per SM and is bound by each SM's FP64 unit:
+  // set up while its predecessor's CTAs still hold some SMs, its CTAs crowd on the
+  // others.  So it starts when they have left (launches overlapped, with and without
+  // its own): VAR fit m = 100, n = 2500, p = 3 5062 -> 3188 us, m = 10, n = 5000, p = 3
+  // 2132 -> 1607, measure m = 10, n = 5000 458 -> 238; small calls pay a launch's
+  // latency: fit_b m = 10, n = 420 312 -> 316.
+  const Lane at(cx.s, cx.s.overlap && sizeof(T) == 4);
+  launch(gemm_kernel<T, TC, TMt, TNt>, grid, NTH, 0, at, M, N, K, kchunk, alpha, A, B, beta, C, ldc,
+         lower, ks > 1 ? cx.part : nullptr);
   if (ks > 1) {
     int64_t tot = (int64_t)M * N;
     if constexpr (sizeof(T) == 4)
