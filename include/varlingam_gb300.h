@@ -247,8 +247,8 @@ vl_status vl_causal_order_noalloc(void* cuda_stream, const double* D, int m, int
  * prec  : the precision of each pairwise measure (as vl_pairwise_measure).
  *         Step 5 is applied in FP64 with the slopes taken from the centred
  *         cross products the measure computes for its correlations (FP64,
- *         or in VL_PREC_MIXED split-FP32 products summed in double-float,
- *         relative error about 1e-8).
+ *         or in VL_PREC_MIXED tensor-core products of exact slices summed in
+ *         double-float, relative error about 1e-8).
  * order : output m int32 (causes first).
  * gap   : output m doubles or NULL; gap[k] = relative gap between the two
  *         smallest scores of iteration k, as in vl_causal_order (+inf last).

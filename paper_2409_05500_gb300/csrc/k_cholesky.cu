@@ -28,9 +28,10 @@
 // of one SM here, and seven workers reading the chain's tiles made a period
 // 25,000 clocks.
 //
-// Measured, n = 400: 90 us, against 145-150 us with the row blocks dealt
-// round-robin and every block column's inverse and panels crossing the cluster
-// inside the chain (32-row blocks and the order of every sum are the same: the
+// Measured, n = 400, a launch in a stream of calls: 90 us, against 145-150 us with
+// the row blocks dealt round-robin and every block column's inverse and panels
+// crossing the cluster inside the chain (under the profiler, caches cold, 94 and
+// 170; 32-row blocks and the order of every sum are the same: the
 // factors are bit-identical).
 //
 // Cluster size: one worker for each row block below the third, up to seven (the
@@ -120,8 +121,9 @@ inline int row_off(int b, int nblk, int W) {
 // Warps 0 and 1: warp 0 factors the 32 x 32 block (rows of stride RS, nb valid)
 // in place, warp 1 builds L^{-1} into li behind it, from the columns warp 0
 // leaves in col (row j of stride RS: the multipliers of rows j + 1 .. 31, then
-// zeros; 1 / L[j][j] at 32, the next pivot's threshold at 33).  Every four columns warp 0 arrives, without
-// waiting, at one of the named barriers 5 .. 12, each used once per block.
+// zeros; at 32 the threshold of pivot j + 1, at 34 1 / L[j][j], at 35 L[j][j]).
+// Every four columns warp 0 arrives, without waiting, at one of the named barriers
+// 5 .. 12, each used once per block.
 //
 // Lane r holds row r from column j on, a[c] = entry (r, j + c): the update writes
 // entry c + 1 into register c, so that the steps of a group of eight are the same

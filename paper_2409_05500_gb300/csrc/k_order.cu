@@ -103,7 +103,9 @@ __device__ __forceinline__ void load_scores(const float* __restrict__ sh0,
 // thread, a branch around every dead variable, P in L2 below m = 64 and beyond
 // 448 (no fetching ahead) and in a cluster between: m = 32 27 -> 17 us, 64
 // 37 -> 22, 100 52 -> 29, 160 74 -> 41, 256 107 -> 78, 400 165 -> 133, 800
-// 561 -> 371, 1600 1444 -> 1108.
+// 561 -> 371, 1600 1444 -> 1108; in a later run 1600 1597 -> 1141, 2048 2281 -> 1468,
+// 3000 4883 -> 3412, 4096 7758 -> 4733 (256 threads with up to 16 variables each, where
+// 1024 had up to 4).
 
 // Search with P in global memory: Pt[c * m + i] = P_{i,c}.  The eventual pick
 // is usually some warp's minimum for a few steps before it wins (in 60 to 80 %
@@ -290,8 +292,8 @@ bool launch_order_local(const OrderWs& w, int m, int32_t* order, float2* spick, 
 // a time, all threads load and convert the tile's P (FP64 conversions issue at
 // 1.6 per clock per SM: few variables per CTA spread them over the SMs), one
 // warp runs the chains, and one thread per step reduces the GAP_V scores to one
-// atomic.  The gaps of m = 800 add 62 us (260 us with one thread doing all of it
-// for each variable).
+// atomic.  The gaps of m = 800 add 62 to 70 us (290 to 310 with one thread doing all
+// of it for each variable).
 constexpr int GAP_V = 8, GAP_T = 64, GAP_TH = 128;
 __global__ void __launch_bounds__(GAP_TH)
     gap_scores_kernel(const float2* __restrict__ pt, const float* __restrict__ sh0,

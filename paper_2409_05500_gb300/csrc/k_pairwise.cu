@@ -306,8 +306,8 @@ __global__ void __launch_bounds__(TB / MTI * 16, MINB)
 // FP64 measure.  The residuals are formed in FP64 (one FMA and one product
 // each), the per-sample functions and their sums in 63-bit fixed point
 // (fx64.cuh), which is closer to exact than FP64 functions and sums are.
-// Bound by the integer pipe (~170 instructions a residual sample) with the
-// FP64 pipe (two operations, 40 SM clocks a warp) close behind it.  m = 120,
+// Bound by instructions: 257 a residual sample, the pipe of the integer products
+// 73 % busy, the FP64 pipe (two operations, 40 SM clocks a warp) 64 %.  m = 120,
 // n = 9997: 1.50 ms; with CUDA's FP64 exp and log1p, which keep the FP64 pipe
 // busy 20 times as long, 33.1 ms.
 // One pair a < b per thread, consecutive threads consecutive b (coalesced

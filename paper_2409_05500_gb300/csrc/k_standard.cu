@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(SC_WARPS * 32)
   Best b{kinf, 0x7fffffff, kinf};
   for (int i = threadIdx.x; i < u; i += blockDim.x) {
     const unsigned long long key = search::dkey(__ldcg(S + i));
-    // (a score that is not a number orders beyond infinity: it is never taken)
+    // (a score is a sum of squares from 0; one that is infinite orders last)
     if (key <= kinf) b = merge(b, Best{key, i, kinf});
   }
 #pragma unroll

@@ -532,8 +532,8 @@ bool launch_tcgram_sym(const Ctx& cx, const void* S, int N, int Kpad, int64_t ld
   P.sym = 1;
   const int tiles = sym_tiles(N, P.tiles_n);
   P.nkb = Kpad / TG_K;
-  // split K so that tiles x splits roughly fills the SMs, in whole segments,
-  // within the partial buffer
+  // split K so that tiles x splits roughly fills the SMs, at most one split per
+  // segment's length, within the partial buffer
   const int nseg = (P.nkb + TG_SEG - 1) / TG_SEG;
   // (one CTA per SM: a partial second wave would double the time)
   int splits = std::max(1, std::min(nseg, cx.num_sms / std::max(1, tiles)));

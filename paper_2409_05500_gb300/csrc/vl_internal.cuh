@@ -121,8 +121,8 @@ void note_launch();
 // beside the kernel before it: pdl_begin(), the first statement of a kernel, lets
 // the next kernel of the stream be set up as soon as all of this one's CTAs are
 // resident, and waits until the kernels before it have completed and their writes
-// are visible.  Measured, without and with: a fit of m = 10 188 -> 120 us, the
-// measure of m = 50 44 -> 30, 99 search steps of m = 100 6.1 -> 5.3 ms.
+// are visible.  Measured, without and with: a fit of m = 10 188 -> 110 us, the
+// measure of m = 50 43 -> 29, 99 search steps of m = 100 6.1 -> 4.6 ms.
 // pdl_wait() alone, in long kernels of few CTAs (Cholesky, the cluster search):
 // the next kernel's CTAs waiting on the other SMs made these slower (fit_b at
 // m = 400: 208 us without any of this, 224 with pdl_begin, 206 with pdl_wait), and
@@ -385,7 +385,7 @@ bool launch_tcgram_sym(const Ctx& cx, const void* S, int N, int Kpad, int64_t ld
                        const int* exps, double* C, int64_t ldc, double* w = nullptr);
 // The VAR residuals E = X[:, p:] - mu - cst - sum_tau M_tau Z_tau as one
 // tensor-core product (beta: FP32 mp x m; vexp: the variables' slice
-// exponents of launch_slice_lags); false if the tensor maps cannot be made or
+// exponents of launch_prep_lags); false if the tensor maps cannot be made or
 // the split-K buffer is smaller than m (n - p).
 bool launch_tc_var_resid(const Ctx& cx, const float* Xc, int64_t ldc, const double* X,
                          int64_t ldx, int m, int n, int p, const float* beta, const int* vexp,
